@@ -210,7 +210,7 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
         reg_destroy(c);
         return reg_fail(REG_ERR_NOMEM, "device allocation failed");
     }
-    if (k_init_twiddles(c) != cudaSuccess) {
+    if (upload_twiddles(c->tw) != cudaSuccess) {
         reg_destroy(c);
         return reg_fail(REG_ERR_CUDA, "twiddle upload failed");
     }

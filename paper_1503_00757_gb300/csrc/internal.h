@@ -143,7 +143,8 @@ bool tiles_valid(int n1, int n2, int R, int C, int P);
 bool tuned_tiles(int dev, int n1, int n2, int* R, int* C, int* P, int* D, int* T);
 
 // ---- launchers (kernels.cu); all asynchronous on ctx->stream ----
-cudaError_t k_init_twiddles(reg_ctx* ctx);
+// copies the REG_TW_TOTAL twiddle entries to the device
+cudaError_t upload_twiddles(float2* dst);
 // host: fill the REG_TW_TOTAL twiddle entries (fft.cuh layout) from FP64 sin / cos
 void fill_twiddles(float2* h);
 // shared memory of a row kernel with R rows of length L, and of the column kernel with C columns

@@ -110,10 +110,13 @@ void fill_twiddles(float2* h) {
     }
 }
 
-cudaError_t k_init_twiddles(reg_ctx* ctx) {
-    std::vector<float2> h(REG_TW_TOTAL);
-    fill_twiddles(h.data());
-    return cudaMemcpy(ctx->tw, h.data(), sizeof(float2) * REG_TW_TOTAL, cudaMemcpyHostToDevice);
+cudaError_t upload_twiddles(float2* dst) {
+    static const std::vector<float2> h = [] {  // the same constants for every context: computed once
+        std::vector<float2> t(REG_TW_TOTAL);
+        fill_twiddles(t.data());
+        return t;
+    }();
+    return cudaMemcpy(dst, h.data(), sizeof(float2) * REG_TW_TOTAL, cudaMemcpyHostToDevice);
 }
 
 // ---------------------------------------------------------------------------

@@ -8,311 +8,361 @@
 // and the full even symbol |k|^2.
 //
 // Layout: real fields are n1 x n2 x n3 floats, index (i1 n2 + i2) n3 + i3; vector fields
-// three such fields back to back.  Spectra are full complex (float2) fields in the same
-// order.  A 3-D transform is three passes of batched 1-D radix-2 Stockham FFTs
-// (k3_fft_pass), one per axis: a CTA stages a tile of 32 lines in shared memory (loads
-// coalesced along the contiguous direction), runs the log2(L) butterfly stages between
-// two shared buffers (row stride padded by one element against bank conflicts; twiddles
-// from a per-CTA table built once from exact fractions) and writes the tile back in
-// natural order.
+// three such fields back to back.
+//
+// Transport solves: a spectral derivative along one axis needs the transform of that axis
+// only (deriv.cuh), so a Heun stage is two launches and no three-dimensional transform:
+// k3_d12 takes the derivatives along axes 1 and 2 (the two as different blocks of one
+// launch), k3_adv / k3_adj take the one along axis 3 and update.
+// Assembly (regularization and projection, which couple the axes): half spectra along axis 3,
+// n1 x n2 x (n3 / 2 + 1) complex entries per field, in five launches: rows real to complex,
+// axis 2, axis 1 forward with the multiplier and back, axis 2 back, rows complex to real.
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <cstdint>
 #include <string>
 
+#include "deriv.cuh"
 #include "internal.h"
 
 namespace {
 
 constexpr int R3_THREADS = 256;
-constexpr int R3_TILE = 32;  // lines per CTA in an FFT pass
+constexpr int R3_BLOCKS = 608;  // 4 per SM of a GB300 for the grid-stride kernels
 
-// line l of a pass starts at (l / Q) P + (l % Q) R; elements are S apart
-struct LineMap {
-    int L, S, Q, P, R, TWL;
-};
-
-// one pass of length-L transforms (forward exp(-2 pi i jk / L), or inverse exp(+...),
-// unnormalized) over TWL consecutive lines per CTA
-template <bool INV>
-__global__ void __launch_bounds__(R3_THREADS) k3_fft_pass(float2* __restrict__ data, LineMap m) {
-    extern __shared__ float2 sbuf[];
-    const int TWL = m.TWL, L = m.L, SP = m.TWL + 1;  // padded stride: line elements fall in distinct banks
-    float2* b0 = sbuf;
-    float2* b1 = sbuf + L * SP;
-    float2* tw = sbuf + 2 * L * SP;  // tw[k] = exp(-2 pi i k / L), k < L / 2
-    const int tile = blockIdx.x;
-    auto base = [&](int w) {
-        const long long l = (long long)tile * TWL + w;
-        return (l / m.Q) * (long long)m.P + (l % m.Q) * (long long)m.R;
-    };
-    for (int k = threadIdx.x; k < L / 2; k += blockDim.x) {
-        float sn, cs;
-        sincospif(2.f * (float)k / (float)L, &sn, &cs);
-        tw[k] = make_float2(cs, -sn);
-    }
-    // stage the tile: b0[p SP + w] = element p of line w (the contiguous direction fastest)
-    for (int e = threadIdx.x; e < L * TWL; e += blockDim.x) {
-        int p, w;
-        if (m.S == 1) { p = e % L; w = e / L; } else { w = e % TWL; p = e / TWL; }
-        b0[p * SP + w] = data[base(w) + (long long)p * m.S];
-    }
-    __syncthreads();
-    float2* src = b0;
-    float2* dst = b1;
-    for (int Ns = 1; Ns < L; Ns <<= 1) {
-        const int step = L / (2 * Ns);  // exp(-i pi k / Ns) = tw[k step]
-        for (int e = threadIdx.x; e < (L / 2) * TWL; e += blockDim.x) {
-            const int w = e % TWL, j = e / TWL;
-            const int k = j & (Ns - 1);
-            const float2 a = src[j * SP + w];
-            const float2 c = src[(j + L / 2) * SP + w];
-            const float2 t0 = tw[k * step];
-            const float ws = INV ? -t0.y : t0.y;
-            const float2 t = make_float2(c.x * t0.x - c.y * ws, c.x * ws + c.y * t0.x);
-            const int d = (j / Ns) * 2 * Ns + k;
-            dst[d * SP + w] = make_float2(a.x + t.x, a.y + t.y);
-            dst[(d + Ns) * SP + w] = make_float2(a.x - t.x, a.y - t.y);
-        }
-        __syncthreads();
-        float2* tmp = src;
-        src = dst;
-        dst = tmp;
-    }
-    for (int e = threadIdx.x; e < L * TWL; e += blockDim.x) {
-        int p, w;
-        if (m.S == 1) { p = e % L; w = e / L; } else { w = e % TWL; p = e / TWL; }
-        data[base(w) + (long long)p * m.S] = src[p * SP + w];
-    }
+// see kernels.cu: wait for the preceding kernel, then let the next one start launching
+__device__ __forceinline__ void pdl_entry() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 struct Dims3 {
     int n1, n2, n3;
     long long N;
+    int l1, l2, l3;  // log2
+    int W1;          // n3 / 2 + 1: entries of a half-spectrum row
+    long long NS;    // n1 n2 W1
 };
 
-// odd (Nyquist zero) and even (Nyquist n/2) wavenumbers of index i on an axis of length n
-__device__ __forceinline__ float k_odd(int i, int n) { return i < n / 2 ? (float)i : (i == n / 2 ? 0.f : (float)(i - n)); }
-__device__ __forceinline__ float k_even(int i, int n) { return i < n / 2 ? (float)i : (float)(i - n); }
-
-__device__ __forceinline__ void wave3(const Dims3& D, long long idx, float& k1, float& k2, float& k3, float& kk) {
-    const int i3 = (int)(idx % D.n3);
-    const long long r = idx / D.n3;
-    const int i2 = (int)(r % D.n2), i1 = (int)(r / D.n2);
-    k1 = k_odd(i1, D.n1);
-    k2 = k_odd(i2, D.n2);
-    k3 = k_odd(i3, D.n3);
-    const float e1 = k_even(i1, D.n1), e2 = k_even(i2, D.n2), e3 = k_even(i3, D.n3);
-    kk = e1 * e1 + e2 * e2 + e3 * e3;
-}
+#define DISPATCH3(LOG, ...)                                   \
+    switch (LOG) {                                            \
+        case 3: { constexpr int LG = 3; __VA_ARGS__; } break; \
+        case 4: { constexpr int LG = 4; __VA_ARGS__; } break; \
+        case 5: { constexpr int LG = 5; __VA_ARGS__; } break; \
+        case 6: { constexpr int LG = 6; __VA_ARGS__; } break; \
+        case 7: { constexpr int LG = 7; __VA_ARGS__; } break; \
+        case 8: { constexpr int LG = 8; __VA_ARGS__; } break; \
+        default: break;                                       \
+    }
 
 #define GRID_STRIDE(i, n) for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
 
-// F = (f, 0) for nf fields of N points
-__global__ void k3_real2c(const float* __restrict__ f, float2* __restrict__ F, long long n) {
-    GRID_STRIDE(i, n) F[i] = make_float2(f[i], 0.f);
-}
-
-// G_d = i k~_d F (three spectra)
-__global__ void k3_grad_spec(const float2* __restrict__ F, float2* __restrict__ G, Dims3 D) {
-    GRID_STRIDE(i, D.N) {
-        float k1, k2, k3, kk;
-        wave3(D, i, k1, k2, k3, kk);
-        const float2 f = F[i];
-        G[i] = make_float2(-k1 * f.y, k1 * f.x);
-        G[D.N + i] = make_float2(-k2 * f.y, k2 * f.x);
-        G[2 * D.N + i] = make_float2(-k3 * f.y, k3 * f.x);
+// ---- transport ----
+// derivatives along axes 1 (blocks [0, tiles1)) and 2 (the rest): columns of float2 (deriv.cuh)
+struct D12Args {
+    DColArgs a1, a2;
+    ColMap m1, m2;
+    int log1, log2, lc1, lc2, tiles1;
+};
+__global__ void __launch_bounds__(256) k3_d12(D12Args a, const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    if ((int)blockIdx.x < a.tiles1) {
+        DISPATCH3(a.log1, dcol_body<LG>(a.a1, a.m1, 1 << a.lc1, a.lc1, blockIdx.x, sm, tw, pdl_entry));
+    } else {
+        DISPATCH3(a.log2, dcol_body<LG>(a.a2, a.m2, 1 << a.lc2, a.lc2, blockIdx.x - a.tiles1, sm, tw, pdl_entry));
     }
 }
 
-// F = sum_d i k~_d U_d
-__global__ void k3_div_spec(const float2* __restrict__ U, float2* __restrict__ F, Dims3 D) {
-    GRID_STRIDE(i, D.N) {
-        float k1, k2, k3, kk;
-        wave3(D, i, k1, k2, k3, kk);
-        const float2 a = U[i], b = U[D.N + i], c = U[2 * D.N + i];
-        const float re = k1 * a.x + k2 * b.x + k3 * c.x, im = k1 * a.y + k2 * b.y + k3 * c.y;
-        F[i] = make_float2(-im, re);
-    }
+template <int LOGL>
+__global__ void __launch_bounds__(128) k3_adv(AdvRow<3> a, long long N, int lines, const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    adv_row_body<LOGL, 3, false>(a, (size_t)N, lines, sm, tw, pdl_entry);
 }
 
-// out = beta |k|^2 V + K^ B (three spectra); mode 0: K = I, 1: incompressible, 2: mass source
-// (K^ = I - k~ k~^T / (|k~|^2 + beta |k|^2 / (beta_w (1 + |k|^2))))
-__global__ void k3_assemble(const float2* __restrict__ V, const float2* Bs, float2* out,  // out may be Bs
-                            Dims3 D, float beta, int mode, float beta_w) {
-    GRID_STRIDE(i, D.N) {
-        float k1, k2, k3, kk;
-        wave3(D, i, k1, k2, k3, kk);
-        float2 b[3] = {Bs[i], Bs[D.N + i], Bs[2 * D.N + i]};
-        if (mode != 0) {
-            const float ko = k1 * k1 + k2 * k2 + k3 * k3;
-            if (ko > 0.f) {
-                const float denom = mode == 1 ? ko : ko + beta * kk / (beta_w * (1.f + kk));
-                const float cre = (k1 * b[0].x + k2 * b[1].x + k3 * b[2].x) / denom;
-                const float cim = (k1 * b[0].y + k2 * b[1].y + k3 * b[2].y) / denom;
-                const float kd[3] = {k1, k2, k3};
+template <int LOGL>
+__global__ void __launch_bounds__(128) k3_adj(AdjRow<3> a, long long N, int lines, const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    adj_row_body<LOGL, 3, false, false>(a, (size_t)N, lines, sm, tw, pdl_entry);
+}
+
+// lam(1) = ca a + cb c (a nullable) and b = w lam grad m(1): the start of an adjoint solve
+__global__ void __launch_bounds__(R3_THREADS) k3_adj_init(const float* __restrict__ a, float ca,
+                                                          const float* __restrict__ c, float cb, float* lam, float* b,
+                                                          const float* __restrict__ gm, float w, long long N) {
+    pdl_entry();
+    GRID_STRIDE(i, N) {
+        float l = cb * c[i];
+        if (a) l = fmaf(ca, a[i], l);
+        lam[i] = l;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) b[d] = make_float2(b[d].x - kd[d] * cre, b[d].y - kd[d] * cim);
+        for (int d = 0; d < 3; ++d) b[d * N + i] = w * l * gm[d * N + i];
+    }
+}
+
+// ---- assembly: half spectra ----
+// rows of up to six real fields (0..2 from p0, 3..5 from p1, planes of N) to half spectra along
+// axis 3: two rows per complex transform, split into entries 0..n3/2 of each
+template <int LOGL>
+__global__ void __launch_bounds__(128) k3_r2c(const float* __restrict__ p0, const float* __restrict__ p1, float2* S,
+                                              Dims3 D, int lines, const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    constexpr int L = 1 << LOGL, T = L >> 3, H = L >> 1;
+    const int q = threadIdx.x / T, t = threadIdx.x - q * T;
+    const int f = blockIdx.y;
+    const float* src = (f < 3 ? p0 + f * D.N : p1 + (f - 3) * D.N);
+    const long long row = ((long long)blockIdx.x * lines + q) * 2;
+    LineTw<LOGL> W;
+    W.load(tw, t);
+    pdl_entry();
+    float2 x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = make_float2(src[row * L + t + k * T], src[(row + 1) * L + t + k * T]);
+    float2* cur = sm + 2 * q * fft_buf(L);
+    float2* nxt = cur + fft_buf(L);
+    auto idx = [](int pos) { return fft_pad(pos); };
+    line_fft<LOGL, false>(x, t, cur, nxt, idx, RowSync<LOGL>(), W);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) nxt[idx(t + k * T)] = x[k];
+    RowSync<LOGL>()();
+    float2* o0 = S + f * D.NS + row * D.W1;
+    float2* o1 = o0 + D.W1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int e = t + k * T;
+        const float2 z = x[k], y = nxt[idx((L - e) & (L - 1))];
+        o0[e] = make_float2(0.5f * (z.x + y.x), 0.5f * (z.y - y.y));
+        o1[e] = make_float2(0.5f * (z.y + y.y), -0.5f * (z.x - y.x));
+    }
+    if (t == 0) {
+        const float2 z = x[4];  // entry H = 4 T
+        o0[H] = make_float2(z.x, 0.f);
+        o1[H] = make_float2(z.y, 0.f);
+    }
+}
+
+// the inverse of k3_r2c for the three planes of out (the 1 / N is in the multiplier)
+template <int LOGL>
+__global__ void __launch_bounds__(128) k3_c2r(const float2* __restrict__ S, float* out, Dims3 D, int lines,
+                                              const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    constexpr int L = 1 << LOGL, T = L >> 3, H = L >> 1;
+    const int q = threadIdx.x / T, t = threadIdx.x - q * T;
+    const int f = blockIdx.y;
+    const long long row = ((long long)blockIdx.x * lines + q) * 2;
+    LineTw<LOGL> W;
+    W.load(tw, t);
+    pdl_entry();
+    const float2* s0 = S + f * D.NS + row * D.W1;
+    const float2* s1 = s0 + D.W1;
+    float2 x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int p = t + k * T;
+        const int e = p <= H ? p : L - p;
+        const float2 A = s0[e], B = s1[e];
+        if (p == 0 || p == H) x[k] = make_float2(A.x, B.x);
+        else x[k] = p < H ? make_float2(A.x - B.y, A.y + B.x) : make_float2(A.x + B.y, -A.y + B.x);
+    }
+    float2* cur = sm + 2 * q * fft_buf(L);
+    float2* nxt = cur + fft_buf(L);
+    line_fft<LOGL, true>(x, t, cur, nxt, [](int pos) { return fft_pad(pos); }, RowSync<LOGL>(), W);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        out[f * D.N + row * L + t + k * T] = x[k].x;
+        out[f * D.N + (row + 1) * L + t + k * T] = x[k].y;
+    }
+}
+
+// axis 2 of nf half spectra in place: column l = ((f n1 + i1) W1 + e), entries W1 apart
+template <int LOGL, bool INV>
+__global__ void __launch_bounds__(128) k3_axis2(float2* S, Dims3 D, int ncols, int C, int lc,
+                                                const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    constexpr int L = 1 << LOGL, T = L >> 3;
+    const int c = threadIdx.x & (C - 1), t = threadIdx.x >> lc;
+    const int l = blockIdx.x * C + c;
+    const bool on = l < ncols;
+    const int g = l / D.W1;
+    float2* p = S + ((long long)g * D.n2) * D.W1 + (l - g * D.W1);
+    LineTw<LOGL> W;
+    W.load(tw, t);
+    pdl_entry();
+    float2 x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = on ? p[(long long)(t + k * T) * D.W1] : make_float2(0.f, 0.f);
+    float2* cur = sm + C * fft_buf(L);
+    float2* nxt = sm;
+    line_fft<LOGL, INV>(x, t, cur, nxt, [&](int pos) { return (fft_pad(pos) << lc) + c; }, [] { __syncthreads(); }, W);
+    if (on) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) p[(long long)(t + k * T) * D.W1] = x[k];
+    }
+}
+
+enum { A3_ASSEMBLE = 0, A3_PRECOND = 1, A3_ENERGY = 2 };
+struct Axis1Args {
+    const float2* B;   // three spectra (A3_ASSEMBLE: of b; A3_PRECOND: of r; A3_ENERGY: unused)
+    const float2* V;   // three spectra of v (A3_ASSEMBLE, A3_ENERGY)
+    float2* out;       // three spectra
+    double* part;      // nullable: per-block energy sums (reg, w), 3 doubles per block (the first 0)
+    float beta, beta_w, invN;
+    int mode;          // K^: 0 identity, 1 incompressible, 2 mass source
+};
+
+__device__ __forceinline__ float k_odd(int i, int n) { return i < n / 2 ? (float)i : (i == n / 2 ? 0.f : (float)(i - n)); }
+__device__ __forceinline__ float k_even(int i, int n) { return i < n / 2 ? (float)i : (float)(i - n); }
+
+// fixed-order sum over the block (a power of two of threads, at most 256)
+__device__ __forceinline__ double block_sum3(double v) {
+    __shared__ double sh[R3_THREADS];
+    __syncthreads();
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+        __syncthreads();
+    }
+    return sh[0];
+}
+
+// axis 1: forward, multiplier, inverse.  Column l = i2 W1 + e, entries n2 W1 apart.
+//   A3_ASSEMBLE: beta |k|^2 V + K^ B, K^ = I - k~ k~^T / (|k~|^2 [+ beta |k|^2 / (beta_w (1 + |k|^2))])
+//   A3_PRECOND:  B / (beta |k|^2), the k = 0 symbol of A replaced by 1 (App. E)
+//   A3_ENERGY:   no output; sums of |k|^2 |V|^2 and (1 + |k|^2) |k~ . V|^2 over the full spectrum
+//                (an entry with 0 < e < n3 / 2 stands for itself and its conjugate)
+template <int LOGL, int OP>
+__global__ void __launch_bounds__(128) k3_axis1(Axis1Args a, Dims3 D, int ncols, int C, int lc,
+                                                const float2* __restrict__ tw) {
+    extern __shared__ __align__(16) float2 sm[];
+    constexpr int L = 1 << LOGL, T = L >> 3;
+    constexpr int NV = OP == A3_PRECOND ? 0 : 3, NB = OP == A3_ENERGY ? 0 : 3;
+    const int c = threadIdx.x & (C - 1), t = threadIdx.x >> lc;
+    const int l = blockIdx.x * C + c;
+    const bool on = l < ncols;
+    const long long S = (long long)D.n2 * D.W1;
+    LineTw<LOGL> W;
+    W.load(tw, t);
+    pdl_entry();
+    float2* cur = sm + C * fft_buf(L);
+    float2* nxt = sm;
+    auto idx = [&](int pos) { return (fft_pad(pos) << lc) + c; };
+    auto sync = [] { __syncthreads(); };
+    float2 xv[NV > 0 ? 3 : 1][8], xb[NB > 0 ? 3 : 1][8];
+#pragma unroll
+    for (int d = 0; d < NV; ++d) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) xv[d][k] = on ? a.V[d * D.NS + l + (t + k * T) * S] : make_float2(0.f, 0.f);
+        line_fft<LOGL, false>(xv[d], t, cur, nxt, idx, sync, W);
+    }
+#pragma unroll
+    for (int d = 0; d < NB; ++d) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) xb[d][k] = on ? a.B[d * D.NS + l + (t + k * T) * S] : make_float2(0.f, 0.f);
+        line_fft<LOGL, false>(xb[d], t, cur, nxt, idx, sync, W);
+    }
+    const int i2 = l / D.W1, e = l - i2 * D.W1;
+    const float k2 = k_odd(i2, D.n2), e2 = k_even(i2, D.n2);
+    const float k3 = e == D.n3 / 2 ? 0.f : (float)e, e3 = (float)e;
+    const double ew = (e == 0 || e == D.n3 / 2) ? 1.0 : 2.0;
+    double er = 0.0, eww = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int p = t + k * T;
+        const float k1 = k_odd(p, L), e1 = k_even(p, L);
+        const float kk = e1 * e1 + e2 * e2 + e3 * e3;
+        const float kd[3] = {k1, k2, k3};
+        if (OP != A3_PRECOND && a.part) {
+            double s = 0.0, wr = 0.0, wi = 0.0;
+#pragma unroll
+            for (int d = 0; d < NV; ++d) {
+                s += (double)xv[d][k].x * xv[d][k].x + (double)xv[d][k].y * xv[d][k].y;
+                wr += (double)kd[d] * xv[d][k].x;
+                wi += (double)kd[d] * xv[d][k].y;
             }
+            er += ew * (double)kk * s;
+            eww += ew * (1.0 + (double)kk) * (wr * wr + wi * wi);
         }
+        if (OP == A3_ASSEMBLE) {
+            const float ko = k1 * k1 + k2 * k2 + k3 * k3;
+            float cre = 0.f, cim = 0.f;
+            if (a.mode != 0 && ko > 0.f) {
+                const float denom = a.mode == 1 ? ko : ko + a.beta * kk / (a.beta_w * (1.f + kk));
+                cre = (k1 * xb[0][k].x + k2 * xb[NB > 1 ? 1 : 0][k].x + k3 * xb[NB > 2 ? 2 : 0][k].x) / denom;
+                cim = (k1 * xb[0][k].y + k2 * xb[NB > 1 ? 1 : 0][k].y + k3 * xb[NB > 2 ? 2 : 0][k].y) / denom;
+            }
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const float2 v = V[d * D.N + i];
-            out[d * D.N + i] = make_float2(beta * kk * v.x + b[d].x, beta * kk * v.y + b[d].y);
-        }
-    }
-}
-
-// f = Re(F) / N
-__global__ void k3_c2real(const float2* __restrict__ F, float* __restrict__ f, long long n, float invN) {
-    GRID_STRIDE(i, n) f[i] = F[i].x * invN;
-}
-
-// advection stage of the state (src == nullptr) or incremental state equation:
-//   k = -grad y . v - src . vt  (grad y = Re(G) / N);  gm_out (optional) = grad y
-//   stage 1: kbuf = k, y_out = y + h k;  stage 2: y_out = y + h / 2 (kbuf + k)
-__global__ void k3_adv_stage(const float2* __restrict__ G, const float* __restrict__ v, const float* __restrict__ src,
-                             const float* __restrict__ vt, const float* y, float* __restrict__ kbuf,
-                             float* y_out, float* __restrict__ gm_out, long long N, float invN, float h,  // y_out may be y
-                             int stage) {
-    GRID_STRIDE(i, N) {
-        const float g0 = G[i].x * invN, g1 = G[N + i].x * invN, g2 = G[2 * N + i].x * invN;
-        if (gm_out) {
-            gm_out[i] = g0;
-            gm_out[N + i] = g1;
-            gm_out[2 * N + i] = g2;
-        }
-        float k = -(g0 * v[i] + g1 * v[N + i] + g2 * v[2 * N + i]);
-        if (src) k -= src[i] * vt[i] + src[N + i] * vt[N + i] + src[2 * N + i] * vt[2 * N + i];
-        if (stage == 1) {
-            kbuf[i] = k;
-            y_out[i] = y[i] + h * k;
-        } else {
-            y_out[i] = y[i] + 0.5f * h * (kbuf[i] + k);
-        }
-    }
-}
-
-// U_d = (lam v_d, 0): the flux of the adjoint transport, ready for the forward transforms
-__global__ void k3_flux(const float* __restrict__ lam, const float* __restrict__ v, float2* __restrict__ U, long long N) {
-    GRID_STRIDE(i, N) {
-        const float l = lam[i];
-        U[i] = make_float2(l * v[i], 0.f);
-        U[N + i] = make_float2(l * v[N + i], 0.f);
-        U[2 * N + i] = make_float2(l * v[2 * N + i], 0.f);
-    }
-}
-
-// adjoint stage, k = div(lam v) = Re(F) / N (time reversed: d_tau lam = div(lam v))
-__global__ void k3_adj_stage(const float2* __restrict__ F, const float* y, float* __restrict__ kbuf,
-                             float* y_out, long long N, float invN, float h, int stage) {  // y_out may be y
-    GRID_STRIDE(i, N) {
-        const float k = F[i].x * invN;
-        if (stage == 1) {
-            kbuf[i] = k;
-            y_out[i] = y[i] + h * k;
-        } else {
-            y_out[i] = y[i] + 0.5f * h * (kbuf[i] + k);
-        }
-    }
-}
-
-// b (+)= w lam grad m (trapezoid weight w; first = 1 overwrites)
-__global__ void k3_body_force(const float* __restrict__ lam, const float* __restrict__ gm, float* __restrict__ b,
-                              long long N, float w, int first) {
-    GRID_STRIDE(i, N) {
-        const float l = w * lam[i];
+            for (int d = 0; d < NB; ++d) {
+                const float2 v = xv[d < NV ? d : 0][k];
+                const float br = xb[d][k].x - kd[d] * cre, bi = xb[d][k].y - kd[d] * cim;
+                xb[d][k] = make_float2((a.beta * kk * v.x + br) * a.invN, (a.beta * kk * v.y + bi) * a.invN);
+            }
+        } else if (OP == A3_PRECOND) {
+            const float s = a.invN / (a.beta * (kk > 0.f ? kk : 1.f));
 #pragma unroll
-        for (int d = 0; d < 3; ++d) b[d * N + i] = (first ? 0.f : b[d * N + i]) + l * gm[d * N + i];
+            for (int d = 0; d < NB; ++d) xb[d][k] = make_float2(xb[d][k].x * s, xb[d][k].y * s);
+        }
+    }
+    if (OP != A3_PRECOND && a.part) {
+        if (!on) er = eww = 0.0;
+        const double s1 = block_sum3(er), s2 = block_sum3(eww);
+        if (threadIdx.x == 0) {
+            a.part[blockIdx.x * 3] = 0.0;
+            a.part[blockIdx.x * 3 + 1] = s1;
+            a.part[blockIdx.x * 3 + 2] = s2;
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < NB; ++d) {
+        line_fft<LOGL, true>(xb[d], t, cur, nxt, idx, sync, W);
+        if (on) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a.out[d * D.NS + l + (t + k * T) * S] = xb[d][k];
+        }
     }
 }
 
-// y = a x (scale), used for lam(1) = m_R - m(1) and lam~(1) = -m~(1)
-__global__ void k3_axpy(const float* __restrict__ x, const float* __restrict__ z, float* __restrict__ y, long long N,
-                        float a, float c) {
-    GRID_STRIDE(i, N) y[i] = a * x[i] + (z ? c * z[i] : 0.f);
-}
-
-// per-block FP64 partial sums of the objective terms, reduced in a fixed order by k3_reduce:
-// data: sum (mR - m1)^2; reg: sum_k |k|^2 |V_d|^2; w: sum_k (1 + |k|^2) |i k~ . V|^2
-__global__ void __launch_bounds__(R3_THREADS) k3_energy_part(const float* __restrict__ mR, const float* __restrict__ m1,
-                                                             const float2* __restrict__ V, Dims3 D, double* part) {
-    __shared__ double s[3][R3_THREADS];
-    double a = 0.0, r = 0.0, wv = 0.0;
-    GRID_STRIDE(i, D.N) {
+// ---- reductions: per-block FP64 partial sums (3 doubles per block), summed in a fixed order by k3_reduce ----
+// sum (mR - m1)^2
+__global__ void __launch_bounds__(R3_THREADS) k3_data_part(const float* __restrict__ mR, const float* __restrict__ m1,
+                                                           long long N, double* part) {
+    pdl_entry();
+    double a = 0.0;
+    GRID_STRIDE(i, N) {
         const double d = (double)mR[i] - (double)m1[i];
         a += d * d;
-        float k1, k2, k3, kk;
-        wave3(D, i, k1, k2, k3, kk);
-        double e = 0.0;
-        float2 vv[3];
+    }
+    const double s = block_sum3(a);
+    if (threadIdx.x < 3) part[blockIdx.x * 3 + threadIdx.x] = threadIdx.x == 0 ? s : 0.0;
+}
+
+__global__ void __launch_bounds__(R3_THREADS) k3_reduce(const double* __restrict__ part, int nblk, double* out) {
+    pdl_entry();
+    double a[3] = {0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nblk; b += blockDim.x)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            vv[c] = V[c * D.N + i];
-            e += (double)vv[c].x * vv[c].x + (double)vv[c].y * vv[c].y;
-        }
-        r += (double)kk * e;
-        const double wre = (double)k1 * vv[0].x + (double)k2 * vv[1].x + (double)k3 * vv[2].x;
-        const double wim = (double)k1 * vv[0].y + (double)k2 * vv[1].y + (double)k3 * vv[2].y;
-        wv += (1.0 + kk) * (wre * wre + wim * wim);
-    }
-    s[0][threadIdx.x] = a;
-    s[1][threadIdx.x] = r;
-    s[2][threadIdx.x] = wv;
-    __syncthreads();
-    for (int o = R3_THREADS / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int q = 0; q < 3; ++q) s[q][threadIdx.x] += s[q][threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x < 3) part[blockIdx.x * 3 + threadIdx.x] = s[threadIdx.x][0];
-}
-
-__global__ void k3_reduce(const double* __restrict__ part, int nblk, double* out) {
-    if (threadIdx.x < 3) {
-        double t = 0.0;
-        for (int b = 0; b < nblk; ++b) t += part[b * 3 + threadIdx.x];
-        out[threadIdx.x] = t;
+        for (int q = 0; q < 3; ++q) a[q] += part[b * 3 + q];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double s = block_sum3(a[q]);
+        if (threadIdx.x == 0) out[q] = s;
     }
 }
 
-// per-block FP64 partial sums of sum_i a_i b_i (fixed-order reduction by k3_reduce)
+// sum_i a_i b_i
 __global__ void __launch_bounds__(R3_THREADS) k3_dot_part(const float* __restrict__ a, const float* __restrict__ b,
                                                           long long n, double* part) {
-    __shared__ double sh[R3_THREADS];
+    pdl_entry();
     double t = 0.0;
     GRID_STRIDE(i, n) t += (double)a[i] * (double)b[i];
-    sh[threadIdx.x] = t;
-    __syncthreads();
-    for (int o = R3_THREADS / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        part[blockIdx.x * 3] = sh[0];
-        part[blockIdx.x * 3 + 1] = 0.0;
-        part[blockIdx.x * 3 + 2] = 0.0;
-    }
+    const double s = block_sum3(t);
+    if (threadIdx.x < 3) part[blockIdx.x * 3 + threadIdx.x] = threadIdx.x == 0 ? s : 0.0;
 }
 
-// y = a x + b y
+// y = a x + b y (b == 0: y is not read)
 __global__ void k3_axpby(const float* x, float* y, long long n, float a, float b) {  // x may be y
-    GRID_STRIDE(i, n) y[i] = a * x[i] + b * y[i];
-}
-
-// (beta A)^-1 on three spectra, the k = 0 symbol of A replaced by 1 (App. E)
-__global__ void k3_precond_spec(float2* X, Dims3 D, float beta) {
-    GRID_STRIDE(i, D.N) {
-        float k1, k2, k3, kk;
-        wave3(D, i, k1, k2, k3, kk);
-        const float s = 1.f / (beta * (kk > 0.f ? kk : 1.f));
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const float2 x = X[d * D.N + i];
-            X[d * D.N + i] = make_float2(x.x * s, x.y * s);
-        }
-    }
+    pdl_entry();
+    GRID_STRIDE(i, n) y[i] = b != 0.f ? a * x[i] + b * y[i] : a * x[i];
 }
 
 }  // namespace
@@ -323,114 +373,219 @@ struct reg3_ctx {
     double beta, gamma;
     int kmode;  // 0: K = I (gamma = 0), 1: incompressible (gamma = inf), 2: mass source
     cudaStream_t stream;
-    float *mT, *mR, *v, *gm, *y, *ys, *kb, *lam, *g3, *bt, *mt;
-    float2 *F, *G;  // one spectrum, three spectra
+    cudaStream_t cap;  // the stream the launch sequences are captured on (created on first use)
+    float *mT, *mR, *v, *vt, *gm, *y, *ys, *lam, *src, *D1, *D2, *bt;
+    float2* S;   // six half spectra: 0..2 of b (and the results), 3..5 of v
+    float2* tw;
     double *d_part, *d_sum, *h_sum;
+    int npart;   // blocks d_part has room for
+    cudaGraphExec_t graphs[4];
     bool have_images, have_lin;
 };
 
 namespace {
 
-constexpr int R3_BLOCKS = 608;  // 4 per SM of a GB300 for the grid-stride kernels
-
 bool pow2_in(int n, int lo, int hi) { return n >= lo && n <= hi && (n & (n - 1)) == 0; }
+int ilog2(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
 
-LineMap line_map(const Dims3& D, int axis) {
-    LineMap m;
-    if (axis == 2) {
-        m.L = D.n3; m.S = 1; m.Q = D.n1 * D.n2; m.P = 0; m.R = D.n3; m.TWL = R3_TILE;
-    } else if (axis == 1) {
-        m.L = D.n2; m.S = D.n3; m.Q = D.n3; m.P = D.n2 * D.n3; m.R = 1; m.TWL = D.n3 < R3_TILE ? D.n3 : R3_TILE;
-    } else {
-        m.L = D.n1; m.S = D.n2 * D.n3; m.Q = D.n2 * D.n3; m.P = 0; m.R = 1; m.TWL = R3_TILE;
-    }
-    return m;
+template <typename... KArgs, typename... Args>
+void launch3(reg3_ctx* c, void (*kern)(KArgs...), dim3 grid, int block, size_t smem, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-size_t pass_smem(const LineMap& m) { return ((size_t)2 * m.L * (m.TWL + 1) + m.L / 2) * sizeof(float2); }
+// threads of a column kernel's block: large enough for 64-byte rows of columns on the longest
+// axis, small enough that a small box still has a block for every SM
+int col_threads(const Dims3& D) { return D.N >= (1 << 20) ? 256 : (D.N >= (1 << 17) ? 128 : 64); }
 
-// in-place 3-D transform of `count` consecutive spectra
-void fft3(reg3_ctx* c, float2* X, int count, bool inverse) {
-    for (int f = 0; f < count; ++f)
-        for (int axis = 2; axis >= 0; --axis) {
-            const LineMap m = line_map(c->D, axis);
-            const int tiles = (int)(c->D.N / m.L / m.TWL);
-            if (inverse)
-                k3_fft_pass<true><<<tiles, R3_THREADS, pass_smem(m), c->stream>>>(X + f * c->D.N, m);
-            else
-                k3_fft_pass<false><<<tiles, R3_THREADS, pass_smem(m), c->stream>>>(X + f * c->D.N, m);
-        }
+// D1 = d_1 (f mul1), D2 = d_2 (f mul2) (no factor where mul is nullptr)
+void d12(reg3_ctx* c, const float* f, const float* mul1, const float* mul2) {
+    const Dims3& D = c->D;
+    const int B = col_threads(D);
+    D12Args a;
+    a.a1 = DColArgs{f, mul1, nullptr, nullptr, c->D1};
+    a.a2 = DColArgs{f, mul2, nullptr, nullptr, c->D2};
+    const int nc1 = D.n2 * D.n3 / 2, nc2 = D.n1 * D.n3 / 2;
+    a.m1 = ColMap{D.l2 + D.l3 - 1, 0, nc1, nc1};
+    a.m2 = ColMap{D.l3 - 1, D.n2 * D.n3 / 2, D.n3 / 2, nc2};
+    a.log1 = D.l1;
+    a.log2 = D.l2;
+    a.lc1 = ilog2(B) + 3 - D.l1;
+    a.lc2 = ilog2(B) + 3 - D.l2;
+    a.tiles1 = (nc1 + (1 << a.lc1) - 1) >> a.lc1;
+    const int tiles2 = (nc2 + (1 << a.lc2) - 1) >> a.lc2;
+    launch3(c, k3_d12, a.tiles1 + tiles2, B, dcol_smem(B / 16, 128), a, c->tw);
 }
 
-// G = the three spectra of grad f (still to be inverse-transformed and scaled by 1 / N)
-void grad_spectra(reg3_ctx* c, const float* f) {
-    k3_real2c<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(f, c->F, c->D.N);
-    fft3(c, c->F, 1, false);
-    k3_grad_spec<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->F, c->G, c->D);
-    fft3(c, c->G, 3, true);
+// row kernels: 128 threads a block (64 for small boxes), at most the box's pairs of rows
+struct Row3 { int lines, threads, grid; size_t smem; };
+Row3 row3(const Dims3& D) {
+    Row3 r;
+    const int T = D.n3 / 8, pairs = D.n1 * D.n2 / 2;
+    int th = D.N >= (1 << 18) ? 128 : 64;
+    if (th < 32) th = 32;
+    r.lines = th / T;
+    if (r.lines > pairs) r.lines = pairs;
+    r.threads = r.lines * T;
+    r.grid = pairs / r.lines;
+    r.smem = drow_smem(r.lines, D.n3);
+    return r;
 }
 
-// state (src == nullptr, from y0 into c->y, gradient history into c->gm) or incremental
-// state (source grad m_j . vt from the stored history, from 0, into c->mt)
-void forward_solve(reg3_ctx* c, const float* y0, const float* vt) {
+void adv(reg3_ctx* c, const AdvRow<3>& a) {
+    const Row3 r = row3(c->D);
+    DISPATCH3(c->D.l3, launch3(c, k3_adv<LG>, r.grid, r.threads, r.smem, a, c->D.N, r.lines, c->tw));
+}
+
+// state (vt == nullptr: y from mT into c->y, gradient history into c->gm) or incremental state
+// (source grad m_j . vt from the stored history, from 0, into c->y)
+void forward_solve(reg3_ctx* c, const float* vt) {
     const long long N = c->D.N;
-    const float h = 1.f / c->nt, invN = 1.f / (float)N;
-    float* y = vt ? c->mt : c->y;
-    if (y0) cudaMemcpyAsync(y, y0, sizeof(float) * N, cudaMemcpyDeviceToDevice, c->stream);
-    else cudaMemsetAsync(y, 0, sizeof(float) * N, c->stream);
+    const float h = 1.f / c->nt;
+    float* y = c->y;
+    AdvRow<3> a = {};
+    a.D[0] = c->D1;
+    a.D[1] = c->D2;
+    a.v = c->v;
+    a.vt = vt;
+    a.h = h;
     for (int j = 0; j < c->nt; ++j) {
-        grad_spectra(c, y);
-        k3_adv_stage<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, c->v, vt ? c->gm + 3 * N * j : nullptr, vt, y,
-                                                              c->kb, c->ys, vt ? nullptr : c->gm + 3 * N * j, N,
-                                                              invN, h, 1);
-        grad_spectra(c, c->ys);
-        k3_adv_stage<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, c->v, vt ? c->gm + 3 * N * (j + 1) : nullptr, vt,
-                                                              y, c->kb, y, nullptr, N, invN, h, 2);
+        const float* yj = j > 0 ? y : (vt ? nullptr : c->mT);
+        a.uj = yj;
+        a.us = nullptr;
+        a.stage = 1;
+        a.u_out = c->ys;
+        a.zero = yj ? 0 : 1;
+        a.late = a.zero;  // the first launch of the solve
+        a.src_in = (vt && j > 0) ? c->src : nullptr;
+        a.gm = vt ? c->gm + 3 * N * j : nullptr;
+        a.src_out = nullptr;
+        a.grad_out = vt ? nullptr : c->gm + 3 * N * j;
+        if (yj) d12(c, yj, nullptr, nullptr);
+        adv(c, a);
+        d12(c, c->ys, nullptr, nullptr);
+        a.us = c->ys;
+        a.stage = 2;
+        a.u_out = y;
+        a.zero = a.late = 0;
+        a.src_in = nullptr;
+        a.gm = vt ? c->gm + 3 * N * (j + 1) : nullptr;
+        a.src_out = (vt && j + 1 < c->nt) ? c->src : nullptr;
+        a.grad_out = nullptr;
+        adv(c, a);
     }
     if (!vt) {  // grad m(t = 1) completes the history
-        grad_spectra(c, y);
-        k3_adv_stage<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, c->v, nullptr, nullptr, y, c->kb, c->ys,
-                                                              c->gm + 3 * N * c->nt, N, invN, h, 1);
+        d12(c, y, nullptr, nullptr);
+        a.uj = y;
+        a.us = nullptr;
+        a.stage = 1;
+        a.u_out = nullptr;
+        a.grad_out = c->gm + 3 * N * c->nt;
+        adv(c, a);
     }
 }
 
-// adjoint transport backward from c->lam = lam(1), accumulating out = int lam grad m dt
-void adjoint_solve(reg3_ctx* c, float* out) {
+// adjoint transport backward from lam(1) = ca x + cb c->y (x nullable), accumulating out = int lam grad m dt
+void adjoint_solve(reg3_ctx* c, const float* x, float ca, float cb, float* out) {
     const long long N = c->D.N;
     const int nt = c->nt;
-    const float h = 1.f / nt, invN = 1.f / (float)N;
+    const float h = 1.f / nt;
+    launch3(c, k3_adj_init, R3_BLOCKS, R3_THREADS, 0, x, ca, c->y, cb, c->lam, out, c->gm + 3 * N * nt, 0.5f * h, N);
+    const Row3 r = row3(c->D);
+    AdjRow<3> a = {};
+    a.D[0] = c->D1;
+    a.D[1] = c->D2;
+    a.v = c->v;
+    a.h = h;
+    a.lj = c->lam;
     for (int j = nt; j >= 1; --j) {
-        k3_body_force<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->lam, c->gm + 3 * N * j, out, N,
-                                                               j == nt ? 0.5f * h : h, j == nt);
-        k3_flux<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->lam, c->v, c->G, N);
-        fft3(c, c->G, 3, false);
-        k3_div_spec<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, c->F, c->D);
-        fft3(c, c->F, 1, true);
-        k3_adj_stage<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->F, c->lam, c->kb, c->ys, N, invN, h, 1);
-        k3_flux<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->ys, c->v, c->G, N);
-        fft3(c, c->G, 3, false);
-        k3_div_spec<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, c->F, c->D);
-        fft3(c, c->F, 1, true);
-        k3_adj_stage<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->F, c->lam, c->kb, c->lam, N, invN, h, 2);
+        d12(c, c->lam, c->v, c->v + N);
+        a.stage = 1;
+        a.ls = nullptr;
+        a.l_out = c->ys;
+        a.b = nullptr;
+        DISPATCH3(c->D.l3, launch3(c, k3_adj<LG>, r.grid, r.threads, r.smem, a, N, r.lines, c->tw));
+        d12(c, c->ys, c->v, c->v + N);
+        a.stage = 2;
+        a.ls = c->ys;
+        a.l_out = c->lam;
+        a.b = out;
+        a.gm = c->gm + 3 * N * (j - 1);
+        a.w = j == 1 ? 0.5f * h : h;
+        DISPATCH3(c->D.l3, launch3(c, k3_adj<LG>, r.grid, r.threads, r.smem, a, N, r.lines, c->tw));
     }
-    k3_body_force<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->lam, c->gm, out, N, 0.5f * h, 0);
 }
 
-// out = beta A x + K b (x, b vector fields); leaves the spectra of x in c->G
-void assemble(reg3_ctx* c, const float* x, const float* b, float* out) {
-    const long long N = c->D.N;
-    // spectra of b in c->G, of x in the scratch g3 (3 complex fields)
-    k3_real2c<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(b, c->G, 3 * N);
-    fft3(c, c->G, 3, false);
-    float2* X = reinterpret_cast<float2*>(c->g3);  // 3 complex fields of scratch (6N floats)
-    k3_real2c<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(x, X, 3 * N);
-    fft3(c, X, 3, false);
-    k3_assemble<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(X, c->G, c->G, c->D, (float)c->beta, c->kmode,
-                                                         (float)c->gamma);
-    fft3(c, c->G, 3, true);
-    k3_c2real<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, out, 3 * N, 1.f / (float)N);
-    k3_energy_part<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->mR, c->y, X, c->D, c->d_part);
-    k3_reduce<<<1, 32, 0, c->stream>>>(c->d_part, R3_BLOCKS, c->d_sum);
+// ---- spectral assembly ----
+void rows_r2c(reg3_ctx* c, const float* p0, const float* p1, float2* S, int nf) {
+    const Row3 r = row3(c->D);
+    DISPATCH3(c->D.l3, launch3(c, k3_r2c<LG>, dim3(r.grid, nf), r.threads, r.smem, p0, p1, S, c->D, r.lines, c->tw));
+}
+void rows_c2r(reg3_ctx* c, const float2* S, float* out) {
+    const Row3 r = row3(c->D);
+    DISPATCH3(c->D.l3, launch3(c, k3_c2r<LG>, dim3(r.grid, 3), r.threads, r.smem, S, out, c->D, r.lines, c->tw));
+}
+// complex column kernels: 128 threads a block
+struct Col3 { int C, lc, grid; size_t smem; };
+Col3 col3(int logl, int ncols) {
+    Col3 k;
+    k.lc = 7 + 3 - logl;
+    k.C = 1 << k.lc;
+    k.grid = (ncols + k.C - 1) / k.C;
+    k.smem = dcol_smem(k.C, 1 << logl);
+    return k;
+}
+void axis2(reg3_ctx* c, float2* S, int nf, bool inv) {
+    const int nc = nf * c->D.n1 * c->D.W1;
+    const Col3 k = col3(c->D.l2, nc);
+    if (inv) DISPATCH3(c->D.l2, launch3(c, k3_axis2<LG, true>, k.grid, 128, k.smem, S, c->D, nc, k.C, k.lc, c->tw))
+    else DISPATCH3(c->D.l2, launch3(c, k3_axis2<LG, false>, k.grid, 128, k.smem, S, c->D, nc, k.C, k.lc, c->tw))
+}
+// returns the number of blocks (partial sums, where a.part is set)
+int axis1(reg3_ctx* c, int op, double* part) {
+    Axis1Args a;
+    a.B = c->S;
+    a.V = c->S + 3 * c->D.NS;
+    a.out = c->S;
+    a.part = part;
+    a.beta = (float)c->beta;
+    a.beta_w = (float)c->gamma;
+    a.invN = 1.f / (float)c->D.N;
+    a.mode = c->kmode;
+    const int nc = c->D.n2 * c->D.W1;
+    const Col3 k = col3(c->D.l1, nc);
+    if (op == A3_ASSEMBLE)
+        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_ASSEMBLE>, k.grid, 128, k.smem, a, c->D, nc, k.C, k.lc, c->tw))
+    else if (op == A3_PRECOND)
+        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_PRECOND>, k.grid, 128, k.smem, a, c->D, nc, k.C, k.lc, c->tw))
+    else
+        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_ENERGY>, k.grid, 128, k.smem, a, c->D, nc, k.C, k.lc, c->tw))
+    return k.grid;
+}
+
+// the parts of J into d_sum: sum (mR - m(1))^2 from the fields, the energies from nblk partial sums
+// that follow the data blocks
+void reduce_objective(reg3_ctx* c, int nblk) {
+    launch3(c, k3_data_part, R3_BLOCKS, R3_THREADS, 0, c->mR, c->y, c->D.N, c->d_part);
+    launch3(c, k3_reduce, 1, R3_THREADS, 0, c->d_part, R3_BLOCKS + nblk, c->d_sum);
+}
+
+// spectra of beta A x + K b left in c->S (rows_c2r finishes); energy: with the sums of J
+void assemble(reg3_ctx* c, const float* x, const float* b, bool energy) {
+    rows_r2c(c, b, x, c->S, 6);
+    axis2(c, c->S, 6, false);
+    const int nblk = axis1(c, A3_ASSEMBLE, energy ? c->d_part + 3 * R3_BLOCKS : nullptr);
+    axis2(c, c->S, 3, true);
+    if (energy) reduce_objective(c, nblk);
 }
 
 int r3_err(const char* what) {
@@ -438,12 +593,57 @@ int r3_err(const char* what) {
     return e == cudaSuccess ? REG_OK : reg_fail(REG_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// Run a launch sequence that touches the context's own buffers only: captured once per context
+// into a CUDA graph on a stream of the context's own (the legacy default stream cannot be
+// captured) and replayed on its working stream.  While the caller captures that stream the
+// launches go into the caller's graph instead.
+enum { G3_GRADIENT = 0, G3_MATVEC = 1, G3_OBJECTIVE = 2 };
+template <typename F>
+int run3(reg3_ctx* c, int kind, F&& body) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) return r3_err("capture status");
+    if (cs != cudaStreamCaptureStatusNone) {
+        body();
+        return r3_err("launch");
+    }
+    if (!c->graphs[kind]) {
+        if (!c->cap && cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess)
+            return r3_err("capture stream");
+        if (cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed) != cudaSuccess) return r3_err("capture");
+        const cudaStream_t s = c->stream;
+        c->stream = c->cap;
+        body();
+        c->stream = s;
+        cudaGraph_t graph = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(c->cap, &graph);
+        if (e != cudaSuccess || !graph) return r3_err("capture");
+        const cudaError_t ei = cudaGraphInstantiate(&c->graphs[kind], graph, 0);
+        cudaGraphDestroy(graph);
+        if (ei != cudaSuccess) {
+            c->graphs[kind] = nullptr;
+            return r3_err("graph");
+        }
+    }
+    cudaGraphLaunch(c->graphs[kind], c->stream);
+    return r3_err("graph launch");
+}
+
+double objective_value(reg3_ctx* c) {
+    const double hv = std::pow(2.0 * M_PI, 3) / (double)c->D.N;
+    double J = 0.5 * hv * c->h_sum[0] + 0.5 * c->beta * hv / (double)c->D.N * c->h_sum[1];
+    if (c->kmode == 2) J += 0.5 * c->gamma * hv / (double)c->D.N * c->h_sum[2];
+    return J;
+}
+
 }  // namespace
 
 extern "C" void reg3_destroy(reg3_ctx* c) {
     if (!c) return;
-    void* ptrs[] = {c->mT, c->mR, c->v, c->gm, c->y, c->ys, c->kb, c->lam, c->g3, c->bt, c->mt, c->F, c->G,
-                    c->d_part, c->d_sum};
+    for (cudaGraphExec_t g : c->graphs)
+        if (g) cudaGraphExecDestroy(g);
+    if (c->cap) cudaStreamDestroy(c->cap);
+    void* ptrs[] = {c->mT, c->mR, c->v, c->vt, c->gm, c->y, c->ys, c->lam, c->src, c->D1, c->D2, c->bt,
+                    c->S, c->tw, c->d_part, c->d_sum};
     for (void* p : ptrs) cudaFree(p);
     cudaFreeHost(c->h_sum);
     delete c;
@@ -458,29 +658,32 @@ extern "C" int reg3_create(int n1, int n2, int n3, int nt, double beta, double g
     if (!(beta > 0.0) || !std::isfinite(beta)) return reg_fail(REG_ERR_ARG, "beta must be positive and finite");
     if (!(gamma >= 0.0)) return reg_fail(REG_ERR_ARG, "gamma must be >= 0 (INFINITY: incompressible)");
     reg3_ctx* c = new reg3_ctx();
-    c->D = Dims3{n1, n2, n3, (long long)n1 * n2 * n3};
+    c->D = Dims3{n1, n2, n3, (long long)n1 * n2 * n3, ilog2(n1), ilog2(n2), ilog2(n3), n3 / 2 + 1,
+                 (long long)n1 * n2 * (n3 / 2 + 1)};
     c->nt = nt;
     c->beta = beta;
     c->gamma = gamma;
     c->kmode = gamma == 0.0 ? 0 : (std::isinf(gamma) ? 1 : 2);
     c->stream = 0;
+    c->npart = R3_BLOCKS + col3(c->D.l1, n2 * c->D.W1).grid;
     const size_t N = (size_t)c->D.N;
     bool ok = true;
     auto M = [&](void** p, size_t bytes) { if (ok && cudaMalloc(p, bytes) != cudaSuccess) ok = false; };
     M((void**)&c->mT, sizeof(float) * N);
     M((void**)&c->mR, sizeof(float) * N);
     M((void**)&c->v, sizeof(float) * 3 * N);
+    M((void**)&c->vt, sizeof(float) * 3 * N);
     M((void**)&c->gm, sizeof(float) * 3 * N * (nt + 1));
     M((void**)&c->y, sizeof(float) * N);
     M((void**)&c->ys, sizeof(float) * N);
-    M((void**)&c->kb, sizeof(float) * N);
     M((void**)&c->lam, sizeof(float) * N);
-    M((void**)&c->g3, sizeof(float) * 6 * N);
+    M((void**)&c->src, sizeof(float) * N);
+    M((void**)&c->D1, sizeof(float) * N);
+    M((void**)&c->D2, sizeof(float) * N);
     M((void**)&c->bt, sizeof(float) * 3 * N);
-    M((void**)&c->mt, sizeof(float) * N);
-    M((void**)&c->F, sizeof(float2) * N);
-    M((void**)&c->G, sizeof(float2) * 3 * N);
-    M((void**)&c->d_part, sizeof(double) * 3 * R3_BLOCKS);
+    M((void**)&c->S, sizeof(float2) * 6 * (size_t)c->D.NS);
+    M((void**)&c->tw, sizeof(float2) * REG_TW_TOTAL);
+    M((void**)&c->d_part, sizeof(double) * 3 * c->npart);
     M((void**)&c->d_sum, sizeof(double) * 3);
     if (ok && cudaMallocHost((void**)&c->h_sum, sizeof(double) * 3) != cudaSuccess) ok = false;
     if (!ok) {
@@ -488,15 +691,7 @@ extern "C" int reg3_create(int n1, int n2, int n3, int nt, double beta, double g
         reg3_destroy(c);
         return reg_fail(REG_ERR_NOMEM, "3-D context allocation failed");
     }
-    // the opt-in is a per-kernel, per-device attribute shared by every context: always the
-    // largest tile any legal grid needs (256-point lines, 32 per CTA), so that a smaller context
-    // created later never lowers it under a larger one
-    LineMap mmax;
-    mmax.L = 256;
-    mmax.TWL = R3_TILE;
-    const size_t smax = pass_smem(mmax);
-    cudaFuncSetAttribute(k3_fft_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
-    cudaFuncSetAttribute(k3_fft_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
+    upload_twiddles(c->tw);
     const int st = r3_err("3-D context set-up");
     if (st != REG_OK) {
         reg3_destroy(c);
@@ -526,17 +721,18 @@ extern "C" int reg3_gradient(reg3_ctx* c, const float* v, float* g, double* J) {
     if (!c->have_images) return reg_fail(REG_ERR_STATE, "reg3_set_images first");
     const long long N = c->D.N;
     cudaMemcpyAsync(c->v, v, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, c->stream);
-    forward_solve(c, c->mT, nullptr);                                                         // m, grad m history
-    k3_axpy<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->mR, c->y, c->lam, N, 1.f, -1.f);     // lam(1) = mR - m(1)
-    adjoint_solve(c, c->bt);                                                                   // b
-    assemble(c, c->v, c->bt, g);                                                               // beta A v + K b, J parts
+    int st = run3(c, G3_GRADIENT, [&] {
+        forward_solve(c, nullptr);                   // m, grad m history
+        adjoint_solve(c, c->mR, 1.f, -1.f, c->bt);   // lam(1) = mR - m(1), b
+        assemble(c, c->v, c->bt, true);              // beta A v + K b, J parts
+    });
+    if (st != REG_OK) return st;
+    rows_c2r(c, c->S, g);
     cudaMemcpyAsync(c->h_sum, c->d_sum, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->stream);
-    int st = r3_err("reg3_gradient");
+    st = r3_err("reg3_gradient");
     if (st != REG_OK) return st;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return r3_err("reg3_gradient");
-    const double hv = std::pow(2.0 * M_PI, 3) / (double)N;
-    double Jv = 0.5 * hv * c->h_sum[0] + 0.5 * c->beta * hv / (double)N * c->h_sum[1];
-    if (c->kmode == 2) Jv += 0.5 * c->gamma * hv / (double)N * c->h_sum[2];
+    const double Jv = objective_value(c);
     if (J) *J = Jv;
     if (!std::isfinite(Jv)) return reg_fail(REG_ERR_NAN, "objective is not finite");
     c->have_lin = true;
@@ -546,14 +742,14 @@ extern "C" int reg3_gradient(reg3_ctx* c, const float* v, float* g, double* J) {
 extern "C" int reg3_hessian_matvec(reg3_ctx* c, const float* vt, float* Hvt) {
     if (!c || !vt || !Hvt) return reg_fail(REG_ERR_ARG, "NULL argument");
     if (!c->have_lin) return reg_fail(REG_ERR_STATE, "reg3_gradient first (it fixes the linearization point)");
-    const long long N = c->D.N;
-    float* vtc = c->g3;  // the direction, kept while the solves run (the assembly reuses g3 after)
-    cudaMemcpyAsync(vtc, vt, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, c->stream);
-    forward_solve(c, nullptr, vtc);                                                           // m~ history end
-    k3_axpy<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->mt, nullptr, c->lam, N, -1.f, 0.f);  // lam~(1) = -m~(1)
-    adjoint_solve(c, c->bt);                                                                   // b~
-    // the assembly transforms x into g3 in place: give it vt from the caller's buffer
-    assemble(c, vt, c->bt, Hvt);
+    cudaMemcpyAsync(c->vt, vt, sizeof(float) * 3 * c->D.N, cudaMemcpyDeviceToDevice, c->stream);
+    const int st = run3(c, G3_MATVEC, [&] {
+        forward_solve(c, c->vt);                       // m~(1)
+        adjoint_solve(c, nullptr, 0.f, -1.f, c->bt);   // lam~(1) = -m~(1), b~
+        assemble(c, c->vt, c->bt, false);
+    });
+    if (st != REG_OK) return st;
+    rows_c2r(c, c->S, Hvt);
     return r3_err("reg3_hessian_matvec");
 }
 
@@ -561,40 +757,40 @@ namespace {
 
 // <a, b> on the grid (trapezoidal weight (2 pi)^3 / N) over 3 N values; synchronous
 double inner3(reg3_ctx* c, const float* a, const float* b) {
-    k3_dot_part<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(a, b, 3 * c->D.N, c->d_part);
-    k3_reduce<<<1, 32, 0, c->stream>>>(c->d_part, R3_BLOCKS, c->d_sum);
+    launch3(c, k3_dot_part, R3_BLOCKS, R3_THREADS, 0, a, b, 3 * c->D.N, c->d_part);
+    launch3(c, k3_reduce, 1, R3_THREADS, 0, c->d_part, R3_BLOCKS, c->d_sum);
     cudaMemcpyAsync(c->h_sum, c->d_sum, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
     return std::pow(2.0 * M_PI, 3) / (double)c->D.N * c->h_sum[0];
 }
 
+void axpby3(reg3_ctx* c, const float* x, float* y, float a, float b) {
+    launch3(c, k3_axpby, R3_BLOCKS, R3_THREADS, 0, x, y, 3 * c->D.N, a, b);
+}
+
 void precond3(reg3_ctx* c, const float* r, float* out) {
-    const long long N = c->D.N;
-    k3_real2c<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(r, c->G, 3 * N);
-    fft3(c, c->G, 3, false);
-    k3_precond_spec<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, c->D, (float)c->beta);
-    fft3(c, c->G, 3, true);
-    k3_c2real<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->G, out, 3 * N, 1.f / (float)N);
+    rows_r2c(c, r, nullptr, c->S, 3);
+    axis2(c, c->S, 3, false);
+    axis1(c, A3_PRECOND, nullptr);
+    axis2(c, c->S, 3, true);
+    rows_c2r(c, c->S, out);
 }
 
 // J at x (one state solve; the gradient history is overwritten, which Algorithm 1 allows:
 // the next gradient evaluation rebuilds it at the accepted point)
 double objective3(reg3_ctx* c, const float* x) {
-    const long long N = c->D.N;
-    cudaMemcpyAsync(c->v, x, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, c->stream);
-    forward_solve(c, c->mT, nullptr);
-    float2* X = reinterpret_cast<float2*>(c->g3);
-    k3_real2c<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(x, X, 3 * N);
-    fft3(c, X, 3, false);
-    k3_energy_part<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(c->mR, c->y, X, c->D, c->d_part);
-    k3_reduce<<<1, 32, 0, c->stream>>>(c->d_part, R3_BLOCKS, c->d_sum);
+    cudaMemcpyAsync(c->v, x, sizeof(float) * 3 * c->D.N, cudaMemcpyDeviceToDevice, c->stream);
+    c->have_lin = false;
+    const int st = run3(c, G3_OBJECTIVE, [&] {
+        forward_solve(c, nullptr);
+        rows_r2c(c, c->v, nullptr, c->S + 3 * c->D.NS, 3);
+        axis2(c, c->S + 3 * c->D.NS, 3, false);
+        reduce_objective(c, axis1(c, A3_ENERGY, c->d_part + 3 * R3_BLOCKS));
+    });
+    if (st != REG_OK) return NAN;  // the caller's error check reports it
     cudaMemcpyAsync(c->h_sum, c->d_sum, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->stream);
     cudaStreamSynchronize(c->stream);
-    const double hv = std::pow(2.0 * M_PI, 3) / (double)N;
-    double J = 0.5 * hv * c->h_sum[0] + 0.5 * c->beta * hv / (double)N * c->h_sum[1];
-    if (c->kmode == 2) J += 0.5 * c->gamma * hv / (double)N * c->h_sum[2];
-    c->have_lin = false;
-    return J;
+    return objective_value(c);
 }
 
 }  // namespace
@@ -641,8 +837,7 @@ extern "C" int reg3_solve(reg3_ctx* c, float* v, double tol, int maxit_newton, i
         // Algorithm 2: preconditioned CG on H v~ = -g to ||r|| < eta ||g||
         const double eta = std::fmin(0.5, std::sqrt(gn / g0));
         cudaMemsetAsync(vt, 0, sizeof(float) * N3, c->stream);
-        cudaMemsetAsync(r, 0, sizeof(float) * N3, c->stream);
-        k3_axpby<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(g, r, N3, -1.f, 0.f);  // r = -g
+        axpby3(c, g, r, -1.f, 0.f);  // r = -g
         precond3(c, r, z);
         cudaMemcpyAsync(sd, z, sizeof(float) * N3, cudaMemcpyDeviceToDevice, c->stream);
         double rz = inner3(c, r, z);
@@ -656,18 +851,18 @@ extern "C" int reg3_solve(reg3_ctx* c, float* v, double tol, int maxit_newton, i
                 break;
             }
             const float kappa = (float)(rz / sHs);
-            k3_axpby<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(sd, vt, N3, kappa, 1.f);
-            k3_axpby<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(Hs, r, N3, -kappa, 1.f);
+            axpby3(c, sd, vt, kappa, 1.f);
+            axpby3(c, Hs, r, -kappa, 1.f);
             if (std::sqrt(inner3(c, r, r)) < eta * gn) break;
             precond3(c, r, z);
             const double rz_new = inner3(c, z, r);
-            k3_axpby<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(z, sd, N3, 1.f, (float)(rz_new / rz));
+            axpby3(c, z, sd, 1.f, (float)(rz_new / rz));
             rz = rz_new;
         }
         double gv = inner3(c, g, vt);
         if (gv >= 0.0) {  // not a descent direction: the preconditioned steepest descent step
             precond3(c, g, vt);
-            k3_axpby<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(vt, vt, N3, 0.f, -1.f);
+            axpby3(c, vt, vt, 0.f, -1.f);
             gv = inner3(c, g, vt);
         }
         // Armijo backtracking on J
@@ -675,7 +870,7 @@ extern "C" int reg3_solve(reg3_ctx* c, float* v, double tol, int maxit_newton, i
         bool accepted = false;
         for (int l = 0; l < max_ls; ++l) {
             cudaMemcpyAsync(vtrial, v, sizeof(float) * N3, cudaMemcpyDeviceToDevice, c->stream);
-            k3_axpby<<<R3_BLOCKS, R3_THREADS, 0, c->stream>>>(vt, vtrial, N3, (float)alpha, 1.f);
+            axpby3(c, vt, vtrial, (float)alpha, 1.f);
             ++nls;
             // a trial beyond the explicit scheme's stability gives a non-finite J: rejected like any
             // other trial that fails the sufficient-decrease test
