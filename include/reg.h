@@ -277,8 +277,8 @@ int reg_autotune(reg_grid grid, int nt, int concurrency, int force, int* rows_pe
                  int* prefetch, int* pdl, double* ms_per_matvec);
 
 /* The tiles and launch mode a context launches with (tuned, else the default
- * rule: the smallest R, C with at least 64 threads, P = 1 for n2 <= 512,
- * D = 1). */
+ * rule: the smallest R with R n2 / 8 >= 64, the smallest C >= 4 (2 for
+ * n1 = 1024) with C n1 / 8 >= 64, P = 1 for n2 <= 512, D = 1). */
 int reg_tile_config(reg_ctx* ctx, int* rows_per_cta, int* cols_per_cta, int* prefetch, int* pdl);
 
 /* Sets a context's tiles (validity as for reg_autotune; R = C = 0 restores

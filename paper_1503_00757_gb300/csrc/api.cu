@@ -9,6 +9,7 @@
 #include <cstring>
 #include <string>
 
+#include "deriv.cuh"
 #include "fft.cuh"
 #include "internal.h"
 
@@ -116,6 +117,7 @@ extern "C" void reg_destroy(reg_ctx* c) {
     for (int i = 0; i < 6; ++i) cudaFree(c->S[i]);
     free_hist(c);
     clear_graphs(c);
+    if (c->cap) cudaStreamDestroy(c->cap);
     for (auto g : c->timing_graphs) cudaGraphExecDestroy(g);
     cudaFree(c->d_scal);
     cudaFree(c->d_part);
@@ -168,6 +170,7 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->nt_cap = 0;
     set_params(c, nt, regnorm, beta, gamma, shear);
     c->stream = 0;
+    c->cap = nullptr;
     c->launches = 0;
     c->tileR = c->tileC = c->tileP = 0;
     c->pdl = true;
@@ -308,13 +311,17 @@ extern "C" int reg_set_stream(reg_ctx* c, void* stream) {
 
 // ---------------------------------------------------------------------------
 // CUDA graphs: each fixed launch sequence (objective, gradient tail, matvec,
-// one PCG iteration) is captured once per (kind, pointers, nt) and replayed.
-// Sequences run directly on the legacy default stream (it cannot be
-// captured) and while per-kernel timing is on.
+// one PCG iteration, det F, displacement) is captured once per (kind, internal
+// pointers, nt) and replayed.  The sequences touch the context's buffers only:
+// a caller's field is copied in before and the last kernel (spectra to the
+// caller's buffer) is launched after, so new buffers cost nothing.  The legacy
+// default stream cannot be captured: its sequences are captured on a stream of
+// the context's own and replayed on it.  While per-kernel timing is on they run
+// directly (legacy stream) or with event nodes.
 // ---------------------------------------------------------------------------
 enum GraphKind {
     GK_OBJECTIVE = 1, GK_GRADIENT = 2, GK_MATVEC = 3, GK_PCG_ITER = 4, GK_PCG_INIT = 5, GK_DETGRAD = 6,
-    GK_GRADIENT_Y = 7, GK_PCG_ITER_Y = 8, GK_PCG_INIT_Y = 9
+    GK_GRADIENT_Y = 7, GK_PCG_ITER_Y = 8, GK_PCG_INIT_Y = 9, GK_DISPLACEMENT = 10, GK_LABELS = 11
 };
 
 template <typename F>
@@ -336,7 +343,7 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         CK(cudaGraphLaunch(exec, c->stream));
         return REG_OK;
     }
-    if (!c->use_graphs || c->timing || c->stream == 0) {
+    if (!c->use_graphs || c->timing) {
         body();
         CKL();
         return REG_OK;
@@ -349,10 +356,20 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         }
     }
     const long long l0 = c->launches;
-    CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed));
+    const cudaStream_t user = c->stream;
+    if (user == 0) {
+        if (!c->cap) CK(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
+        c->stream = c->cap;
+    }
+    cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed);
+    if (e != cudaSuccess) {
+        c->stream = user;
+        return reg_fail(REG_ERR_CUDA, std::string("stream capture: ") + cudaGetErrorString(e));
+    }
     body();
     cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamEndCapture(c->stream, &graph);
+    e = cudaStreamEndCapture(c->stream, &graph);
+    c->stream = user;
     const long long nk = c->launches - l0;
     c->launches = l0;
     if (e != cudaSuccess || graph == nullptr) {
@@ -411,8 +428,21 @@ static SpecParams spec_params(reg_ctx* c, float coefA) {
 
 static double hh(reg_ctx* c) { return (2.0 * M_PI / c->n1) * (2.0 * M_PI / c->n2); }
 
-// grad of a scalar field into out (2N)
+static bool overlap(const float* a, size_t na, const float* b, size_t nb) { return a < b + nb && b < a + na; }
+
+// grad of a scalar field into out (2N).  The two derivatives are written while f is still read, so
+// a caller's f inside out is copied first.
 static void sp_grad(reg_ctx* c, const float* f, float* out) {
+    const size_t N = c->N;
+    if (overlap(f, N, out, 2 * N)) {
+        cudaMemcpyAsync(c->vx, f, sizeof(float) * N, cudaMemcpyDeviceToDevice, c->stream);
+        f = c->vx;
+    }
+    launch_grad(c, f, out);
+}
+
+// the same through the 2-D half spectrum
+static void sp_grad_spec(reg_ctx* c, const float* f, float* out) {
     launch_r2c_scalar(c, f, c->S[0]);
     const float2* in[1] = {c->S[0]};
     float2* o[2] = {c->S[1], c->S[2]};
@@ -421,11 +451,13 @@ static void sp_grad(reg_ctx* c, const float* f, float* out) {
 }
 
 static void sp_div(reg_ctx* c, const float* u, float* out) {
-    launch_r2c_vec(c, u, u + c->N, c->S[0], c->S[1]);
-    const float2* in[2] = {c->S[0], c->S[1]};
-    float2* o[1] = {c->S[2]};
-    launch_col(c, OP_DIV, in, o, spec_params(c, 0.f), nullptr);
-    launch_c2r_scalar(c, c->S[2], out);
+    const size_t N = c->N;
+    if (overlap(u, 2 * N, out, N)) {  // as above
+        cudaMemcpyAsync(c->vx, u, sizeof(float) * 2 * N, cudaMemcpyDeviceToDevice, c->stream);
+        u = c->vx;
+    }
+    launch_dcol(c, DColArgs{u, nullptr, nullptr, nullptr, out});
+    launch_add_d2(c, u + c->N, out);
 }
 
 static void sp_vec(reg_ctx* c, int op, float coefA, const float* u, float* out) {
@@ -436,14 +468,15 @@ static void sp_vec(reg_ctx* c, int op, float coefA, const float* u, float* out) 
     launch_c2r_vec(c, c->S[2], c->S[3], out, out + c->N);
 }
 
-// out = coefA A u + K b  (reduced gradient / Hessian assembly, Eq. (e:control-eq-elim), (e:inc-control-eq-elim))
+// out = coefA A u + K b  (reduced gradient / Hessian assembly, Eq. (e:control-eq-elim), (e:inc-control-eq-elim));
+// out == nullptr: the spectra stay in S[4], S[5] (finish_out)
 static void sp_assemble(reg_ctx* c, float coefA, const float* u, const float* b, float* out) {
     launch_r2c_vec(c, u, u + c->N, c->S[0], c->S[1]);
     launch_r2c_vec(c, b, b + c->N, c->S[2], c->S[3]);
     const float2* in[4] = {c->S[0], c->S[1], c->S[2], c->S[3]};
     float2* o[2] = {c->S[4], c->S[5]};
     launch_col(c, OP_ASSEMBLE, in, o, spec_params(c, coefA), nullptr);
-    launch_c2r_vec(c, c->S[4], c->S[5], out, out + c->N);
+    if (out) launch_c2r_vec(c, c->S[4], c->S[5], out, out + c->N);
 }
 
 // ---- preconditioned coordinates y = Q v, Q^ = (beta_v A'^)^(1/2), A'(0) = 1 ----
@@ -469,6 +502,12 @@ static void sp_qnorm(reg_ctx* c, const float* x, int slot) {
 static void sp_grad_vec(reg_ctx* c, const float* u, float* gv) {
     sp_grad(c, u, gv);
     sp_grad(c, u + c->N, gv + 2 * (size_t)c->N);
+}
+// for the shear model's strain, whose viscosity magnifies a change of its last bits: H v~ of the
+// nu = 3 test point moves by 1e-5 between the two ways to take the same gradient
+static void sp_grad_vec_spec(reg_ctx* c, const float* u, float* gv) {
+    sp_grad_spec(c, u, gv);
+    sp_grad_spec(c, u + c->N, gv + 2 * (size_t)c->N);
 }
 
 // out = div T (2 planes) of a symmetric tensor T = (T11, T12, T22)
@@ -502,7 +541,7 @@ static void shear_mass_assemble(reg_ctx* c, const float* T, float* Et, const flo
     if (c->pmode == PROJ_MASS) launch_axpby(c, 2 * N, 1.f, c->vx, 1.f, out, -1, -1, out);
 }
 
-// out = P_L(coefA div T + b), T = 3 planes (shear model)
+// out = P_L(coefA div T + b), T = 3 planes (shear model); out == nullptr: the spectra stay in S[5], S[0]
 static void sp_divt_proj(reg_ctx* c, float coefA, const float* T, const float* b, float* out) {
     const size_t N = c->N;
     launch_r2c_vec(c, T, T + N, c->S[0], c->S[1]);
@@ -511,13 +550,25 @@ static void sp_divt_proj(reg_ctx* c, float coefA, const float* T, const float* b
     const float2* in[5] = {c->S[0], c->S[1], c->S[2], c->S[3], c->S[4]};
     float2* o[2] = {c->S[5], c->S[0]};
     launch_col(c, OP_DIVT_PROJ, in, o, spec_params(c, coefA), nullptr);
-    launch_c2r_vec(c, c->S[5], c->S[0], out, out + N);
+    if (out) launch_c2r_vec(c, c->S[5], c->S[0], out, out + N);
+}
+
+// the result of gradient_launches / matvec_launches with a null output, into the caller's buffer
+static int finish_out(reg_ctx* c, float* out) {
+    if (!c->shear_model)
+        launch_c2r_vec(c, c->S[4], c->S[5], out, out + c->N);
+    else if (c->pmode == PROJ_LERAY)
+        launch_c2r_vec(c, c->S[5], c->S[0], out, out + c->N);
+    else
+        CK(cudaMemcpyAsync(out, c->vtmp2, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
+    CKL();
+    return REG_OK;
 }
 
 // regularization energy into d_scal[SL_JREG]
 static void reg_energy(reg_ctx* c, const float* v) {
     if (c->shear_model) {
-        sp_grad_vec(c, v, c->gtmp);
+        sp_grad_vec_spec(c, v, c->gtmp);
         int np = launch_shear_strain(c, c->gtmp, (float)c->nu, nullptr, nullptr, nullptr, c->d_part);
         const double coef = c->beta_v * (2.0 * c->nu / (c->nu + 1.0)) * hh(c);
         launch_finalize(c, c->d_part, np, c->d_scal + SL_JREG, coef, 0, 0);
@@ -541,19 +592,17 @@ static void reg_energy(reg_ctx* c, const float* v) {
 static float* mh(reg_ctx* c, int j) { return c->m_hist + (size_t)j * c->N; }
 static float* gmh(reg_ctx* c, int j) { return c->gm_hist + (size_t)j * 2 * c->N; }
 
+static float* lamh(reg_ctx* c, int j) { return c->lam_hist + (size_t)j * c->N; }
+static float* gmth(reg_ctx* c, int j) { return c->gmt_hist + (size_t)j * 2 * c->N; }
+
+// ---- the same solves with the stages in the row spectra (kernels.cu): H2 and H3 problems ----
+static bool sp_transport(const reg_ctx* c) { return c->ypath; }
+
 // State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[0..nt], gm_hist[0..nt].
 // The column pass transforms only d1 (OP_GRAD1); d2 is diagonal in the row
 // spectra and is formed by the row kernel from the stage's own spectrum S[0].
-// init (nullable): the field transported instead of the template m_T.
-static void state_solve(reg_ctx* c, const float* v, int nt, const float* init = nullptr) {
+static void state_solve_sp(reg_ctx* c, const float* v, int nt, const float* m0) {
     const float h = 1.0f / (float)nt;
-    const float* m0 = init ? init : c->mT;
-    if (c->use_tc && !c->full_newton) {
-        TcArgs a = {};
-        a.nt = nt; a.h = h; a.v = v; a.mT = m0; a.m_hist = c->m_hist; a.gm_hist = c->gm_hist; a.us = c->w0;
-        launch_transport_cluster(c, TC_STATE, a);
-        return;
-    }
     cudaMemcpyAsync(mh(c, 0), m0, sizeof(float) * c->N, cudaMemcpyDeviceToDevice, c->stream);
     launch_r2c_scalar(c, mh(c, 0), c->S[0]);
     const float2* in[1] = {c->S[0]};
@@ -581,19 +630,12 @@ static void state_solve(reg_ctx* c, const float* v, int nt, const float* init = 
 // (Eq. (e:inc-adj-eq-elim)) backward in time from lam_nt = ca*a + cb*cf, with
 // the body force b = int lam grad m dt (trapezoid) accumulated into bout.
 // lhist (nullable): store lam_j at lhist + j N for j = 0..nt (the full Newton matvec reads it).
-static void adjoint_solve(reg_ctx* c, const float* v, int nt, const float* a, float ca, const float* cf, float cb,
-                          float* bout, double* part_jdata, float* lhist = nullptr) {
+static void adjoint_solve_sp(reg_ctx* c, const float* v, int nt, const float* a, float ca, const float* cf, float cb,
+                          float* bout, float* lhist) {
     const float h = 1.0f / (float)nt;
-    if (c->use_tc && !part_jdata && !lhist) {
-        TcArgs t = {};
-        t.nt = nt; t.h = h; t.v = v; t.gm_hist = c->gm_hist; t.lj = c->w1; t.ls = c->w2;
-        t.adj_a = a; t.adj_ca = ca; t.adj_c = cf; t.adj_cb = cb; t.b = bout;
-        launch_transport_cluster(c, TC_ADJOINT, t);
-        return;
-    }
     float* lst = c->w2;
     auto lam_at = [&](int j) { return lhist ? lhist + (size_t)j * c->N : c->w1; };
-    launch_adj_init(c, a, ca, cf, cb, v, lam_at(nt), bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2], part_jdata);
+    launch_adj_init_sp(c, a, ca, cf, cb, v, lam_at(nt), bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2], nullptr);
     const float2* Fin[2] = {c->S[1], c->S[2]};
     float2* D[1] = {c->S[0]};
     const SpecParams P = spec_params(c, 0.f);
@@ -612,18 +654,15 @@ static void adjoint_solve(reg_ctx* c, const float* v, int nt, const float* a, fl
     }
 }
 
-static float* lamh(reg_ctx* c, int j) { return c->lam_hist + (size_t)j * c->N; }
-static float* gmth(reg_ctx* c, int j) { return c->gmt_hist + (size_t)j * 2 * c->N; }
-
 // Full-Newton incremental adjoint (Eq. (e:inc-adj-eq-elim) with the lambda term), backward from
 // lam~_nt = -m~_nt (c->w3): the flux of every divergence is lam~ v + lam v~ with lam from the
 // gradient's adjoint history at the time the divergence is evaluated, and the incremental body
 // force is b~ = sum_j w_j (lam~_j grad m_j + lam_j grad m~_j) (trapezoid).
-static void inc_adjoint_full(reg_ctx* c, const float* v, const float* vt, int nt, float* bout) {
+static void inc_adjoint_full_sp(reg_ctx* c, const float* v, const float* vt, int nt, float* bout) {
     const float h = 1.0f / (float)nt;
     float* lam = c->w1;
     float* lst = c->w2;
-    launch_adj_init(c, nullptr, 0.f, c->w3, -1.f, v, lam, bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2], nullptr,
+    launch_adj_init_sp(c, nullptr, 0.f, c->w3, -1.f, v, lam, bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2], nullptr,
                     lamh(c, nt), vt, gmth(c, nt));
     const float2* Fin[2] = {c->S[1], c->S[2]};
     float2* D[1] = {c->S[0]};
@@ -648,9 +687,7 @@ static void inc_adjoint_full(reg_ctx* c, const float* v, const float* vt, int nt
 // Incremental state (Eq. (e:inc-state-eq-elim)); leaves m~(1) in c->w3.
 // m~(0) = 0 is passed as u_j = nullptr to both stages of the first step.  gmt (nullable):
 // store grad m~_j at gmt + j 2N for j = 0..nt (the full Newton matvec reads it).
-// gm_fixed (nullable): a source gradient used at every time instead of the grad m history.
-static void inc_state_solve(reg_ctx* c, const float* v, const float* vt, int nt, float* gmt = nullptr,
-                            const float* gm_fixed = nullptr) {
+static void inc_state_solve_sp(reg_ctx* c, const float* v, const float* vt, int nt, float* gmt) {
     const float h = 1.0f / (float)nt;
     float* mj = c->w3;
     float* ms = c->w0;
@@ -663,7 +700,7 @@ static void inc_state_solve(reg_ctx* c, const float* v, const float* vt, int nt,
             launch_col(c, OP_GRAD1, in, G, P, nullptr);
             a.G1 = c->S[1]; a.Sd2 = c->S[0];
         }
-        a.uj = (j > 0) ? mj : nullptr; a.us = nullptr; a.v = v; a.gm = gm_fixed ? gm_fixed : gmh(c, j); a.vt = vt;
+        a.uj = (j > 0) ? mj : nullptr; a.us = nullptr; a.v = v; a.gm = gmh(c, j); a.vt = vt;
         a.u_out = ms; a.grad_out = gmt ? gmt + (size_t)j * 2 * c->N : nullptr; a.S_out = c->S[0]; a.h = h;
         a.stage = 1;
         // the first launch of the solve: v~ may come from the launch just before (Q^-1 s in
@@ -673,11 +710,149 @@ static void inc_state_solve(reg_ctx* c, const float* v, const float* vt, int nt,
         a.late = 0;
         launch_col(c, OP_GRAD1, in, G, P, nullptr);
         a.G1 = c->S[1]; a.Sd2 = c->S[0];
-        a.us = ms; a.gm = gm_fixed ? gm_fixed : gmh(c, j + 1); a.u_out = mj; a.stage = 2; a.grad_out = nullptr;
+        a.us = ms; a.gm = gmh(c, j + 1); a.u_out = mj; a.stage = 2; a.grad_out = nullptr;
         a.S_out = (j + 1 < nt) ? c->S[0] : nullptr;
         launch_row_adv(c, a);
     }
-    if (gmt) sp_grad(c, mj, gmt + (size_t)nt * 2 * c->N);
+    if (gmt) sp_grad_spec(c, mj, gmt + (size_t)nt * 2 * c->N);
+}
+
+// buffers of the transport solves: the x^1 derivative of the stage's field and the stored source
+// term.  They share memory with spectra that only the spectral operators use.
+static float* dbuf(reg_ctx* c) { return reinterpret_cast<float*>(c->S[1]); }
+static float* srcbuf(reg_ctx* c) { return reinterpret_cast<float*>(c->S[0]); }
+
+static void d1_of(reg_ctx* c, const float* f, const float* mul = nullptr, const float* f2 = nullptr,
+                  const float* mul2 = nullptr) {
+    launch_dcol(c, DColArgs{f, mul, f2, mul2, dbuf(c)});
+}
+
+// State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[1..nt], gm_hist[0..nt].
+// init (nullable): the field transported instead of the template m_T.
+static void state_solve(reg_ctx* c, const float* v, int nt, const float* init = nullptr) {
+    const float h = 1.0f / (float)nt;
+    const float* m0 = init ? init : c->mT;
+    if (c->use_tc && !c->full_newton) {
+        TcArgs a = {};
+        a.nt = nt; a.h = h; a.v = v; a.mT = m0; a.m_hist = c->m_hist; a.gm_hist = c->gm_hist; a.us = c->w0;
+        launch_transport_cluster(c, TC_STATE, a);
+        return;
+    }
+    if (sp_transport(c)) {
+        state_solve_sp(c, v, nt, m0);
+        return;
+    }
+    AdvStage<2> a = {};
+    a.D[0] = dbuf(c); a.v = v; a.h = h;
+    for (int j = 0; j < nt; ++j) {
+        a.uj = j > 0 ? mh(c, j) : m0;
+        d1_of(c, a.uj);
+        a.us = nullptr; a.u_out = c->w0; a.grad_out = gmh(c, j); a.stage = 1;
+        launch_row_adv(c, a);
+        d1_of(c, c->w0);
+        a.us = c->w0; a.u_out = mh(c, j + 1); a.grad_out = nullptr; a.stage = 2;
+        launch_row_adv(c, a);
+    }
+    d1_of(c, mh(c, nt));
+    a.uj = mh(c, nt); a.us = nullptr; a.u_out = nullptr; a.grad_out = gmh(c, nt); a.stage = 1;
+    launch_row_adv(c, a);
+}
+
+// Adjoint (Eq. (e:adj-eq-elim)) or Gauss-Newton incremental adjoint
+// (Eq. (e:inc-adj-eq-elim)) backward in time from lam_nt = ca*a + cb*cf, with
+// the body force b = int lam grad m dt (trapezoid) accumulated into bout.
+// lhist (nullable): store lam_j at lhist + j N for j = 0..nt (the full Newton matvec reads it).
+// vt (nullable): full Newton (Eq. (e:inc-adj-eq-elim) with the lambda term): the flux of every
+// divergence is lam~ v + lam v~ with lam from the gradient's adjoint history at the time the
+// divergence is evaluated, and b~ = sum_j w_j (lam~_j grad m_j + lam_j grad m~_j).
+static void adjoint_solve(reg_ctx* c, const float* v, int nt, const float* a, float ca, const float* cf, float cb,
+                          float* bout, float* lhist = nullptr, const float* vt = nullptr) {
+    const float h = 1.0f / (float)nt;
+    if (c->use_tc && !lhist && !vt) {
+        TcArgs t = {};
+        t.nt = nt; t.h = h; t.v = v; t.gm_hist = c->gm_hist; t.lj = c->w1; t.ls = c->w2;
+        t.adj_a = a; t.adj_ca = ca; t.adj_c = cf; t.adj_cb = cb; t.b = bout;
+        launch_transport_cluster(c, TC_ADJOINT, t);
+        return;
+    }
+    if (sp_transport(c)) {
+        if (vt) inc_adjoint_full_sp(c, v, vt, nt, bout);
+        else adjoint_solve_sp(c, v, nt, a, ca, cf, cb, bout, lhist);
+        return;
+    }
+    float* lst = c->w2;
+    auto lam_at = [&](int j) { return lhist ? lhist + (size_t)j * c->N : c->w1; };
+    launch_adj_init(c, a, ca, cf, cb, lam_at(nt), bout, gmh(c, nt), 0.5f * h, vt ? lamh(c, nt) : nullptr,
+                    vt ? gmth(c, nt) : nullptr);
+    AdjStage<2> s = {};
+    s.D[0] = dbuf(c); s.v = v; s.h = h; s.vt = vt;
+    for (int j = nt; j >= 1; --j) {
+        s.lsrc = vt ? lamh(c, j) : nullptr;
+        d1_of(c, lam_at(j), v, s.lsrc, vt);
+        s.lj = lam_at(j); s.ls = nullptr; s.l_out = lst; s.b = nullptr; s.stage = 1;
+        launch_row_adj(c, s);
+        s.lsrc = vt ? lamh(c, j - 1) : nullptr;
+        d1_of(c, lst, v, s.lsrc, vt);
+        s.ls = lst; s.l_out = lam_at(j - 1); s.stage = 2;
+        s.b = bout; s.gm = gmh(c, j - 1); s.gmt = vt ? gmth(c, j - 1) : nullptr;
+        s.w = (j - 1 == 0) ? 0.5f * h : h;
+        launch_row_adj(c, s);
+    }
+}
+
+// Incremental state (Eq. (e:inc-state-eq-elim)); leaves m~(1) in c->w3.
+// m~(0) = 0 is passed as u_j = nullptr to both stages of the first step.  gmt (nullable):
+// store grad m~_j at gmt + j 2N for j = 0..nt (the full Newton matvec reads it).
+static void inc_state_solve(reg_ctx* c, const float* v, const float* vt, int nt, float* gmt = nullptr) {
+    if (sp_transport(c)) {
+        inc_state_solve_sp(c, v, vt, nt, gmt);
+        return;
+    }
+    const float h = 1.0f / (float)nt;
+    float* mj = c->w3;
+    float* ms = c->w0;
+    AdvStage<2> a = {};
+    a.D[0] = dbuf(c); a.v = v; a.vt = vt; a.h = h;
+    for (int j = 0; j < nt; ++j) {
+        if (j > 0) d1_of(c, mj);
+        a.uj = (j > 0) ? mj : nullptr; a.us = nullptr; a.stage = 1;
+        a.src_in = j > 0 ? srcbuf(c) : nullptr; a.gm = gmh(c, j); a.src_out = nullptr;
+        a.u_out = ms; a.grad_out = gmt ? gmt + (size_t)j * 2 * c->N : nullptr;
+        // the first launch of the solve: v~ may come from the launch just before (Q^-1 s in
+        // preconditioned coordinates, or a caller's kernel), so it is read after the wait
+        a.zero = a.late = (j == 0) ? 1 : 0;
+        launch_row_adv(c, a);
+        a.zero = a.late = 0;
+        d1_of(c, ms);
+        a.us = ms; a.stage = 2;
+        a.src_in = nullptr; a.gm = gmh(c, j + 1); a.src_out = j + 1 < nt ? srcbuf(c) : nullptr;
+        a.u_out = mj; a.grad_out = nullptr;
+        launch_row_adv(c, a);
+    }
+    if (gmt) {
+        d1_of(c, mj);
+        a.uj = mj; a.us = nullptr; a.stage = 1; a.gm = nullptr; a.src_out = nullptr; a.u_out = nullptr;
+        a.grad_out = gmt + (size_t)nt * 2 * c->N;
+        launch_row_adv(c, a);
+    }
+}
+
+// Displacement (Eq. (e:displacement)): both components u_a of d_t u_a + grad u_a . v = v_a, u_a(0) = 0,
+// in one launch each (blockIdx.y); the source of component a is v_a itself
+static void displacement_solve(reg_ctx* c, const float* v, int nt, float* u, float* us, float* D) {
+    const long long N = c->N;
+    AdvStage<2> a = {};
+    a.D[0] = D; a.v = v; a.src_in = v; a.h = 1.0f / (float)nt; a.bs = (uint32_t)N;
+    for (int j = 0; j < nt; ++j) {
+        if (j > 0) launch_dcol(c, DColArgs{u, nullptr, nullptr, nullptr, D}, 2, N);
+        a.uj = j > 0 ? u : nullptr; a.us = nullptr; a.u_out = us; a.stage = 1;
+        a.zero = a.late = (j == 0) ? 1 : 0;
+        launch_row_adv(c, a, 2);
+        a.zero = a.late = 0;
+        launch_dcol(c, DColArgs{us, nullptr, nullptr, nullptr, D}, 2, N);
+        a.us = us; a.u_out = u; a.stage = 2;
+        launch_row_adv(c, a, 2);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -719,9 +894,9 @@ static int objective_dev(reg_ctx* c, const float* v, int nt, const float* y = nu
 }
 
 static void gradient_launches(reg_ctx* c, const float* v, float* g, int nt) {
-    adjoint_solve(c, v, nt, c->mR, 1.f, mh(c, nt), -1.f, c->bvec, nullptr, c->full_newton ? c->lam_hist : nullptr);
+    adjoint_solve(c, v, nt, c->mR, 1.f, mh(c, nt), -1.f, c->bvec, c->full_newton ? c->lam_hist : nullptr);
     if (c->shear_model) {
-        sp_grad_vec(c, v, c->gtmp);
+        sp_grad_vec_spec(c, v, c->gtmp);
         launch_shear_strain(c, c->gtmp, (float)c->nu, c->E_lin, c->eta_lin, c->T3, nullptr);
         // mean viscosity of the linearization point (App. A.2: eta = eta^ + eta_bar)
         const int np = launch_sum_partial(c, c->eta_lin, c->N, c->d_part);
@@ -730,18 +905,27 @@ static void gradient_launches(reg_ctx* c, const float* v, float* g, int nt) {
             sp_divt_proj(c, -(float)c->beta_v, c->T3, c->bvec, g);
         } else {
             cudaMemcpyAsync(c->T3b, c->E_lin, sizeof(float) * 3 * c->N, cudaMemcpyDeviceToDevice, c->stream);
-            shear_mass_assemble(c, c->T3, c->T3b, c->bvec, g);
+            shear_mass_assemble(c, c->T3, c->T3b, c->bvec, g ? g : c->vtmp2);
         }
     } else {
         sp_assemble(c, (float)c->beta_v, v, c->bvec, g);
     }
+}
+
+// the velocity becomes the context's linearization point first: the sequences read it from there
+static int set_lin(reg_ctx* c, const float* v) {
+    c->have_lin = false;
     if (v != c->v_lin)
-        cudaMemcpyAsync(c->v_lin, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        CK(cudaMemcpyAsync(c->v_lin, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
+    return REG_OK;
 }
 
 static int gradient_dev(reg_ctx* c, const float* v, float* g, int nt) {
-    RET(objective_dev(c, v, nt));
-    RET(run_seq(c, GK_GRADIENT, v, g, nt, [&] { gradient_launches(c, v, g, nt); }));
+    RET(set_lin(c, v));
+    RET(objective_dev(c, c->v_lin, nt));
+    float* out = g == c->g ? g : nullptr;  // reg_solve's own buffer, or finished outside the sequence
+    RET(run_seq(c, GK_GRADIENT, out, nullptr, nt, [&] { gradient_launches(c, c->v_lin, out, nt); }));
+    if (!out) RET(finish_out(c, g));
     c->nt_lin = nt;
     c->have_lin = true;
     return REG_OK;
@@ -749,12 +933,11 @@ static int gradient_dev(reg_ctx* c, const float* v, float* g, int nt) {
 
 // Gradient in preconditioned coordinates: g_y = Q^-1 g_v = Pi0 y + Q^-1 K b, at v = Q^-1 y
 static int gradient_dev_y(reg_ctx* c, const float* v, const float* y, float* gy, int nt) {
-    RET(objective_dev(c, v, nt, y));
-    RET(run_seq(c, GK_GRADIENT_Y, v, y, nt, [&] {  // gy is always c->g
-        adjoint_solve(c, v, nt, c->mR, 1.f, mh(c, nt), -1.f, c->bvec, nullptr, c->full_newton ? c->lam_hist : nullptr);
+    RET(set_lin(c, v));
+    RET(objective_dev(c, c->v_lin, nt, y));
+    RET(run_seq(c, GK_GRADIENT_Y, y, nullptr, nt, [&] {  // gy is always c->g
+        adjoint_solve(c, c->v_lin, nt, c->mR, 1.f, mh(c, nt), -1.f, c->bvec, c->full_newton ? c->lam_hist : nullptr);
         sp_assemble_y(c, y, c->bvec, gy);
-        if (v != c->v_lin)
-            cudaMemcpyAsync(c->v_lin, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
     }));
     c->nt_lin = nt;
     c->have_lin = true;
@@ -766,7 +949,7 @@ static int gradient_dev_y(reg_ctx* c, const float* v, const float* y, float* gy,
 static void inc_solves(reg_ctx* c, const float* vt, int nt) {
     if (c->full_newton) {
         inc_state_solve(c, c->v_lin, vt, nt, c->gmt_hist);
-        inc_adjoint_full(c, c->v_lin, vt, nt, c->bvec);
+        adjoint_solve(c, c->v_lin, nt, nullptr, 0.f, c->w3, -1.f, c->bvec, nullptr, vt);
         return;
     }
     if (c->use_tc) {
@@ -778,7 +961,7 @@ static void inc_solves(reg_ctx* c, const float* vt, int nt) {
         return;
     }
     inc_state_solve(c, c->v_lin, vt, nt);
-    adjoint_solve(c, c->v_lin, nt, nullptr, 0.f, c->w3, -1.f, c->bvec, nullptr);
+    adjoint_solve(c, c->v_lin, nt, nullptr, 0.f, c->w3, -1.f, c->bvec);
 }
 
 // Hessian product in preconditioned coordinates: H_y s = Q^-1 H_v Q^-1 s = Pi0 s + Q^-1 K b~(v~ = Q^-1 s)
@@ -793,13 +976,13 @@ static void matvec_launches(reg_ctx* c, const float* vt, float* Hvt) {
     const int nt = c->nt_lin;
     inc_solves(c, vt, nt);
     if (c->shear_model) {
-        sp_grad_vec(c, vt, c->gtmp);
+        sp_grad_vec_spec(c, vt, c->gtmp);
         launch_shear_second(c, c->gtmp, c->E_lin, c->eta_lin, (float)c->nu, c->T3);
         if (c->pmode == PROJ_LERAY) {
             sp_divt_proj(c, -(float)c->beta_v, c->T3, c->bvec, Hvt);
         } else {
             launch_shear_strain(c, c->gtmp, (float)c->nu, c->T3b, nullptr, nullptr, nullptr);  // E[v~]
-            shear_mass_assemble(c, c->T3, c->T3b, c->bvec, Hvt);
+            shear_mass_assemble(c, c->T3, c->T3b, c->bvec, Hvt ? Hvt : c->vtmp2);
         }
     } else {
         sp_assemble(c, (float)c->beta_v, vt, c->bvec, Hvt);
@@ -808,7 +991,9 @@ static void matvec_launches(reg_ctx* c, const float* vt, float* Hvt) {
 
 static int matvec_dev(reg_ctx* c, const float* vt, float* Hvt) {
     if (!c->have_lin) return reg_fail(REG_ERR_STATE, "reg_hessian_matvec called before reg_gradient");
-    return run_seq(c, GK_MATVEC, vt, Hvt, c->nt_lin, [&] { matvec_launches(c, vt, Hvt); });
+    CK(cudaMemcpyAsync(c->vtil, vt, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
+    RET(run_seq(c, GK_MATVEC, nullptr, nullptr, c->nt_lin, [&] { matvec_launches(c, c->vtil, nullptr); }));
+    return finish_out(c, Hvt);
 }
 
 static void precond_dev(reg_ctx* c, const float* r, float* z) {
@@ -840,7 +1025,7 @@ extern "C" int reg_apply_reg(reg_ctx* c, const float* v, float* out) {
     CTX_CHECK(c);
     RET(check_ptr(v, "v")); RET(check_ptr(out, "out"));
     if (c->shear_model) {
-        sp_grad_vec(c, v, c->gtmp);
+        sp_grad_vec_spec(c, v, c->gtmp);
         launch_shear_strain(c, c->gtmp, (float)c->nu, nullptr, nullptr, c->T3, nullptr);
         // beta_v A[v] = -beta_v div(2 eta E), without projection: use the divergence of each row of T
         const size_t N = c->N;
@@ -896,7 +1081,9 @@ extern "C" int reg_objective(reg_ctx* c, const float* v, float* m1, double* J) {
     CTX_CHECK(c);
     RET(check_ptr(v, "v"));
     if (m1) RET(check_ptr(m1, "m1"));
-    RET(objective_dev(c, v, c->nt));
+    if (v != c->vtrial)
+        CK(cudaMemcpyAsync(c->vtrial, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
+    RET(objective_dev(c, c->vtrial, c->nt));
     c->have_lin = false;  // history now belongs to this v, but grad/adjoint data do not
     if (m1) CK(cudaMemcpyAsync(m1, mh(c, c->nt), sizeof(float) * c->N, cudaMemcpyDeviceToDevice, c->stream));
     if (J) {
@@ -1215,16 +1402,10 @@ extern "C" int reg_displacement(reg_ctx* c, const float* v, float* u_out) {
     RET(check_ptr(v, "v")); RET(check_ptr(u_out, "u_out"));
     const int nt = c->nt;
     const size_t N = c->N;
-    // Component a solves d_t u_a + grad u_a . v = v_a from u_a = 0: the incremental-state
-    // stage with source -(e . grad) where grad := v at every time and e = -(unit vector a),
-    // so that the source is exactly v_a in FP32.
-    float* e = c->vtmp;
-    for (int comp = 0; comp < 2; ++comp) {
-        launch_fill(c, 2 * (long long)N, e, 0.f);
-        launch_fill(c, N, e + comp * N, -1.f);
-        inc_state_solve(c, v, e, nt, nullptr, v);
-        CK(cudaMemcpyAsync(u_out + comp * N, c->w3, sizeof(float) * N, cudaMemcpyDeviceToDevice, c->stream));
-    }
+    CK(cudaMemcpyAsync(c->vtil, v, sizeof(float) * 2 * N, cudaMemcpyDeviceToDevice, c->stream));
+    RET(run_seq(c, GK_DISPLACEMENT, nullptr, nullptr, nt,
+                [&] { displacement_solve(c, c->vtil, nt, c->vtmp, c->vx, c->gtmp); }));
+    CK(cudaMemcpyAsync(u_out, c->vtmp, sizeof(float) * 2 * N, cudaMemcpyDeviceToDevice, c->stream));
     CKL();
     return REG_OK;
 }
@@ -1246,8 +1427,10 @@ extern "C" int reg_label_overlap(reg_ctx* c, const float* v, const float* labels
     float2* o[1] = {c->S[1]};
     launch_col(c, OP_SMOOTH, in, o, spec_params(c, a), nullptr);
     launch_c2r_scalar(c, c->S[1], sm);
-    state_solve(c, v, nt, sm);  // overwrites the state history
+    CK(cudaMemcpyAsync(c->vtil, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
     c->have_lin = false;
+    // overwrites the state history
+    RET(run_seq(c, GK_LABELS, nullptr, nullptr, nt, [&] { state_solve(c, c->vtil, nt, sm); }));
     if (transported)
         CK(cudaMemcpyAsync(transported, mh(c, nt), sizeof(float) * c->N, cudaMemcpyDeviceToDevice, c->stream));
     const int np = launch_overlap_counts(c, mh(c, nt), labels_R, 0.5f, c->d_part);
@@ -1266,28 +1449,26 @@ extern "C" int reg_label_overlap(reg_ctx* c, const float* v, const float* labels
 // ---------------------------------------------------------------------------
 // deformation gradient (Eq. (e:def-grad)) and its measures (Appendix F)
 // ---------------------------------------------------------------------------
-static void detgrad_launches(reg_ctx* c, const float* v, float* detF, int nt) {
+// F1 of the flow of v into c->F (nt even) or c->gF (nt odd); the x^1 derivatives of all four planes are one launch
+static void detgrad_launches(reg_ctx* c, const float* v, int nt) {
     const size_t N = c->N;
-    const float h = 1.0f / (float)nt;
     sp_grad_vec(c, v, c->gv);
-    float* Fa = c->F;     // F_j
-    float* Fb = c->gtmp;  // F_{j+1} (ping-pong)
+    float* Fa = c->F;      // F_j
+    float* Fb = c->gF;     // F_{j+1} (ping-pong)
+    DefGradStage a = {};
+    a.D = c->gF + 4 * N; a.v = v; a.gv = c->gv; a.h = 1.0f / (float)nt;
     launch_fill(c, 4 * (long long)N, Fa, 0.f);  // F(0) = I
     launch_fill(c, N, Fa, 1.f);
     launch_fill(c, N, Fa + 3 * N, 1.f);
     for (int j = 0; j < nt; ++j) {
-        for (int comp = 0; comp < 4; ++comp) sp_grad(c, Fa + comp * N, c->gF + 2 * comp * N);
-        launch_defgrad_stage(c, 1, Fa, nullptr, c->gF, c->gv, v, h, c->Fs);
-        for (int comp = 0; comp < 4; ++comp) sp_grad(c, c->Fs + comp * N, c->gF + 2 * comp * N);
-        launch_defgrad_stage(c, 2, Fa, c->Fs, c->gF, c->gv, v, h, Fb);
+        launch_dcol(c, DColArgs{Fa, nullptr, nullptr, nullptr, c->gF + 4 * N}, 4, N);
+        a.F = Fa; a.Fs = nullptr; a.out = c->Fs; a.stage = 1;
+        launch_defgrad_stage(c, a);
+        launch_dcol(c, DColArgs{c->Fs, nullptr, nullptr, nullptr, c->gF + 4 * N}, 4, N);
+        a.Fs = c->Fs; a.out = Fb; a.stage = 2;
+        launch_defgrad_stage(c, a);
         float* t = Fa; Fa = Fb; Fb = t;
     }
-    const int np = launch_det_stats(c, Fa, detF, c->d_part);
-    launch_finalize(c, c->d_part + 0 * np, np, c->d_scal + SL_DET0 + 0, 1.0, 0, 2);
-    launch_finalize(c, c->d_part + 1 * np, np, c->d_scal + SL_DET0 + 1, 1.0 / (double)N, 0, 0);
-    launch_finalize(c, c->d_part + 2 * np, np, c->d_scal + SL_DET0 + 2, 1.0, 0, 1);
-    launch_finalize(c, c->d_part + 3 * np, np, c->d_scal + SL_DET0 + 3, 1.0, 0, 1);
-    launch_finalize(c, c->d_part + 4 * np, np, c->d_scal + SL_DET0 + 4, 1.0 / (double)N, 0, 0);
 }
 
 extern "C" int reg_detgrad(reg_ctx* c, const float* v, float* detF, double* stats) {
@@ -1295,7 +1476,10 @@ extern "C" int reg_detgrad(reg_ctx* c, const float* v, float* detF, double* stat
     RET(check_ptr(v, "v"));
     if (detF) RET(check_ptr(detF, "detF"));
     const int nt = c->nt;
-    RET(run_seq(c, GK_DETGRAD, v, detF, nt, [&] { detgrad_launches(c, v, detF, nt); }));
+    CK(cudaMemcpyAsync(c->vtil, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
+    RET(run_seq(c, GK_DETGRAD, nullptr, nullptr, nt, [&] { detgrad_launches(c, c->vtil, nt); }));
+    launch_det_stats(c, (nt & 1) ? c->gF : c->F, detF, c->d_part, c->d_scal + SL_DET0);
+    CKL();
     if (stats) {
         RET(read_scalars(c));
         for (int q = 0; q < 5; ++q) stats[q] = c->h_scal[SL_DET0 + q];

@@ -78,6 +78,7 @@ struct reg_ctx {
     int pmode;
     bool shear_model;
     cudaStream_t stream;
+    cudaStream_t cap;  // launch sequences are captured here when `stream` is the legacy default stream
 
     // images and history
     float *mT, *mR;
@@ -103,7 +104,7 @@ struct reg_ctx {
     float *ybuf, *ytrial, *vtil;
     bool ypath;      // reg_solve iterates on y (quadratic H2 regularization, see reg_solve)
     // det F workspace
-    float *F, *Fs, *gF, *gv;  // 4N, 4N, 8N, 4N
+    float *F, *Fs, *gF, *gv;  // 4N, 4N, 8N (F of the next step, D), 4N
 
     double* d_scal;  // SL_COUNT
     double* d_part;  // partial sums
@@ -152,12 +153,32 @@ size_t row_smem(int R, int L);
 size_t col_smem(int C, int L, bool div1);
 
 void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S);
-void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, float2* S2);
+// nb vector fields back to back (2 N floats each; spectra S1, S2: N entries apart from field to field)
+void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, float2* S2, int nb = 1);
 void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f);
-void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2);
+void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb = 1,
+                    float scale = 1.f);
+// nb > 1 (OP_SMOOTH_PROJ only): fields N entries apart
 void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* out, const SpecParams& P,
-                double* part_out);
+                double* part_out, int nb = 1);
 
+// transport stages (deriv.cuh)
+struct DColArgs;
+template <int DIM> struct AdvStage;
+template <int DIM> struct AdjStage;
+void launch_dcol(reg_ctx* ctx, const DColArgs& a, int nb = 1, long long bs = 0);
+void launch_row_adv(reg_ctx* ctx, const AdvStage<2>& a, int nb = 1);
+void launch_row_adj(reg_ctx* ctx, const AdjStage<2>& a);
+struct DefGradStage;
+void launch_defgrad_stage(reg_ctx* ctx, const DefGradStage& a);
+// out (2 planes) = grad f; out += d_2 f
+void launch_grad(reg_ctx* ctx, const float* f, float* out);
+void launch_add_d2(reg_ctx* ctx, const float* f, float* out);
+// lam = ca * a + cb * c (a nullable); b = w lam gm (+ w lsrc gmt, full Newton)
+void launch_adj_init(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, float* lam, float* b,
+                     const float* gm, float w, const float* lsrc = nullptr, const float* gmt = nullptr);
+
+// RK2 stages in the row spectra (kernels.cu)
 struct AdvArgs {
     const float2 *G1, *G2;  // spectra of d1 u_s, d2 u_s; G1 == nullptr -> zero gradient
     const float2* Sd2;      // G2 == nullptr: row spectrum of u_s, d2 u_s = (i k2~ / n2) Sd2
@@ -196,7 +217,7 @@ void launch_row_adj(reg_ctx* ctx, const AdjArgs& a);
 // lam = ca * a + cb * c (a nullable); b = w lam gm; flux spectra of lam v;
 // optional FP64 partials of 0.5 * sum(lam^2) * h1 h2.  Full Newton (lsrc != nullptr):
 // b += w lsrc gmt and the flux is lam v + lsrc vt.
-void launch_adj_init(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, const float* v,
+void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, const float* v,
                      float* lam, float* b, const float* gm, float w, float2* F1, float2* F2, double* part,
                      const float* lsrc = nullptr, const float* vt = nullptr, const float* gmt = nullptr);
 
@@ -222,10 +243,8 @@ void launch_fill(reg_ctx* ctx, long long n, float* y, float val);
 // (f > thr), (L > 0.5) and both; returns nb
 int launch_overlap_counts(reg_ctx* ctx, const float* f, const float* L, float thr, double* part);
 
-// deformation gradient
-void launch_defgrad_stage(reg_ctx* ctx, int stage, const float* F, const float* Fs, const float* gF,
-                          const float* gv, const float* v, float h, float* out);
-int launch_det_stats(reg_ctx* ctx, const float* F, float* detF, double* part);
+// det F1 (nullable output) and its five statistics into out (min, mean, max det, max D, mean D)
+void launch_det_stats(reg_ctx* ctx, const float* F, float* detF, double* part, double* out);
 
 // shear model
 // from grad v (gv: d1v1, d2v1, d1v2, d2v2) compute E (3 planes) and eta; and

@@ -14,45 +14,13 @@
 // deformation gradient (Eq. (e:def-grad)); FP64 accumulation for all sums.
 #include <cmath>
 #include <cstdio>
-#include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include "fft.cuh"
 #include "fft_reg.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
-#define NTHREADS 256
-#define NBLK_RED 304  // 2 x 152 SMs
-
-// Programmatic dependent launch: every kernel waits for the grid it depends
-// on (it has completed and its writes are visible after the wait) and then
-// lets the next kernel in the stream begin launching, so the launch, CTA
-// scheduling and prologue of kernel k+1 overlap the tail of kernel k.  Since
-// each kernel triggers only after its own wait, a kernel that starts early
-// may read, before its wait, anything written two or more launches back
-// (the RK2 row-stage kernels prefetch their pointwise operands that way).
-// Without a programmatic dependency both instructions are no-ops.
-__device__ __forceinline__ void pdl_entry() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-// Launch with the programmatic-stream-serialization attribute (ctx->pdl) or plainly.
-template <typename... KArgs, typename... Args>
-static void launch_k(reg_ctx* ctx, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = ctx->pdl ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
 
 // ---------------------------------------------------------------------------
 // timing hooks
@@ -186,10 +154,21 @@ __device__ __forceinline__ void stage_chunk(float2* dst, const float2* __restric
     for (int i = threadIdx.x; i < n / 2; i += blockDim.x) d4[i] = s4[i];
 }
 
+// blockIdx.y: independent fields, f floats and s spectrum entries apart
+struct Batch {
+    long long f, s;
+};
+
 template <int LOGL, bool VEC>
 __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const float* __restrict__ f2,
-                                             float2* S1, float2* S2, int R, const float2* __restrict__ tw) {
+                                             float2* S1, float2* S2, int R, const float2* __restrict__ tw, Batch bt) {
     pdl_entry();
+    f1 += blockIdx.y * bt.f;
+    S1 += blockIdx.y * bt.s;
+    if (VEC) {
+        f2 += blockIdx.y * bt.f;
+        S2 += blockIdx.y * bt.s;
+    }
     extern __shared__ __align__(16) float2 sm[];
     constexpr int L = 1 << LOGL, T = L >> 3, W = L >> 1;
     float2* A = sm;
@@ -234,8 +213,14 @@ __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const
 template <int LOGL, bool VEC>
 __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, const float2* __restrict__ S2,
                                              float* __restrict__ f1, float* __restrict__ f2, int R,
-                                             const float2* __restrict__ tw) {
+                                             const float2* __restrict__ tw, Batch bt, float scale) {
     pdl_entry();
+    f1 += blockIdx.y * bt.f;
+    S1 += blockIdx.y * bt.s;
+    if (VEC) {
+        f2 += blockIdx.y * bt.f;
+        S2 += blockIdx.y * bt.s;
+    }
     extern __shared__ __align__(16) float2 sm[];
     constexpr int L = 1 << LOGL, T = L >> 3, W = L >> 1;
     float2* A = sm;
@@ -262,17 +247,24 @@ __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, cons
             const int j = t + k * T;
             if (VEC) {
                 const size_t idx = (size_t)(row0 + q) * L + j;
-                f1[idx] = x[k].x;
-                f2[idx] = x[k].y;
+                f1[idx] = scale * x[k].x;
+                f2[idx] = scale * x[k].y;
             } else {
                 const size_t idx = (size_t)(row0 + 2 * q) * L + j;
-                f1[idx] = x[k].x;
-                f1[idx + L] = x[k].y;
+                f1[idx] = scale * x[k].x;
+                f1[idx + L] = scale * x[k].y;
             }
         }
     }
 }
 
+// ---------------------------------------------------------------------------
+// RK2 stages in the row spectra: the transport of the H2 and H3 solves (api.cu, sp_transport).
+// transport.cu's axis-wise stages do the same step in less time with other roundings; those solves
+// amplify a change of rounding by 10^3 to 10^5 (the velocities of two 128^2 H2 solves, beta_v =
+// 1e-3, stopped after the same two Newton steps, differ by 1e-5 to 1e-1 when the last bits of b~
+// do), so they keep the arithmetic that their users' results came from.
+// ---------------------------------------------------------------------------
 // ---------------------------------------------------------------------------
 // RK2 (Heun) advection stage of the state and incremental state equations
 // (Eq. (e:state-eq-elim), (e:inc-state-eq-elim)):
@@ -282,7 +274,7 @@ __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, cons
 // result u_out leaves as its packed spectrum S_out for the next column pass.
 // ---------------------------------------------------------------------------
 template <int LOGL, bool PRE>
-__global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adv(AdvArgs a, int N, int R,
+__global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adv_sp(AdvArgs a, int N, int R,
                                                                            const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
     constexpr int L = 1 << LOGL, T = L >> 3, W = L >> 1;
@@ -409,7 +401,7 @@ __device__ __forceinline__ void flux_fft_store(float2 (&x)[8], int q, int t, int
 // is evaluated) and stage 2 adds w lam_src grad m~ to the body force.  Compiled only without
 // prefetch, with a smaller load batch (more operands per element).
 template <int LOGL, bool PRE, bool FULL>
-__global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adj(AdjArgs a, int N, int R,
+__global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adj_sp(AdjArgs a, int N, int R,
                                                                            const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
     constexpr int L = 1 << LOGL, T = L >> 3, W = L >> 1;
@@ -421,7 +413,7 @@ __global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adj(AdjArgs 
     const size_t rowbase = (size_t)(row0 + q) * L;
     // Operands written at least two launches earlier (lam_j, lam*, v, b, grad m)
     // are loaded before waiting on the preceding column kernel, which writes D
-    // (after the FFT with PRE = false, as in k_row_adv).
+    // (after the FFT with PRE = false, as in k_row_adv_sp).
     float plj[8], pls[8], pv1[8], pv2[8], pb1[8], pb2[8], pg1[8], pg2[8];
     float psrc[8], pt1[8], pt2[8], ph1[8], ph2[8];
     auto load_ops = [&](int k) {
@@ -473,7 +465,7 @@ __global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adj(AdjArgs 
     for (int k0 = 0; k0 < 8; k0 += BATCH) {
         if (!PRE || FULL) {
 #pragma unroll
-            for (int k = k0; k < k0 + BATCH; ++k) load_ops(k);  // batched, as in k_row_adv
+            for (int k = k0; k < k0 + BATCH; ++k) load_ops(k);  // batched, as in k_row_adv_sp
         }
 #pragma unroll
         for (int k = k0; k < k0 + BATCH; ++k) {
@@ -504,7 +496,7 @@ __global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adj(AdjArgs 
 // lam = ca*a + cb*c; b = w lam gm; flux spectra; partial 0.5*sum(lam^2).  With lsrc (full
 // Newton): b += w lsrc gmt and the flux is lam v + lsrc v~.
 template <int LOGL>
-__global__ void __launch_bounds__(512) k_adj_init(const float* __restrict__ a, float ca, const float* __restrict__ c,
+__global__ void __launch_bounds__(512) k_adj_init_sp(const float* __restrict__ a, float ca, const float* __restrict__ c,
                                                   float cb, const float* __restrict__ v, float* lam, float* b,
                                                   const float* __restrict__ gm, float w, float2* F1, float2* F2,
                                                   double* part, int N, int R, const float2* __restrict__ tw,
@@ -554,6 +546,7 @@ __global__ void __launch_bounds__(512) k_adj_init(const float* __restrict__ a, f
 // the partner entry at -k1 before the multiplier is applied.
 // ---------------------------------------------------------------------------
 struct ColArgs {
+    long long bs;   // blockIdx.y: stride of independent fields (0: one field)
     const float2* in[5];
     float2* out[2];
     SpecParams P;
@@ -704,7 +697,7 @@ __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict
     float2 xin[NIN][8];
 #pragma unroll
     for (int f = 0; f < NIN; ++f) {
-        const float2* src = a.in[f];
+        const float2* src = a.in[f] + blockIdx.y * a.bs;
         for (int idx = threadIdx.x; idx < C * L; idx += blockDim.x) {
             const int g = idx >> g_shift;
             const int rem = idx & g_mask;
@@ -773,7 +766,7 @@ __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict
 #pragma unroll
         for (int k = 0; k < 8; ++k) A[c * L + t + k * T] = y[o][k];
         __syncthreads();
-        float2* dst = a.out[o];
+        float2* dst = a.out[o] + blockIdx.y * a.bs;
         const float cd2 = 1.0f / (float)a.n2;
         for (int idx = threadIdx.x; idx < C * L; idx += blockDim.x) {
             const int g = idx >> g_shift;
@@ -796,14 +789,16 @@ __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict
 // launch helpers
 // ---------------------------------------------------------------------------
 // Default tile choices.  R rows per row CTA: a multiple of 4 with at least 64
-// threads (T = L/8 per row); C spectrum columns per column CTA: at least 2
-// (64-byte segments) and 64 threads.  reg_autotune may replace both per grid.
+// transform entries in flight per 8 (T = L/8 per row); C columns per column CTA: at least 4 where
+// that fits 256 threads (32-byte sectors of the transport's fields; 512^2 matvec, nt = 16: 364 us
+// against 395 us with 2, 256^2: 281 against 285) and 64 threads.  reg_autotune may replace both per
+// grid.
 void default_tiles(int n1, int n2, int* R_out, int* C_out, int* P_out) {
     if (P_out) *P_out = n2 <= 512 ? 1 : 0;
     int R = 4;
     while (R * (n2 / 8) < 64 && R * 2 <= n1) R *= 2;
     const int W = n2 / 2;
-    int C = 2;
+    int C = n1 <= 512 ? 4 : 2;
     while (C * (n1 / 8) < 64 && C * 2 <= W) C *= 2;
     *R_out = R;
     *C_out = C > W ? W : C;
@@ -831,62 +826,6 @@ bool tiles_valid(int n1, int n2, int R, int C, int P) {
     return true;
 }
 
-static int rows_per_cta(const reg_ctx* ctx) {
-    int R, C, P;
-    default_tiles(ctx->n1, ctx->n2, &R, &C, &P);
-    return ctx->tileR > 0 ? ctx->tileR : R;
-}
-
-static int cols_per_cta(const reg_ctx* ctx) {
-    int R, C, P;
-    default_tiles(ctx->n1, ctx->n2, &R, &C, &P);
-    return ctx->tileC > 0 ? ctx->tileC : C;
-}
-
-static bool prefetch_rows(const reg_ctx* ctx) {
-    int R, C, P;
-    default_tiles(ctx->n1, ctx->n2, &R, &C, &P);
-    return (ctx->tileR > 0 ? ctx->tileP : P) != 0;
-}
-
-// Opt in to more than 48 KB of dynamic shared memory once per (device, kernel instantiation)
-// and size: the attribute applies to the current device only (contexts on several host
-// threads launch concurrently, hence the lock).
-struct SmemKey {
-    int dev;
-    const void* kern;
-    bool operator==(const SmemKey& o) const { return dev == o.dev && kern == o.kern; }
-};
-struct SmemKeyHash {
-    size_t operator()(const SmemKey& k) const { return std::hash<const void*>()(k.kern) * 31u + (size_t)k.dev; }
-};
-template <typename K>
-static void set_smem(K kern, size_t bytes) {
-    if (bytes <= 32 * 1024) return;  // static shared memory (reductions) also counts toward the 48 KB default
-    static std::mutex mu;
-    static std::unordered_map<SmemKey, size_t, SmemKeyHash> done;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const SmemKey key{dev, (const void*)kern};
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = done.find(key);
-    if (it != done.end() && it->second >= bytes) return;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    done[key] = bytes;
-}
-
-#define DISPATCH_LOG(LOG, ...)                        \
-    switch (LOG) {                                    \
-        case 4: { constexpr int LG = 4; __VA_ARGS__; } break;   \
-        case 5: { constexpr int LG = 5; __VA_ARGS__; } break;   \
-        case 6: { constexpr int LG = 6; __VA_ARGS__; } break;   \
-        case 7: { constexpr int LG = 7; __VA_ARGS__; } break;   \
-        case 8: { constexpr int LG = 8; __VA_ARGS__; } break;   \
-        case 9: { constexpr int LG = 9; __VA_ARGS__; } break;   \
-        case 10: { constexpr int LG = 10; __VA_ARGS__; } break; \
-        default: break;                               \
-    }
-
 struct RowCfg { int R, threads; size_t smem; int grid; bool pre; };
 static RowCfg row_cfg(reg_ctx* ctx) {
     RowCfg c;
@@ -905,18 +844,19 @@ void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S) {
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_r2c<LG, false>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw);
+        launch_k(ctx, kern, g.grid, g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw, Batch{0, 0});
     });
     ktimer_end(ctx);
 }
 
-void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, float2* S2) {
+void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, float2* S2, int nb) {
     const RowCfg g = row_cfg(ctx);
-    ktimer_begin(ctx, KC_ROW, 16.0 * ctx->N);
+    ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_r2c<LG, true>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, u1, u2, S1, S2, g.R, ctx->tw);
+        launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, u1, u2, S1, S2, g.R, ctx->tw,
+                 Batch{2LL * ctx->N, (long long)ctx->N});
     });
     ktimer_end(ctx);
 }
@@ -927,18 +867,19 @@ void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f) {
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_c2r<LG, false>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, S, nullptr, f, nullptr, g.R, ctx->tw);
+        launch_k(ctx, kern, g.grid, g.threads, g.smem, S, nullptr, f, nullptr, g.R, ctx->tw, Batch{0, 0}, 1.f);
     });
     ktimer_end(ctx);
 }
 
-void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2) {
+void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb, float scale) {
     const RowCfg g = row_cfg(ctx);
-    ktimer_begin(ctx, KC_ROW, 16.0 * ctx->N);
+    ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_c2r<LG, true>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, S1, S2, u1, u2, g.R, ctx->tw);
+        launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, S1, S2, u1, u2, g.R, ctx->tw,
+                 Batch{2LL * ctx->N, (long long)ctx->N}, scale);
     });
     ktimer_end(ctx);
 }
@@ -951,7 +892,7 @@ void launch_row_adv(reg_ctx* ctx, const AdvArgs& a) {
                 (a.S_out ? 1 : 0);
     ktimer_begin(ctx, KC_ROWSTAGE, 4.0 * fl * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = (g.pre && LG <= 9) ? k_row_adv<LG, (LG <= 9)> : k_row_adv<LG, false>;
+        auto kern = (g.pre && LG <= 9) ? k_row_adv_sp<LG, (LG <= 9)> : k_row_adv_sp<LG, false>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, g.grid, g.threads, g.smem, a, ctx->N, g.R, ctx->tw);
     });
@@ -966,22 +907,22 @@ void launch_row_adj(reg_ctx* ctx, const AdjArgs& a) {
                 (a.lsrc ? 3 + (a.b ? 2 : 0) : 0);
     ktimer_begin(ctx, KC_ROWSTAGE, 4.0 * fl * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = a.lsrc ? k_row_adj<LG, false, true>
-                           : ((g.pre && LG <= 9) ? k_row_adj<LG, (LG <= 9), false> : k_row_adj<LG, false, false>);
+        auto kern = a.lsrc ? k_row_adj_sp<LG, false, true>
+                           : ((g.pre && LG <= 9) ? k_row_adj_sp<LG, (LG <= 9), false> : k_row_adj_sp<LG, false, false>);
         set_smem(kern, g.smem);
         launch_k(ctx, kern, g.grid, g.threads, g.smem, a, ctx->N, g.R, ctx->tw);
     });
     ktimer_end(ctx);
 }
 
-void launch_adj_init(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, const float* v, float* lam,
+void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, const float* v, float* lam,
                      float* b, const float* gm, float w, float2* F1, float2* F2, double* part, const float* lsrc,
                      const float* vt, const float* gmt) {
     const RowCfg g = row_cfg(ctx);
     // a 1 (optional), c 1, v 2, lam 1, b 2 + gm 2, flux spectra 2; full Newton: lsrc 1, v~ 2, grad m~ 2
     ktimer_begin(ctx, KC_ROW, 4.0 * ((a ? 1 : 0) + 1 + 2 + 1 + 4 + 2 + (lsrc ? 5 : 0)) * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = k_adj_init<LG>;
+        auto kern = k_adj_init_sp<LG>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, g.grid, g.threads, g.smem, a, ca, c, cb, v, lam, b, gm, w, F1, F2, part, ctx->N, g.R,
                  ctx->tw, lsrc, vt, gmt);
@@ -989,15 +930,14 @@ void launch_adj_init(reg_ctx* ctx, const float* a, float ca, const float* c, flo
     ktimer_end(ctx);
 }
 
-int row_blocks(reg_ctx* ctx) { return row_cfg(ctx).grid; }
-
 template <int NIN, int NOUT, int OP>
 static void launch_col_t(reg_ctx* ctx, const float2* const* in, float2* const* out, const SpecParams& P,
-                         double* part) {
+                         double* part, int nb = 1) {
     const int L = ctx->n1, W = ctx->n2 / 2;
-    const int cpb = cols_per_cta(ctx);
+    const int cpb = spec_cols_per_cta(ctx);
     const size_t smem = col_smem(cpb, L, OP == OP_DIV1);
     ColArgs a;
+    a.bs = nb > 1 ? ctx->N : 0;
     for (int f = 0; f < 5; ++f) a.in[f] = (f < NIN) ? in[f] : nullptr;
     if (OP == OP_DIV1) a.in[1] = in[1];  // read untransformed in the store phase
     for (int o = 0; o < 2; ++o) a.out[o] = (o < NOUT) ? out[o] : nullptr;
@@ -1007,19 +947,19 @@ static void launch_col_t(reg_ctx* ctx, const float2* const* in, float2* const* o
     a.lcpb = 0;
     while ((1 << a.lcpb) < cpb) ++a.lcpb;
     a.n2 = ctx->n2;
-    ktimer_begin(ctx, KC_COL, 4.0 * (NIN + NOUT + (OP == OP_DIV1 ? 1 : 0)) * ctx->N);
+    ktimer_begin(ctx, KC_COL, 4.0 * nb * (NIN + NOUT + (OP == OP_DIV1 ? 1 : 0)) * ctx->N);
     DISPATCH_LOG(ctx->log1, {
         auto kern = k_col<LG, NIN, NOUT, OP>;
         set_smem(kern, smem);
-        launch_k(ctx, kern, W / cpb, cpb * (L / 8), smem, a, ctx->tw);
+        launch_k(ctx, kern, dim3(W / cpb, nb), cpb * (L / 8), smem, a, ctx->tw);
     });
     ktimer_end(ctx);
 }
 
-int col_blocks(reg_ctx* ctx) { return (ctx->n2 / 2) / cols_per_cta(ctx); }
+int col_blocks(reg_ctx* ctx) { return (ctx->n2 / 2) / spec_cols_per_cta(ctx); }
 
 void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* out, const SpecParams& P,
-                double* part) {
+                double* part, int nb) {
     switch (op) {
         case OP_GRAD: launch_col_t<1, 2, OP_GRAD>(ctx, in, out, P, part); break;
         case OP_DIV: launch_col_t<2, 1, OP_DIV>(ctx, in, out, P, part); break;
@@ -1031,7 +971,7 @@ void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* ou
         case OP_DIVT_PROJ: launch_col_t<5, 2, OP_DIVT_PROJ>(ctx, in, out, P, part); break;
         case OP_GRAD1: launch_col_t<1, 1, OP_GRAD1>(ctx, in, out, P, part); break;
         case OP_DIV1: launch_col_t<1, 1, OP_DIV1>(ctx, in, out, P, part); break;
-        case OP_SMOOTH_PROJ: launch_col_t<2, 2, OP_SMOOTH_PROJ>(ctx, in, out, P, part); break;
+        case OP_SMOOTH_PROJ: launch_col_t<2, 2, OP_SMOOTH_PROJ>(ctx, in, out, P, part, nb); break;
         case OP_SMOOTH: launch_col_t<1, 1, OP_SMOOTH>(ctx, in, out, P, part); break;
         case OP_MASSP: launch_col_t<2, 2, OP_MASSP>(ctx, in, out, P, part); break;
         case OP_QINV: launch_col_t<2, 2, OP_QINV>(ctx, in, out, P, part); break;
@@ -1211,40 +1151,6 @@ int launch_overlap_counts(reg_ctx* ctx, const float* f, const float* L, float th
     return NBLK_RED;
 }
 
-// deformation gradient stage (Eq. (e:def-grad)); F planes (F11, F12, F21, F22),
-// gF planes (d1 F11, d2 F11, d1 F12, d2 F12, ...), gv planes (d1 v1, d2 v1, d1 v2, d2 v2)
-__global__ void k_defgrad_stage(int N, int stage, const float* __restrict__ F, const float* __restrict__ Fs,
-                                const float* __restrict__ gF, const float* __restrict__ gv,
-                                const float* __restrict__ v, float h, float* out) {
-    pdl_entry();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        const float* Fin = (stage == 1) ? F : Fs;
-        float Fv[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) Fv[c] = Fin[(size_t)c * N + i];
-        const float v1 = v[i], v2 = v[N + i];
-        const float g[4] = {gv[i], gv[(size_t)N + i], gv[2 * (size_t)N + i], gv[3 * (size_t)N + i]};
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const int c = 2 * a + b;
-                float rhs = -(v1 * gF[(size_t)(2 * c) * N + i] + v2 * gF[(size_t)(2 * c + 1) * N + i]);
-                rhs += g[2 * a] * Fv[b] + g[2 * a + 1] * Fv[2 + b];
-                const float f0 = F[(size_t)c * N + i];
-                out[(size_t)c * N + i] = (stage == 1) ? fmaf(h, rhs, f0) : 0.5f * (f0 + Fs[(size_t)c * N + i] + h * rhs);
-            }
-        }
-    }
-}
-
-void launch_defgrad_stage(reg_ctx* ctx, int stage, const float* F, const float* Fs, const float* gF, const float* gv,
-                          const float* v, float h, float* out) {
-    ktimer_begin(ctx, KC_POINT, 4.0 * (4 + (stage == 2 ? 4 : 0) + 8 + 4 + 2 + 4) * ctx->N);
-    launch_k(ctx, k_defgrad_stage, NBLK_RED, NTHREADS, 0, ctx->N, stage, F, Fs, gF, gv, v, h, out);
-    ktimer_end(ctx);
-}
-
 __global__ void k_det_stats(int N, const float* __restrict__ F, float* detF, double* part) {
     pdl_entry();
     double mn = 1e300, mx = -1e300, sm = 0.0, dmx = 0.0, dsm = 0.0;
@@ -1272,11 +1178,25 @@ __global__ void k_det_stats(int N, const float* __restrict__ F, float* detF, dou
     if (threadIdx.x == 0) part[4 * gridDim.x + blockIdx.x] = r;
 }
 
-int launch_det_stats(reg_ctx* ctx, const float* F, float* detF, double* part) {
+// the five statistics from their partials: block q reduces quantity q
+__global__ void k_det_final(const double* __restrict__ part, int np, double* out, double invN) {
+    pdl_entry();
+    const double* p = part + blockIdx.x * np;
+    const int q = blockIdx.x;
+    double acc = (q == 1 || q == 4) ? 0.0 : p[0];
+    for (int i = threadIdx.x; i < np; i += blockDim.x)
+        acc = q == 0 ? red_op<2>(acc, p[i]) : ((q == 1 || q == 4) ? acc + p[i] : red_op<1>(acc, p[i]));
+    const double s = q == 0 ? block_reduce<2>(acc) : ((q == 1 || q == 4) ? block_reduce<0>(acc) : block_reduce<1>(acc));
+    if (threadIdx.x == 0) out[q] = (q == 1 || q == 4) ? s * invN : s;
+}
+
+void launch_det_stats(reg_ctx* ctx, const float* F, float* detF, double* part, double* out) {
     ktimer_begin(ctx, KC_POINT, 4.0 * (4 + (detF ? 1 : 0)) * ctx->N);
     launch_k(ctx, k_det_stats, NBLK_RED, NTHREADS, 0, ctx->N, F, detF, part);
     ktimer_end(ctx);
-    return NBLK_RED;
+    ktimer_begin(ctx, KC_POINT, 8.0 * 5 * NBLK_RED);
+    launch_k(ctx, k_det_final, 5, NTHREADS, 0, part, NBLK_RED, out, 1.0 / (double)ctx->N);
+    ktimer_end(ctx);
 }
 
 // shear control: strain rate, viscosity, stress (Eqs. (e:shear-control-reg-v), (e:1st-var-reg-v-nls))

@@ -63,27 +63,27 @@ struct Dims3 {
 struct D12Args {
     DColArgs a1, a2;
     ColMap m1, m2;
-    int log1, log2, lc1, lc2, tiles1;
+    int log1, log2, tiles1;
 };
-__global__ void __launch_bounds__(256) k3_d12(D12Args a, const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(128, 4) k3_d12(D12Args a, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
     if ((int)blockIdx.x < a.tiles1) {
-        DISPATCH3(a.log1, dcol_body<LG>(a.a1, a.m1, 1 << a.lc1, a.lc1, blockIdx.x, sm, tw, pdl_entry));
+        DISPATCH3(a.log1, dcol_body<LG, 10 - LG, true>(a.a1, a.m1, blockIdx.x, sm, tw, pdl_entry));
     } else {
-        DISPATCH3(a.log2, dcol_body<LG>(a.a2, a.m2, 1 << a.lc2, a.lc2, blockIdx.x - a.tiles1, sm, tw, pdl_entry));
+        DISPATCH3(a.log2, dcol_body<LG, 10 - LG, true>(a.a2, a.m2, blockIdx.x - a.tiles1, sm, tw, pdl_entry));
     }
 }
 
 template <int LOGL>
-__global__ void __launch_bounds__(128) k3_adv(AdvRow<3> a, long long N, int lines, const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(128, 4) k3_adv(AdvStage<3> a, long long N, int lines, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
-    adv_row_body<LOGL, 3, false>(a, (size_t)N, lines, sm, tw, pdl_entry);
+    adv_row_body<LOGL, 3, true, 8>(a, (uint32_t)N, lines, sm, tw, pdl_entry);
 }
 
 template <int LOGL>
-__global__ void __launch_bounds__(128) k3_adj(AdjRow<3> a, long long N, int lines, const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(128, 4) k3_adj(AdjStage<3> a, long long N, int lines, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
-    adj_row_body<LOGL, 3, false, false>(a, (size_t)N, lines, sm, tw, pdl_entry);
+    adj_row_body<LOGL, 3, true, false, 8>(a, (uint32_t)N, lines, sm, tw, pdl_entry);
 }
 
 // lam(1) = ca a + cb c (a nullable) and b = w lam grad m(1): the start of an adjoint solve
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(128) k3_r2c(const float* __restrict__ p0, cons
     const int f = blockIdx.y;
     const float* src = (f < 3 ? p0 + f * D.N : p1 + (f - 3) * D.N);
     const long long row = ((long long)blockIdx.x * lines + q) * 2;
-    LineTw<LOGL> W;
+    LineTw<LOGL, false> W;
     W.load(tw, t);
     pdl_entry();
     float2 x[8];
@@ -120,17 +120,16 @@ __global__ void __launch_bounds__(128) k3_r2c(const float* __restrict__ p0, cons
     for (int k = 0; k < 8; ++k) x[k] = make_float2(src[row * L + t + k * T], src[(row + 1) * L + t + k * T]);
     float2* cur = sm + 2 * q * fft_buf(L);
     float2* nxt = cur + fft_buf(L);
-    auto idx = [](int pos) { return fft_pad(pos); };
-    line_fft<LOGL, false>(x, t, cur, nxt, idx, RowSync<LOGL>(), W);
+    line_fft<LOGL, false, 1>(x, t, cur, nxt, RowSync<LOGL>(), W);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) nxt[idx(t + k * T)] = x[k];
+    for (int k = 0; k < 8; ++k) nxt[fft_pad(t + k * T)] = x[k];
     RowSync<LOGL>()();
     float2* o0 = S + f * D.NS + row * D.W1;
     float2* o1 = o0 + D.W1;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int e = t + k * T;
-        const float2 z = x[k], y = nxt[idx((L - e) & (L - 1))];
+        const float2 z = x[k], y = nxt[fft_pad((L - e) & (L - 1))];
         o0[e] = make_float2(0.5f * (z.x + y.x), 0.5f * (z.y - y.y));
         o1[e] = make_float2(0.5f * (z.y + y.y), -0.5f * (z.x - y.x));
     }
@@ -150,7 +149,7 @@ __global__ void __launch_bounds__(128) k3_c2r(const float2* __restrict__ S, floa
     const int q = threadIdx.x / T, t = threadIdx.x - q * T;
     const int f = blockIdx.y;
     const long long row = ((long long)blockIdx.x * lines + q) * 2;
-    LineTw<LOGL> W;
+    LineTw<LOGL, false> W;
     W.load(tw, t);
     pdl_entry();
     const float2* s0 = S + f * D.NS + row * D.W1;
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(128) k3_c2r(const float2* __restrict__ S, floa
     }
     float2* cur = sm + 2 * q * fft_buf(L);
     float2* nxt = cur + fft_buf(L);
-    line_fft<LOGL, true>(x, t, cur, nxt, [](int pos) { return fft_pad(pos); }, RowSync<LOGL>(), W);
+    line_fft<LOGL, true, 1>(x, t, cur, nxt, RowSync<LOGL>(), W);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         out[f * D.N + row * L + t + k * T] = x[k].x;
@@ -176,24 +175,23 @@ __global__ void __launch_bounds__(128) k3_c2r(const float2* __restrict__ S, floa
 
 // axis 2 of nf half spectra in place: column l = ((f n1 + i1) W1 + e), entries W1 apart
 template <int LOGL, bool INV>
-__global__ void __launch_bounds__(128) k3_axis2(float2* S, Dims3 D, int ncols, int C, int lc,
-                                                const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(128) k3_axis2(float2* S, Dims3 D, int ncols, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
-    constexpr int L = 1 << LOGL, T = L >> 3;
-    const int c = threadIdx.x & (C - 1), t = threadIdx.x >> lc;
+    constexpr int L = 1 << LOGL, T = L >> 3, C = 1024 / L;
+    const int c = threadIdx.x & (C - 1), t = threadIdx.x / C;
     const int l = blockIdx.x * C + c;
     const bool on = l < ncols;
     const int g = l / D.W1;
     float2* p = S + ((long long)g * D.n2) * D.W1 + (l - g * D.W1);
-    LineTw<LOGL> W;
+    LineTw<LOGL, false> W;
     W.load(tw, t);
     pdl_entry();
     float2 x[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) x[k] = on ? p[(long long)(t + k * T) * D.W1] : make_float2(0.f, 0.f);
-    float2* cur = sm + C * fft_buf(L);
-    float2* nxt = sm;
-    line_fft<LOGL, INV>(x, t, cur, nxt, [&](int pos) { return (fft_pad(pos) << lc) + c; }, [] { __syncthreads(); }, W);
+    float2* cur = sm + C * fft_buf(L) + c;
+    float2* nxt = sm + c;
+    line_fft<LOGL, INV, C>(x, t, cur, nxt, [] { __syncthreads(); }, W);
     if (on) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) p[(long long)(t + k * T) * D.W1] = x[k];
@@ -232,34 +230,32 @@ __device__ __forceinline__ double block_sum3(double v) {
 //   A3_ENERGY:   no output; sums of |k|^2 |V|^2 and (1 + |k|^2) |k~ . V|^2 over the full spectrum
 //                (an entry with 0 < e < n3 / 2 stands for itself and its conjugate)
 template <int LOGL, int OP>
-__global__ void __launch_bounds__(128) k3_axis1(Axis1Args a, Dims3 D, int ncols, int C, int lc,
-                                                const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(128) k3_axis1(Axis1Args a, Dims3 D, int ncols, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
-    constexpr int L = 1 << LOGL, T = L >> 3;
+    constexpr int L = 1 << LOGL, T = L >> 3, C = 1024 / L;
     constexpr int NV = OP == A3_PRECOND ? 0 : 3, NB = OP == A3_ENERGY ? 0 : 3;
-    const int c = threadIdx.x & (C - 1), t = threadIdx.x >> lc;
+    const int c = threadIdx.x & (C - 1), t = threadIdx.x / C;
     const int l = blockIdx.x * C + c;
     const bool on = l < ncols;
     const long long S = (long long)D.n2 * D.W1;
-    LineTw<LOGL> W;
+    LineTw<LOGL, false> W;
     W.load(tw, t);
     pdl_entry();
-    float2* cur = sm + C * fft_buf(L);
-    float2* nxt = sm;
-    auto idx = [&](int pos) { return (fft_pad(pos) << lc) + c; };
+    float2* cur = sm + C * fft_buf(L) + c;
+    float2* nxt = sm + c;
     auto sync = [] { __syncthreads(); };
     float2 xv[NV > 0 ? 3 : 1][8], xb[NB > 0 ? 3 : 1][8];
 #pragma unroll
     for (int d = 0; d < NV; ++d) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) xv[d][k] = on ? a.V[d * D.NS + l + (t + k * T) * S] : make_float2(0.f, 0.f);
-        line_fft<LOGL, false>(xv[d], t, cur, nxt, idx, sync, W);
+        line_fft<LOGL, false, C>(xv[d], t, cur, nxt, sync, W);
     }
 #pragma unroll
     for (int d = 0; d < NB; ++d) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) xb[d][k] = on ? a.B[d * D.NS + l + (t + k * T) * S] : make_float2(0.f, 0.f);
-        line_fft<LOGL, false>(xb[d], t, cur, nxt, idx, sync, W);
+        line_fft<LOGL, false, C>(xb[d], t, cur, nxt, sync, W);
     }
     const int i2 = l / D.W1, e = l - i2 * D.W1;
     const float k2 = k_odd(i2, D.n2), e2 = k_even(i2, D.n2);
@@ -314,7 +310,7 @@ __global__ void __launch_bounds__(128) k3_axis1(Axis1Args a, Dims3 D, int ncols,
     }
 #pragma unroll
     for (int d = 0; d < NB; ++d) {
-        line_fft<LOGL, true>(xb[d], t, cur, nxt, idx, sync, W);
+        line_fft<LOGL, true, C>(xb[d], t, cur, nxt, sync, W);
         if (on) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) a.out[d * D.NS + l + (t + k * T) * S] = xb[d][k];
@@ -403,14 +399,9 @@ void launch3(reg3_ctx* c, void (*kern)(KArgs...), dim3 grid, int block, size_t s
     cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-// threads of a column kernel's block: large enough for 64-byte rows of columns on the longest
-// axis, small enough that a small box still has a block for every SM
-int col_threads(const Dims3& D) { return D.N >= (1 << 20) ? 256 : (D.N >= (1 << 17) ? 128 : 64); }
-
 // D1 = d_1 (f mul1), D2 = d_2 (f mul2) (no factor where mul is nullptr)
 void d12(reg3_ctx* c, const float* f, const float* mul1, const float* mul2) {
     const Dims3& D = c->D;
-    const int B = col_threads(D);
     D12Args a;
     a.a1 = DColArgs{f, mul1, nullptr, nullptr, c->D1};
     a.a2 = DColArgs{f, mul2, nullptr, nullptr, c->D2};
@@ -419,11 +410,10 @@ void d12(reg3_ctx* c, const float* f, const float* mul1, const float* mul2) {
     a.m2 = ColMap{D.l3 - 1, D.n2 * D.n3 / 2, D.n3 / 2, nc2};
     a.log1 = D.l1;
     a.log2 = D.l2;
-    a.lc1 = ilog2(B) + 3 - D.l1;
-    a.lc2 = ilog2(B) + 3 - D.l2;
-    a.tiles1 = (nc1 + (1 << a.lc1) - 1) >> a.lc1;
-    const int tiles2 = (nc2 + (1 << a.lc2) - 1) >> a.lc2;
-    launch3(c, k3_d12, a.tiles1 + tiles2, B, dcol_smem(B / 16, 128), a, c->tw);
+    const int C1 = 1024 / D.n1, C2 = 1024 / D.n2;  // columns of a block
+    a.tiles1 = (nc1 + C1 - 1) / C1;
+    const int tiles2 = (nc2 + C2 - 1) / C2;
+    launch3(c, k3_d12, a.tiles1 + tiles2, 128, dcol_smem(C1, D.n1), a, c->tw);
 }
 
 // row kernels: 128 threads a block (64 for small boxes), at most the box's pairs of rows
@@ -441,9 +431,13 @@ Row3 row3(const Dims3& D) {
     return r;
 }
 
-void adv(reg3_ctx* c, const AdvRow<3>& a) {
+void adv(reg3_ctx* c, const AdvStage<3>& a) {
     const Row3 r = row3(c->D);
     DISPATCH3(c->D.l3, launch3(c, k3_adv<LG>, r.grid, r.threads, r.smem, a, c->D.N, r.lines, c->tw));
+}
+void adj(reg3_ctx* c, const AdjStage<3>& a) {
+    const Row3 r = row3(c->D);
+    DISPATCH3(c->D.l3, launch3(c, k3_adj<LG>, r.grid, r.threads, r.smem, a, c->D.N, r.lines, c->tw));
 }
 
 // state (vt == nullptr: y from mT into c->y, gradient history into c->gm) or incremental state
@@ -452,7 +446,7 @@ void forward_solve(reg3_ctx* c, const float* vt) {
     const long long N = c->D.N;
     const float h = 1.f / c->nt;
     float* y = c->y;
-    AdvRow<3> a = {};
+    AdvStage<3> a = {};
     a.D[0] = c->D1;
     a.D[1] = c->D2;
     a.v = c->v;
@@ -500,8 +494,7 @@ void adjoint_solve(reg3_ctx* c, const float* x, float ca, float cb, float* out) 
     const int nt = c->nt;
     const float h = 1.f / nt;
     launch3(c, k3_adj_init, R3_BLOCKS, R3_THREADS, 0, x, ca, c->y, cb, c->lam, out, c->gm + 3 * N * nt, 0.5f * h, N);
-    const Row3 r = row3(c->D);
-    AdjRow<3> a = {};
+    AdjStage<3> a = {};
     a.D[0] = c->D1;
     a.D[1] = c->D2;
     a.v = c->v;
@@ -513,7 +506,7 @@ void adjoint_solve(reg3_ctx* c, const float* x, float ca, float cb, float* out) 
         a.ls = nullptr;
         a.l_out = c->ys;
         a.b = nullptr;
-        DISPATCH3(c->D.l3, launch3(c, k3_adj<LG>, r.grid, r.threads, r.smem, a, N, r.lines, c->tw));
+        adj(c, a);
         d12(c, c->ys, c->v, c->v + N);
         a.stage = 2;
         a.ls = c->ys;
@@ -521,7 +514,7 @@ void adjoint_solve(reg3_ctx* c, const float* x, float ca, float cb, float* out) 
         a.b = out;
         a.gm = c->gm + 3 * N * (j - 1);
         a.w = j == 1 ? 0.5f * h : h;
-        DISPATCH3(c->D.l3, launch3(c, k3_adj<LG>, r.grid, r.threads, r.smem, a, N, r.lines, c->tw));
+        adj(c, a);
     }
 }
 
@@ -535,20 +528,16 @@ void rows_c2r(reg3_ctx* c, const float2* S, float* out) {
     DISPATCH3(c->D.l3, launch3(c, k3_c2r<LG>, dim3(r.grid, 3), r.threads, r.smem, S, out, c->D, r.lines, c->tw));
 }
 // complex column kernels: 128 threads a block
-struct Col3 { int C, lc, grid; size_t smem; };
+struct Col3 { int grid; size_t smem; };
 Col3 col3(int logl, int ncols) {
-    Col3 k;
-    k.lc = 7 + 3 - logl;
-    k.C = 1 << k.lc;
-    k.grid = (ncols + k.C - 1) / k.C;
-    k.smem = dcol_smem(k.C, 1 << logl);
-    return k;
+    const int C = 1024 >> logl;
+    return Col3{(ncols + C - 1) / C, dcol_smem(C, 1 << logl)};
 }
 void axis2(reg3_ctx* c, float2* S, int nf, bool inv) {
     const int nc = nf * c->D.n1 * c->D.W1;
     const Col3 k = col3(c->D.l2, nc);
-    if (inv) DISPATCH3(c->D.l2, launch3(c, k3_axis2<LG, true>, k.grid, 128, k.smem, S, c->D, nc, k.C, k.lc, c->tw))
-    else DISPATCH3(c->D.l2, launch3(c, k3_axis2<LG, false>, k.grid, 128, k.smem, S, c->D, nc, k.C, k.lc, c->tw))
+    if (inv) DISPATCH3(c->D.l2, launch3(c, k3_axis2<LG, true>, k.grid, 128, k.smem, S, c->D, nc, c->tw))
+    else DISPATCH3(c->D.l2, launch3(c, k3_axis2<LG, false>, k.grid, 128, k.smem, S, c->D, nc, c->tw))
 }
 // returns the number of blocks (partial sums, where a.part is set)
 int axis1(reg3_ctx* c, int op, double* part) {
@@ -564,11 +553,11 @@ int axis1(reg3_ctx* c, int op, double* part) {
     const int nc = c->D.n2 * c->D.W1;
     const Col3 k = col3(c->D.l1, nc);
     if (op == A3_ASSEMBLE)
-        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_ASSEMBLE>, k.grid, 128, k.smem, a, c->D, nc, k.C, k.lc, c->tw))
+        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_ASSEMBLE>, k.grid, 128, k.smem, a, c->D, nc, c->tw))
     else if (op == A3_PRECOND)
-        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_PRECOND>, k.grid, 128, k.smem, a, c->D, nc, k.C, k.lc, c->tw))
+        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_PRECOND>, k.grid, 128, k.smem, a, c->D, nc, c->tw))
     else
-        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_ENERGY>, k.grid, 128, k.smem, a, c->D, nc, k.C, k.lc, c->tw))
+        DISPATCH3(c->D.l1, launch3(c, k3_axis1<LG, A3_ENERGY>, k.grid, 128, k.smem, a, c->D, nc, c->tw))
     return k.grid;
 }
 
