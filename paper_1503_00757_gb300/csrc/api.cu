@@ -1061,10 +1061,16 @@ extern "C" int reg_apply_precond_sqrt(reg_ctx* c, const float* x, float* out, in
     return REG_OK;
 }
 
-int apply_smooth_proj(reg_ctx* c, float a, const float* b, float* out) {
+int apply_smooth_proj(reg_ctx* c, float a, const float* b, float* out, int nb, float2* spec, float scale) {
     CTX_CHECK(c);
-    RET(check_ptr(b, "b")); RET(check_ptr(out, "out"));
-    sp_vec(c, OP_SMOOTH_PROJ, a, b, out);
+    const size_t N = c->N;
+    // the column pass works in place: a block reads its columns before it writes them
+    float2 *S1 = spec, *S2 = spec + N / 2;
+    launch_r2c_vec(c, b, b + N, S1, S2, nb);
+    const float2* in[2] = {S1, S2};
+    float2* o[2] = {S1, S2};
+    launch_col(c, OP_SMOOTH_PROJ, in, o, spec_params(c, a), nullptr, nb);
+    launch_c2r_vec(c, S1, S2, out, out + N, nb, scale);
     CKL();
     return REG_OK;
 }

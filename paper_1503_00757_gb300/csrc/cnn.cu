@@ -1103,6 +1103,24 @@ __global__ void k_adam_pack(float* params, const float* __restrict__ gW, const f
     }
 }
 
+// the padded gradients in the flat parameter layout (W (Cout, Cin, 3, 3) then b (Cout) per layer)
+__global__ void k_unpack_grads(const float* __restrict__ gW, const float* __restrict__ gb, int nparams,
+                               const LayerDesc* __restrict__ layers, int nlayers, const long long* __restrict__ gwoff,
+                               const long long* __restrict__ gboff, float* out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nparams) return;
+    int l = 0;
+    while (l + 1 < nlayers && i >= layers[l + 1].woff) ++l;
+    const LayerDesc L = layers[l];
+    if (i < L.boff) {
+        const int j = (int)(i - L.woff), co = j / (L.cin * 9), rem = j - co * L.cin * 9, ci = rem / 9, tap = rem - ci * 9;
+        out[i] = gW[gwoff[l] + ((long long)co * 9 + tap) * L.cinp + ci];
+    } else {
+        const int co = (int)(i - L.boff);
+        out[i] = gb[gboff[l] + co];
+    }
+}
+
 __global__ void k_bias_pad(const float* __restrict__ params, const LayerDesc* __restrict__ layers, int nlayers,
                            float* bpad) {
     for (int l = 0; l < nlayers; ++l)
@@ -1144,7 +1162,8 @@ struct reg_net {
     bool record;               // keep every layer's output gradient (reg_net_layer_tensor)
     bf16* dz_rec[NLAYER];
     reg_ctx* proj_fine;        // output map on the (2H, 2W) grid of reg_net_forward_fine (created on first use)
-    float *coarse_img, *fine_v;  // restricted images (maxB x 2 x H x W), prolonged prediction (maxB x 2 x 2H x 2W)
+    // restricted images (maxB x 2 x H x W), prolonged prediction and its spectra (maxB x 2 x 2H x 2W each)
+    float *coarse_img, *fine_v, *fine_spec;
 };
 
 static size_t conv_smem(int cin, int cout) {
@@ -1269,6 +1288,7 @@ extern "C" void reg_net_destroy(reg_net* n) {
     if (n->proj_fine) reg_destroy(n->proj_fine);
     cudaFree(n->coarse_img);
     cudaFree(n->fine_v);
+    cudaFree(n->fine_spec);
     void* ptrs[] = {n->d_layers, n->params, n->m1, n->m2, n->gW, n->gb, n->d_gwoff, n->d_gboff, n->d_wfoff,
                     n->wf, n->wt, n->bpad, n->dzA, n->dzB, n->out, n->pred, n->res, n->dout, n->partial,
                     n->bpartial, n->d_part, n->d_err};
@@ -1415,16 +1435,11 @@ extern "C" int reg_net_get_params(reg_net* n, float* params) {
     return e == cudaSuccess ? REG_OK : reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));
 }
 
-// out = P G in per velocity (the output map; also its adjoint G P, since P and G
-// are commuting symmetric Fourier multipliers)
-static int leray_batch(reg_net* n, const float* in, float* out, int B) {
-    const size_t f = (size_t)2 * n->H * n->W;
+// out = scale P G in for B velocities (the output map; also its adjoint G P, since P and G
+// are commuting symmetric Fourier multipliers) in three launches; scratch: B 2 H W floats
+static int leray_batch(reg_net* n, const float* in, float* out, int B, float* scratch, float scale = 1.f) {
     const double sigma = 2.0 * (2.0 * M_PI / (double)(n->H > n->W ? n->H : n->W));
-    for (int b = 0; b < B; ++b) {
-        const int st = apply_smooth_proj(n->proj, (float)(0.5 * sigma * sigma), in + b * f, out + b * f);
-        if (st != REG_OK) return st;
-    }
-    return REG_OK;
+    return apply_smooth_proj(n->proj, (float)(0.5 * sigma * sigma), in, out, B, reinterpret_cast<float2*>(scratch), scale);
 }
 
 // a tensor-core conv of an earlier call that reported an MMA timeout (sticky; read from
@@ -1433,7 +1448,7 @@ static int conv_status(reg_net* n) {
     return *n->h_err ? reg_fail(REG_ERR_TIMEOUT, "tensor-core convolution: MMA completion timed out") : REG_OK;
 }
 
-static int net_forward(reg_net* n, const float* images, int B) {
+static int net_forward(reg_net* n, const float* images, int B, float* out, float scale) {
     const int H = n->H, W = n->W;
     int st = conv_status(n);
     if (st != REG_OK) return st;
@@ -1454,23 +1469,13 @@ static int net_forward(reg_net* n, const float* images, int B) {
     cudaMemcpyAsync(n->h_err, n->d_err, sizeof(int), cudaMemcpyDeviceToHost, n->stream);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, std::string("net forward: ") + cudaGetErrorString(e));
-    return leray_batch(n, n->out, n->pred, B);
+    return leray_batch(n, n->out, out, B, n->dout, scale);  // dout is free until the backward pass
 }
 
 extern "C" int reg_net_forward(reg_net* n, const float* images, int B, float* v_out) {
     if (!n || !images || !v_out) return reg_fail(REG_ERR_ARG, "NULL argument");
     if (B < 1 || B > n->maxB) return reg_fail(REG_ERR_ARG, "batch out of range");
-    const int st = net_forward(n, images, B);
-    if (st != REG_OK) return st;
-    cudaError_t e;
-    if (n->out_scale != 1.f) {
-        launch_axpby(n->proj, 2LL * B * n->H * n->W, n->out_scale, n->pred, 0.f, n->pred, -1, -1, v_out);
-        e = cudaGetLastError();
-    } else {
-        e = cudaMemcpyAsync(v_out, n->pred, sizeof(float) * 2 * B * n->H * n->W, cudaMemcpyDeviceToDevice,
-                            n->stream);
-    }
-    return e == cudaSuccess ? REG_OK : reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));
+    return net_forward(n, images, B, v_out, n->out_scale);
 }
 
 extern "C" int reg_net_set_output_scale(reg_net* n, float scale) {
@@ -1480,15 +1485,15 @@ extern "C" int reg_net_set_output_scale(reg_net* n, float scale) {
     return REG_OK;
 }
 
-// forward, loss, backward into n->gW / n->gb
-static int net_loss_grad(reg_net* n, const float* images, const float* targets, int B, double* loss) {
+// forward, loss, backward into n->gW / n->gb and, in the flat parameter layout, grads (nullable)
+static int net_loss_grad(reg_net* n, const float* images, const float* targets, int B, double* loss, float* grads) {
     const int H = n->H, W = n->W;
-    int st = net_forward(n, images, B);
+    int st = net_forward(n, images, B, n->pred, 1.f);
     if (st != REG_OK) return st;
     const long long M = 2LL * B * H * W;
     k_residual<<<256, 256, 0, n->stream>>>(n->pred, targets, n->res, M, n->d_part);
     cudaMemcpyAsync(n->h_part, n->d_part, sizeof(double) * 256, cudaMemcpyDeviceToHost, n->stream);
-    st = leray_batch(n, n->res, n->dout, B);  // dL/d out = G P r / M (scaled below)
+    st = leray_batch(n, n->res, n->dout, B, n->pred);  // dL/d out = G P r / M (scaled below)
     if (st != REG_OK) return st;
     k_pack_grad<<<304, 256, 0, n->stream>>>(n->dout, n->dzA, B, H, W);
     const float invM = 1.0f / (float)M;
@@ -1538,6 +1543,9 @@ static int net_loss_grad(reg_net* n, const float* images, const float* targets, 
     // scale gradients in place
     launch_axpby(n->proj, ngw, invM, n->gW, 0.f, n->gW, -1, -1, n->gW);
     launch_axpby(n->proj, ngb, invM, n->gb, 0.f, n->gb, -1, -1, n->gb);
+    if (grads)
+        k_unpack_grads<<<((int)n->nparams + 255) / 256, 256, 0, n->stream>>>(n->gW, n->gb, (int)n->nparams, n->d_layers,
+                                                                             NLAYER, n->d_gwoff, n->d_gboff, grads);
     cudaMemcpyAsync(n->h_err, n->d_err, sizeof(int), cudaMemcpyDeviceToHost, n->stream);
     e = cudaStreamSynchronize(n->stream);
     if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, std::string("net backward: ") + cudaGetErrorString(e));
@@ -1553,35 +1561,14 @@ extern "C" int reg_net_loss_grad(reg_net* n, const float* images, const float* t
                                  float* grads) {
     if (!n || !images || !targets) return reg_fail(REG_ERR_ARG, "NULL argument");
     if (B < 1 || B > n->maxB) return reg_fail(REG_ERR_ARG, "batch out of range");
-    int st = net_loss_grad(n, images, targets, B, loss);
-    if (st != REG_OK) return st;
-    if (grads) {
-        // unpack padded gradients into the flat oracle layout
-        std::vector<float> hw(n->gwoff.back() + (size_t)n->layers.back().coutp * 9 * n->layers.back().cinp);
-        std::vector<float> hb(n->gboff.back() + n->layers.back().coutp);
-        cudaMemcpy(hw.data(), n->gW, sizeof(float) * hw.size(), cudaMemcpyDeviceToHost);
-        cudaMemcpy(hb.data(), n->gb, sizeof(float) * hb.size(), cudaMemcpyDeviceToHost);
-        std::vector<float> flat(n->nparams);
-        for (int l = 0; l < NLAYER; ++l) {
-            const LayerDesc& L = n->layers[l];
-            for (int co = 0; co < L.cout; ++co)
-                for (int ci = 0; ci < L.cin; ++ci)
-                    for (int tap = 0; tap < 9; ++tap)
-                        flat[L.woff + ((long long)co * L.cin + ci) * 9 + tap] =
-                            hw[n->gwoff[l] + ((long long)co * 9 + tap) * L.cinp + ci];
-            for (int co = 0; co < L.cout; ++co) flat[L.boff + co] = hb[n->gboff[l] + co];
-        }
-        const cudaError_t e = cudaMemcpy(grads, flat.data(), sizeof(float) * n->nparams, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));
-    }
-    return REG_OK;
+    return net_loss_grad(n, images, targets, B, loss, grads);
 }
 
 extern "C" int reg_net_train_step(reg_net* n, const float* images, const float* targets, int B, float lr,
                                   double* loss) {
     if (!n || !images || !targets) return reg_fail(REG_ERR_ARG, "NULL argument");
     if (B < 1 || B > n->maxB) return reg_fail(REG_ERR_ARG, "batch out of range");
-    const int st = net_loss_grad(n, images, targets, B, loss);
+    const int st = net_loss_grad(n, images, targets, B, loss, nullptr);
     if (st != REG_OK) return st;
     repack(n, 1, lr);
     const cudaError_t e = cudaGetLastError();
@@ -1707,29 +1694,28 @@ extern "C" int reg_net_forward_fine(reg_net* n, const float* images, int B, floa
         }
         const size_t pix = (size_t)n->maxB * H * W;
         if (cudaMalloc((void**)&n->coarse_img, sizeof(float) * 2 * pix) != cudaSuccess ||
-            cudaMalloc((void**)&n->fine_v, sizeof(float) * 8 * pix) != cudaSuccess) {
+            cudaMalloc((void**)&n->fine_v, sizeof(float) * 8 * pix) != cudaSuccess ||
+            cudaMalloc((void**)&n->fine_spec, sizeof(float) * 8 * pix) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(n->coarse_img);
-            n->coarse_img = nullptr;
+            cudaFree(n->fine_v);
+            n->coarse_img = n->fine_v = nullptr;
             reg_destroy(pf);
             return reg_fail(REG_ERR_NOMEM, "fine-grid warm-start buffers");
         }
         n->proj_fine = pf;
     }
     k_restrict2<<<304, 256, 0, n->stream>>>(images, n->coarse_img, 2 * B, H, W);
-    int st = net_forward(n, n->coarse_img, B);  // n->pred = P G net(x) on the H x W grid
+    int st = net_forward(n, n->coarse_img, B, n->pred, 1.f);  // n->pred = P G net(x) on the H x W grid
     if (st != REG_OK) return st;
     k_prolong2<<<304, 256, 0, n->stream>>>(n->pred, n->fine_v, 2 * B, H, W);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));
     // the fine grid's own output map P G (sigma = 2 h of that grid), then the output scale
-    const size_t ff = (size_t)2 * Hf * Wf;
     const double sigma = 2.0 * (2.0 * M_PI / (double)(Hf > Wf ? Hf : Wf));
-    for (int b = 0; b < B; ++b) {
-        st = apply_smooth_proj(n->proj_fine, (float)(0.5 * sigma * sigma), n->fine_v + b * ff, v_out + b * ff);
-        if (st != REG_OK) return st;
-    }
-    if (n->out_scale != 1.f) launch_axpby(n->proj_fine, (long long)B * ff, n->out_scale, v_out, 0.f, v_out, -1, -1, v_out);
+    st = apply_smooth_proj(n->proj_fine, (float)(0.5 * sigma * sigma), n->fine_v, v_out, B,
+                           reinterpret_cast<float2*>(n->fine_spec), n->out_scale);
+    if (st != REG_OK) return st;
     e = cudaGetLastError();
     return e == cudaSuccess ? REG_OK : reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));
 }

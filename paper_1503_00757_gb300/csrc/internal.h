@@ -260,9 +260,10 @@ void ktimer_end(reg_ctx* ctx);
 
 int reg_fail(int status, const std::string& msg);
 
-// out = exp(-a |k|^2) P_L b on the context's grid (velocity fields, device):
-// the output map of the warm-start network (Gaussian low-pass, then Leray).
-int apply_smooth_proj(reg_ctx* ctx, float a, const float* b, float* out);
+// out = scale exp(-a |k|^2) P_L b on the context's grid for nb velocity fields back to back (device):
+// the output map of the warm-start network (Gaussian low-pass, then Leray).  spec: nb N spectrum
+// entries of scratch.
+int apply_smooth_proj(reg_ctx* ctx, float a, const float* b, float* out, int nb, float2* spec, float scale);
 
 // ---- cluster-resident transport solves (transport_cluster.cu) ----
 enum TcMode { TC_STATE = 0, TC_ADJOINT = 1, TC_MATVEC = 2 };
