@@ -175,6 +175,7 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->tileR = c->tileC = c->tileP = 0;
     c->pdl = true;
     c->tc_ok = tc_max_active_clusters(c->n1, c->n2) > 0;
+    c->use_rs = rs_available(c->log1, c->log2);
     c->use_tc = false;  // the row / column kernel pairs unless the autotuner measured the cluster kernel faster
     {
         int dev = 0, R, C, P, D, T;
@@ -267,8 +268,9 @@ extern "C" int reg_set_transport(reg_ctx* c, int cluster) {
     if (cluster && !c->tc_ok)
         return reg_fail(REG_ERR_ARG, "the cluster-resident transport kernel does not run on this grid or device");
     const bool on = cluster != 0;
-    if (on != c->use_tc) clear_graphs(c);  // captures bake in the kernels
+    if (on != c->use_tc || c->use_rs) clear_graphs(c);  // captures bake in the kernels
     c->use_tc = on;
+    c->use_rs = false;
     return REG_OK;
 }
 
@@ -727,7 +729,11 @@ static void d1_of(reg_ctx* c, const float* f, const float* mul = nullptr, const 
     launch_dcol(c, DColArgs{f, mul, f2, mul2, dbuf(c)});
 }
 
-// State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[1..nt], gm_hist[0..nt].
+// whole solves in one launch (transport_resident.cu)
+static bool resident(const reg_ctx* c) { return c->use_rs && !c->full_newton && !sp_transport(c); }
+
+// State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[nt] and gm_hist[0..nt]
+// (the kernel pairs also m_hist[1..nt-1]).
 // init (nullable): the field transported instead of the template m_T.
 static void state_solve(reg_ctx* c, const float* v, int nt, const float* init = nullptr) {
     const float h = 1.0f / (float)nt;
@@ -740,6 +746,12 @@ static void state_solve(reg_ctx* c, const float* v, int nt, const float* init = 
     }
     if (sp_transport(c)) {
         state_solve_sp(c, v, nt, m0);
+        return;
+    }
+    if (resident(c)) {
+        RsArgs r = {};
+        r.nt = nt; r.h = h; r.v = v; r.m0 = m0; r.m_out = mh(c, nt); r.gm_out = c->gm_hist;
+        launch_resident(c, RS_STATE, r);
         return;
     }
     AdvStage<2> a = {};
@@ -778,6 +790,12 @@ static void adjoint_solve(reg_ctx* c, const float* v, int nt, const float* a, fl
     if (sp_transport(c)) {
         if (vt) inc_adjoint_full_sp(c, v, vt, nt, bout);
         else adjoint_solve_sp(c, v, nt, a, ca, cf, cb, bout, lhist);
+        return;
+    }
+    if (resident(c) && a && !lhist) {
+        RsArgs r = {};
+        r.nt = nt; r.h = h; r.v = v; r.gm = c->gm_hist; r.adj_a = a; r.ca = ca; r.adj_c = cf; r.cb = cb; r.b = bout;
+        launch_resident(c, RS_ADJOINT, r);
         return;
     }
     float* lst = c->w2;
@@ -958,6 +976,12 @@ static void inc_solves(reg_ctx* c, const float* vt, int nt) {
         a.uj = c->w3; a.us = c->w0; a.lj = c->w1; a.ls = c->w2;
         a.adj_a = nullptr; a.adj_ca = 0.f; a.adj_c = nullptr; a.adj_cb = -1.f; a.b = c->bvec;
         launch_transport_cluster(c, TC_MATVEC, a);
+        return;
+    }
+    if (resident(c)) {
+        RsArgs r = {};
+        r.nt = nt; r.h = 1.0f / (float)nt; r.v = c->v_lin; r.vt = vt; r.gm = c->gm_hist; r.b = c->bvec;
+        launch_resident(c, RS_MATVEC, r);
         return;
     }
     inc_state_solve(c, c->v_lin, vt, nt);

@@ -119,6 +119,7 @@ struct reg_ctx {
     float *lam_hist;   // (nt_cap + 1) * N
     float *gmt_hist;   // (nt_cap + 1) * 2N
     bool tc_ok;        // the cluster-resident transport kernel can run on this grid and device
+    bool use_rs;       // Gauss-Newton transport solves in the resident kernel (small grids)
     bool use_tc;       // transport solves run in the cluster-resident kernel (else the two-pass kernels)
     int tileR, tileC;  // rows per row-kernel CTA, spectrum columns per column-kernel CTA (0: default)
     int tileP;         // 1: RK2 row kernels prefetch their operands (used when tileR > 0)
@@ -264,6 +265,25 @@ int reg_fail(int status, const std::string& msg);
 // the output map of the warm-start network (Gaussian low-pass, then Leray).  spec: nb N spectrum
 // entries of scratch.
 int apply_smooth_proj(reg_ctx* ctx, float a, const float* b, float* out, int nb, float2* spec, float scale);
+
+// ---- small grids: whole transport solves resident in one cluster (transport_resident.cu) ----
+enum RsMode { RS_STATE = 0, RS_ADJOINT = 1, RS_MATVEC = 2 };
+struct RsArgs {
+    int nt;
+    float h;             // 1 / nt
+    const float* v;      // velocity (2N)
+    const float* vt;     // RS_MATVEC: incremental velocity (2N)
+    const float* m0;     // RS_STATE: the transported field at t = 0
+    float* m_out;        // RS_STATE: m(1)
+    float* gm_out;       // RS_STATE: grad m_j, j = 0..nt (2N each)
+    const float* gm;     // the others: that history
+    const float *adj_a, *adj_c;  // RS_ADJOINT: lam(1) = ca adj_a + cb adj_c (RS_MATVEC: -m~(1))
+    float ca, cb;
+    float* b;            // body force (2N): written
+};
+// grids of 64 to 256 points per axis on a device that fits the clusters (prepares the kernels)
+bool rs_available(int log1, int log2);
+void launch_resident(reg_ctx* ctx, int mode, const RsArgs& a);
 
 // ---- cluster-resident transport solves (transport_cluster.cu) ----
 enum TcMode { TC_STATE = 0, TC_ADJOINT = 1, TC_MATVEC = 2 };

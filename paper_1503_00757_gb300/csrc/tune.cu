@@ -51,6 +51,7 @@ double time_matvec(reg_grid grid, int nt, int R, int C, int P, int D, int T, std
         L.ctx->tileP = P;
         L.ctx->pdl = D != 0;
         L.ctx->use_tc = T != 0 && L.ctx->tc_ok;
+        L.ctx->use_rs = false;  // the tiles are those of the kernel pairs
         float* o = out + i * N2;
         ok = reg_set_stream(L.ctx, L.st) == REG_OK && reg_set_images(L.ctx, mT, mR) == REG_OK &&
              reg_gradient(L.ctx, v, o, nullptr) == REG_OK;
