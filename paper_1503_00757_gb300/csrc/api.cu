@@ -114,7 +114,7 @@ extern "C" void reg_destroy(reg_ctx* c) {
                     &c->bvec, &c->vtmp, &c->vtmp2, &c->gtmp, &c->T3, &c->T3b, &c->vx, &c->g, &c->r, &c->z, &c->s, &c->Hs,
                     &c->vt, &c->vtrial, &c->F, &c->Fs, &c->gF, &c->gv, &c->ybuf, &c->ytrial, &c->vtil};
     for (auto p : fl) cudaFree(*p);
-    for (int i = 0; i < 6; ++i) cudaFree(c->S[i]);
+    cudaFree(c->S[0]);
     free_hist(c);
     clear_graphs(c);
     if (c->cap) cudaStreamDestroy(c->cap);
@@ -175,7 +175,7 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->tileR = c->tileC = c->tileP = 0;
     c->pdl = true;
     c->tc_ok = tc_max_active_clusters(c->n1, c->n2) > 0;
-    c->use_rs = rs_available(c->log1, c->log2);
+    c->use_rs = rs_available(c->log1, c->log2) && rs_sp_available(c->log1, c->log2);
     c->use_tc = false;  // the row / column kernel pairs unless the autotuner measured the cluster kernel faster
     {
         int dev = 0, R, C, P, D, T;
@@ -202,8 +202,8 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     A(&c->vt, 2 * N); A(&c->vtrial, 2 * N);
     A(&c->ybuf, 2 * N); A(&c->ytrial, 2 * N); A(&c->vtil, 2 * N);
     A(&c->F, 4 * N); A(&c->Fs, 4 * N); A(&c->gF, 8 * N); A(&c->gv, 4 * N);
-    for (int i = 0; i < 6 && ok; ++i)
-        if (cudaMalloc(&c->S[i], sizeof(float2) * N / 2) != cudaSuccess) ok = false;
+    if (ok && cudaMalloc(&c->S[0], sizeof(float2) * 6 * (N / 2)) != cudaSuccess) ok = false;
+    for (int i = 1; i < 6 && ok; ++i) c->S[i] = c->S[0] + i * (N / 2);  // one block: batched passes stride through it
     c->npart = 5 * 304 + 4096;
     if (ok && cudaMalloc(&c->d_scal, sizeof(double) * SL_COUNT) != cudaSuccess) ok = false;
     if (ok && cudaMalloc(&c->d_part, sizeof(double) * c->npart) != cudaSuccess) ok = false;
@@ -508,8 +508,13 @@ static void sp_grad_vec(reg_ctx* c, const float* u, float* gv) {
 // for the shear model's strain, whose viscosity magnifies a change of its last bits: H v~ of the
 // nu = 3 test point moves by 1e-5 between the two ways to take the same gradient
 static void sp_grad_vec_spec(reg_ctx* c, const float* u, float* gv) {
-    sp_grad_spec(c, u, gv);
-    sp_grad_spec(c, u + c->N, gv + 2 * (size_t)c->N);
+    // spectra of the two components in S[0], S[0] + N / 2 entries and so on: consecutive halves of one block
+    const long long half = c->N / 2;
+    launch_r2c_scalar(c, u, c->S[0], 2, 3 * half);
+    const float2* in[1] = {c->S[0]};
+    float2* o[2] = {c->S[0] + half, c->S[0] + 2 * half};
+    launch_col(c, OP_GRAD, in, o, spec_params(c, 0.f), nullptr, 2, 3 * half);
+    launch_c2r_vec(c, c->S[0] + half, c->S[0] + 2 * half, gv, gv + c->N, 2, 1.f, 3 * half);
 }
 
 // out = div T (2 planes) of a symmetric tensor T = (T11, T12, T22)
@@ -600,6 +605,14 @@ static float* gmth(reg_ctx* c, int j) { return c->gmt_hist + (size_t)j * 2 * c->
 // ---- the same solves with the stages in the row spectra (kernels.cu): H2 and H3 problems ----
 static bool sp_transport(const reg_ctx* c) { return c->ypath; }
 
+// grad m(1) from the row spectra of m(1) in S[0]
+static void grad_end_sp(reg_ctx* c, int nt) {
+    const float2* in[1] = {c->S[0]};
+    float2* G[2] = {c->S[1], c->S[2]};
+    launch_col(c, OP_GRAD, in, G, spec_params(c, 0.f), nullptr);
+    launch_c2r_vec(c, c->S[1], c->S[2], gmh(c, nt), gmh(c, nt) + c->N);
+}
+
 // State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[0..nt], gm_hist[0..nt].
 // The column pass transforms only d1 (OP_GRAD1); d2 is diagonal in the row
 // spectra and is formed by the row kernel from the stage's own spectrum S[0].
@@ -623,9 +636,7 @@ static void state_solve_sp(reg_ctx* c, const float* v, int nt, const float* m0) 
         a.us = c->w0; a.u_out = mh(c, j + 1); a.grad_out = nullptr; a.stage = 2;
         launch_row_adv(c, a);
     }
-    float2* G2[2] = {c->S[1], c->S[2]};
-    launch_col(c, OP_GRAD, in, G2, P, nullptr);
-    launch_c2r_vec(c, c->S[1], c->S[2], gmh(c, nt), gmh(c, nt) + c->N);
+    grad_end_sp(c, nt);
 }
 
 // Adjoint (Eq. (e:adj-eq-elim)) or Gauss-Newton incremental adjoint
@@ -730,7 +741,7 @@ static void d1_of(reg_ctx* c, const float* f, const float* mul = nullptr, const 
 }
 
 // whole solves in one launch (transport_resident.cu)
-static bool resident(const reg_ctx* c) { return c->use_rs && !c->full_newton && !sp_transport(c); }
+static bool resident(const reg_ctx* c) { return c->use_rs && !c->full_newton; }
 
 // State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[nt] and gm_hist[0..nt]
 // (the kernel pairs also m_hist[1..nt-1]).
@@ -742,6 +753,13 @@ static void state_solve(reg_ctx* c, const float* v, int nt, const float* init = 
         TcArgs a = {};
         a.nt = nt; a.h = h; a.v = v; a.mT = m0; a.m_hist = c->m_hist; a.gm_hist = c->gm_hist; a.us = c->w0;
         launch_transport_cluster(c, TC_STATE, a);
+        return;
+    }
+    if (sp_transport(c) && resident(c)) {
+        RsArgs r = {};
+        r.nt = nt; r.h = h; r.v = v; r.m0 = m0; r.m_out = mh(c, nt); r.gm_out = c->gm_hist; r.s_out = c->S[0];
+        launch_resident_sp(c, RS_STATE, r);
+        grad_end_sp(c, nt);
         return;
     }
     if (sp_transport(c)) {
@@ -787,15 +805,16 @@ static void adjoint_solve(reg_ctx* c, const float* v, int nt, const float* a, fl
         launch_transport_cluster(c, TC_ADJOINT, t);
         return;
     }
-    if (sp_transport(c)) {
-        if (vt) inc_adjoint_full_sp(c, v, vt, nt, bout);
-        else adjoint_solve_sp(c, v, nt, a, ca, cf, cb, bout, lhist);
-        return;
-    }
     if (resident(c) && a && !lhist) {
         RsArgs r = {};
         r.nt = nt; r.h = h; r.v = v; r.gm = c->gm_hist; r.adj_a = a; r.ca = ca; r.adj_c = cf; r.cb = cb; r.b = bout;
-        launch_resident(c, RS_ADJOINT, r);
+        if (sp_transport(c)) launch_resident_sp(c, RS_ADJOINT, r);
+        else launch_resident(c, RS_ADJOINT, r);
+        return;
+    }
+    if (sp_transport(c)) {
+        if (vt) inc_adjoint_full_sp(c, v, vt, nt, bout);
+        else adjoint_solve_sp(c, v, nt, a, ca, cf, cb, bout, lhist);
         return;
     }
     float* lst = c->w2;
@@ -981,7 +1000,8 @@ static void inc_solves(reg_ctx* c, const float* vt, int nt) {
     if (resident(c)) {
         RsArgs r = {};
         r.nt = nt; r.h = 1.0f / (float)nt; r.v = c->v_lin; r.vt = vt; r.gm = c->gm_hist; r.b = c->bvec;
-        launch_resident(c, RS_MATVEC, r);
+        if (sp_transport(c)) launch_resident_sp(c, RS_MATVEC, r);
+        else launch_resident(c, RS_MATVEC, r);
         return;
     }
     inc_state_solve(c, c->v_lin, vt, nt);
@@ -1093,7 +1113,7 @@ int apply_smooth_proj(reg_ctx* c, float a, const float* b, float* out, int nb, f
     launch_r2c_vec(c, b, b + N, S1, S2, nb);
     const float2* in[2] = {S1, S2};
     float2* o[2] = {S1, S2};
-    launch_col(c, OP_SMOOTH_PROJ, in, o, spec_params(c, a), nullptr, nb);
+    launch_col(c, OP_SMOOTH_PROJ, in, o, spec_params(c, a), nullptr, nb, (long long)N);
     launch_c2r_vec(c, S1, S2, out, out + N, nb, scale);
     CKL();
     return REG_OK;

@@ -491,6 +491,19 @@ __device__ __forceinline__ void adj_row_body(const AdjStage<DIM>& a, uint32_t N,
             x[k] = make_float2(fmaf(l.x, m.x, x[k].x), fmaf(l.y, m.y, x[k].y));
         }
     }
+    // 2-D: the gradient history comes from HBM on large grids, so it is fetched ahead of the wait as
+    // well (3-D blocks are held to 128 registers and live on warps in flight instead)
+    constexpr bool EARLYB = PRE && !FULL && DIM == 2;
+    float2 gE[EARLYB ? DIM : 1][8], bE[EARLYB ? DIM : 1][8];
+    if (EARLYB && a.b) {
+#pragma unroll
+        for (int d = 0; d < (EARLYB ? DIM : 0); ++d)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                gE[d][k] = pair(a.gm, d * N, k);
+                bE[d][k] = pair(a.b, d * N, k);
+            }
+    }
     row_deriv<LOGL>(x, t, q, sm, W);
     if (PRE) wait();
     constexpr int B = PRE ? 8 : BATCH;
@@ -551,7 +564,8 @@ __device__ __forceinline__ void adj_row_body(const AdjStage<DIM>& a, uint32_t N,
         float2 b[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const float2 g = pair(a.gm, d * N, k), o = pair(a.b, d * N, k), l = cscale(u[k], a.w);
+            const float2 g = EARLYB ? gE[EARLYB ? d : 0][k] : pair(a.gm, d * N, k);
+            const float2 o = EARLYB ? bE[EARLYB ? d : 0][k] : pair(a.b, d * N, k), l = cscale(u[k], a.w);
             b[k] = make_float2(fmaf(l.x, g.x, o.x), fmaf(l.y, g.y, o.y));
             if (FULL) {
                 const float2 m = cscale(pair(a.lsrc, 0, k), a.w), gt = pair(a.gmt, d * N, k);

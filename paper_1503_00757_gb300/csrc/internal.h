@@ -92,7 +92,7 @@ struct reg_ctx {
     float *E_lin, *eta_lin;
 
     // spectra (transposed packed layout, N/2 float2 each)
-    float2 *S[6];
+    float2 *S[6];  // one allocation
     // scalar work fields
     float *w0, *w1, *w2, *w3;
     // vector work fields (2N each)
@@ -153,15 +153,16 @@ void fill_twiddles(float2* h);
 size_t row_smem(int R, int L);
 size_t col_smem(int C, int L, bool div1);
 
-void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S);
+// nb fields back to back, spectra ss entries apart
+void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S, int nb = 1, long long ss = 0);
 // nb vector fields back to back (2 N floats each; spectra S1, S2: N entries apart from field to field)
 void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, float2* S2, int nb = 1);
 void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f);
 void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb = 1,
-                    float scale = 1.f);
-// nb > 1 (OP_SMOOTH_PROJ only): fields N entries apart
+                    float scale = 1.f, long long ss = 0);  // ss: entries from field to field (0: N)
+// nb > 1 (OP_GRAD and OP_SMOOTH_PROJ only): independent fields, bs spectrum entries apart
 void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* out, const SpecParams& P,
-                double* part_out, int nb = 1);
+                double* part_out, int nb = 1, long long bs = 0);
 
 // transport stages (deriv.cuh)
 struct DColArgs;
@@ -275,7 +276,8 @@ struct RsArgs {
     const float* vt;     // RS_MATVEC: incremental velocity (2N)
     const float* m0;     // RS_STATE: the transported field at t = 0
     float* m_out;        // RS_STATE: m(1)
-    float* gm_out;       // RS_STATE: grad m_j, j = 0..nt (2N each)
+    float* gm_out;       // RS_STATE: grad m_j, j = 0..nt (spectral stages: j < nt) (2N each)
+    float2* s_out;       // RS_STATE, spectral stages: row spectra of m(1)
     const float* gm;     // the others: that history
     const float *adj_a, *adj_c;  // RS_ADJOINT: lam(1) = ca adj_a + cb adj_c (RS_MATVEC: -m~(1))
     float ca, cb;
@@ -284,6 +286,9 @@ struct RsArgs {
 // grids of 64 to 256 points per axis on a device that fits the clusters (prepares the kernels)
 bool rs_available(int log1, int log2);
 void launch_resident(reg_ctx* ctx, int mode, const RsArgs& a);
+// the same with the spectral stages (transport_resident_sp.cu)
+bool rs_sp_available(int log1, int log2);
+void launch_resident_sp(reg_ctx* ctx, int mode, const RsArgs& a);
 
 // ---- cluster-resident transport solves (transport_cluster.cu) ----
 enum TcMode { TC_STATE = 0, TC_ADJOINT = 1, TC_MATVEC = 2 };

@@ -838,13 +838,14 @@ static RowCfg row_cfg(reg_ctx* ctx) {
     return c;
 }
 
-void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S) {
+void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S, int nb, long long ss) {
     const RowCfg g = row_cfg(ctx);
-    ktimer_begin(ctx, KC_ROW, 8.0 * ctx->N);
+    ktimer_begin(ctx, KC_ROW, 8.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_r2c<LG, false>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw, Batch{0, 0});
+        launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw,
+                 Batch{(long long)ctx->N, ss});
     });
     ktimer_end(ctx);
 }
@@ -872,14 +873,15 @@ void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f) {
     ktimer_end(ctx);
 }
 
-void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb, float scale) {
+void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb, float scale,
+                    long long ss) {
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_c2r<LG, true>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, S1, S2, u1, u2, g.R, ctx->tw,
-                 Batch{2LL * ctx->N, (long long)ctx->N}, scale);
+                 Batch{2LL * ctx->N, ss > 0 ? ss : (long long)ctx->N}, scale);
     });
     ktimer_end(ctx);
 }
@@ -932,12 +934,12 @@ void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, 
 
 template <int NIN, int NOUT, int OP>
 static void launch_col_t(reg_ctx* ctx, const float2* const* in, float2* const* out, const SpecParams& P,
-                         double* part, int nb = 1) {
+                         double* part, int nb = 1, long long bs = 0) {
     const int L = ctx->n1, W = ctx->n2 / 2;
     const int cpb = spec_cols_per_cta(ctx);
     const size_t smem = col_smem(cpb, L, OP == OP_DIV1);
     ColArgs a;
-    a.bs = nb > 1 ? ctx->N : 0;
+    a.bs = bs;
     for (int f = 0; f < 5; ++f) a.in[f] = (f < NIN) ? in[f] : nullptr;
     if (OP == OP_DIV1) a.in[1] = in[1];  // read untransformed in the store phase
     for (int o = 0; o < 2; ++o) a.out[o] = (o < NOUT) ? out[o] : nullptr;
@@ -959,9 +961,9 @@ static void launch_col_t(reg_ctx* ctx, const float2* const* in, float2* const* o
 int col_blocks(reg_ctx* ctx) { return (ctx->n2 / 2) / spec_cols_per_cta(ctx); }
 
 void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* out, const SpecParams& P,
-                double* part, int nb) {
+                double* part, int nb, long long bs) {
     switch (op) {
-        case OP_GRAD: launch_col_t<1, 2, OP_GRAD>(ctx, in, out, P, part); break;
+        case OP_GRAD: launch_col_t<1, 2, OP_GRAD>(ctx, in, out, P, part, nb, bs); break;
         case OP_DIV: launch_col_t<2, 1, OP_DIV>(ctx, in, out, P, part); break;
         case OP_REG: launch_col_t<2, 2, OP_REG>(ctx, in, out, P, part); break;
         case OP_PROJ: launch_col_t<2, 2, OP_PROJ>(ctx, in, out, P, part); break;
@@ -971,7 +973,7 @@ void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* ou
         case OP_DIVT_PROJ: launch_col_t<5, 2, OP_DIVT_PROJ>(ctx, in, out, P, part); break;
         case OP_GRAD1: launch_col_t<1, 1, OP_GRAD1>(ctx, in, out, P, part); break;
         case OP_DIV1: launch_col_t<1, 1, OP_DIV1>(ctx, in, out, P, part); break;
-        case OP_SMOOTH_PROJ: launch_col_t<2, 2, OP_SMOOTH_PROJ>(ctx, in, out, P, part, nb); break;
+        case OP_SMOOTH_PROJ: launch_col_t<2, 2, OP_SMOOTH_PROJ>(ctx, in, out, P, part, nb, bs); break;
         case OP_SMOOTH: launch_col_t<1, 1, OP_SMOOTH>(ctx, in, out, P, part); break;
         case OP_MASSP: launch_col_t<2, 2, OP_MASSP>(ctx, in, out, P, part); break;
         case OP_QINV: launch_col_t<2, 2, OP_QINV>(ctx, in, out, P, part); break;

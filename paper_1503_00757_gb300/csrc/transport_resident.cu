@@ -15,33 +15,12 @@
 #include <map>
 #include <mutex>
 
+#include "cluster.cuh"
 #include "deriv.cuh"
 #include "internal.h"
 #include "launch.cuh"
 
 namespace {
-
-__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t cl_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// address of this CTA's shared location p in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t cl_map(const void* p, int rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ float2 cl_load(uint32_t a) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ void cl_store(uint32_t a, float2 v) {
-    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
-}
 
 template <int LOG1, int LOG2>
 struct RsGeom {
@@ -258,46 +237,15 @@ __global__ void __launch_bounds__(2 * RsGeom<LOG1, LOG2>::TB, 1) k_resident(RsAr
 template <int LOG1, int LOG2, int MODE>
 cudaLaunchConfig_t rs_config(cudaStream_t st, cudaLaunchAttribute* attr, bool pdl) {
     using G = RsGeom<LOG1, LOG2>;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(G::CS);
-    cfg.blockDim = dim3(2 * G::TB);
-    cfg.dynamicSmemBytes = G::SMEM;
-    cfg.stream = st;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = G::CS;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 2 : 1;
-    return cfg;
+    return cluster_config(G::CS, 2 * G::TB, G::SMEM, st, attr, pdl);
 }
 
 template <int LOG1, int LOG2, int MODE>
 bool rs_prepare() {
-    using G = RsGeom<LOG1, LOG2>;
-    auto k = k_resident<LOG1, LOG2, MODE>;
-    int num = 0;
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = rs_config<LOG1, LOG2, MODE>(0, attr, false);
-    const bool ok =
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&num, k, &cfg) == cudaSuccess && num > 0;
-    if (!ok) cudaGetLastError();
-    return ok;
+    const cudaLaunchConfig_t cfg = rs_config<LOG1, LOG2, MODE>(0, attr, false);
+    return cluster_prepare(k_resident<LOG1, LOG2, MODE>, cfg);
 }
-
-#define RS_CASE(L1, L2, ...) \
-    case (L1)*16 + (L2): { constexpr int B1 = L1, B2 = L2; __VA_ARGS__; } break;
-#define RS_DISPATCH(L1, L2, ...)                                                              \
-    switch ((L1)*16 + (L2)) {                                                                 \
-        RS_CASE(6, 6, __VA_ARGS__) RS_CASE(6, 7, __VA_ARGS__) RS_CASE(6, 8, __VA_ARGS__)      \
-        RS_CASE(7, 6, __VA_ARGS__) RS_CASE(7, 7, __VA_ARGS__) RS_CASE(7, 8, __VA_ARGS__)      \
-        RS_CASE(8, 6, __VA_ARGS__) RS_CASE(8, 7, __VA_ARGS__)                                 \
-        default: break;                                                                       \
-    }
 
 }  // namespace
 

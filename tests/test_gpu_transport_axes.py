@@ -61,6 +61,8 @@ def test_gradient_and_matvec_at_grid_edges(n1, n2, nt):
 
 
 @pytest.mark.parametrize("n1,n2,nt,gamma,shear", [
+    (64, 64, 3, 1e-3, "H2"), (64, 128, 1, math.inf, "H2"), (64, 256, 2, 0.0, "H3"), (128, 64, 2, 1e-3, "H2"),
+    (128, 128, 5, math.inf, "H2"), (128, 256, 2, 1e-3, "H2"), (256, 64, 3, math.inf, "H3"), (256, 128, 2, 0.0, "H2"),
     (64, 64, 1, 0.0, 0.0), (64, 128, 4, 1e-3, 0.0), (64, 256, 3, math.inf, 0.0), (128, 64, 2, math.inf, 0.5),
     (128, 128, 7, 1e-3, 0.0), (128, 256, 2, 0.0, 0.0), (256, 64, 3, math.inf, 0.0), (256, 128, 2, 1e-3, -0.5),
     (256, 256, 5, math.inf, 0.0)])
@@ -73,7 +75,9 @@ def test_resident_solves_equal_the_kernel_pairs(n1, n2, nt, gamma, shear):
     outs = []
     for resident in (True, False):
         for stream in (None, torch.cuda.Stream()):
-            ctx = Context(n1, n2, nt, regnorm=1, beta=1e-3, gamma=gamma, shear=shear, stream=stream)
+            norm = {"H2": 2, "H3": 3}.get(shear, 1)  # the seminorms that keep the spectral stages
+            ctx = Context(n1, n2, nt, regnorm=norm, beta=1e-3, gamma=gamma, shear=shear if norm == 1 else 0.0,
+                          stream=stream)
             if not resident:
                 ctx.set_transport(False)
             ctx.set_images(mTd, mRd)
