@@ -241,6 +241,133 @@ __device__ __forceinline__ void dcol_body(const DColArgs& a, const ColMap& m, in
     }
 }
 
+// ---- 16 entries a thread: lines of 128 and 256 points with one exchange per transform ----
+// On fields that fill the chip dcol_body is bound by shared memory (l1tex 78 % busy at 128^3): two
+// exchanges per transform of such a line.  A thread with 16 entries needs one: a DFT of length 16
+// over its entries t + k T (T = L / 16), the factors w^(t j), one exchange, then a DFT of length T
+// over t.  Half the threads per line, so it is for grids that have blocks to spare.
+template <bool INV>
+__device__ __forceinline__ void line_dft4(float2& a0, float2& a1, float2& a2, float2& a3) {
+    const float2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = mul_mi<INV>(csub(a1, a3));
+    a0 = cadd(t0, t2);
+    a1 = cadd(t1, t3);
+    a2 = csub(t0, t2);
+    a3 = csub(t1, t3);
+}
+template <bool INV>
+__device__ __forceinline__ void line_dft16(float2 (&x)[16]) {
+    // k = k1 + 4 k2, j = j2 + 4 j1: DFT-4 over k2, w16^(k1 j2), DFT-4 over k1
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) line_dft4<INV>(x[k1], x[k1 + 4], x[k1 + 8], x[k1 + 12]);
+    const float c = 0.92387953251128675613f, s = 0.38268343236508977173f, r = 0.70710678118654752440f;
+    const float2 w[10] = {{1.f, 0.f}, {c, -s}, {r, -r}, {s, -c}, {0.f, -1.f}, {0.f, 0.f}, {-r, -r}, {0.f, 0.f}, {0.f, 0.f}, {-c, s}};
+#pragma unroll
+    for (int j2 = 1; j2 < 4; ++j2)
+#pragma unroll
+        for (int k1 = 1; k1 < 4; ++k1) {
+            if (j2 * k1 == 4) {
+                x[k1 + 4 * j2] = mul_mi<INV>(x[k1 + 4 * j2]);
+            } else {
+                const float2 u = w[j2 * k1];
+                x[k1 + 4 * j2] = cmul(x[k1 + 4 * j2], make_float2(u.x, INV ? -u.y : u.y));
+            }
+        }
+    float2 y[16];
+#pragma unroll
+    for (int j2 = 0; j2 < 4; ++j2) {
+        line_dft4<INV>(x[4 * j2], x[4 * j2 + 1], x[4 * j2 + 2], x[4 * j2 + 3]);
+#pragma unroll
+        for (int j1 = 0; j1 < 4; ++j1) y[j2 + 4 * j1] = x[4 * j2 + j1];
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = y[k];
+}
+
+template <int LOGL>
+struct Wide {
+    static constexpr int L = 1 << LOGL, T = L / 16, C = 128 / T;      // 128 threads: C columns
+    static constexpr int P = C >= 16 ? T : T + 1;                     // pitch of a row j of the exchange (16 lanes of
+                                                                      // an access fall on distinct banks)
+    static constexpr size_t SMEM = 2 * (size_t)16 * P * C * sizeof(float2);
+};
+
+template <int LOGL, bool INV>
+__device__ __forceinline__ void wide_fft(float2 (&x)[16], int t, float2* buf, const float2 (&w)[15]) {
+    using G = Wide<LOGL>;
+    constexpr int C = G::C, P = G::P;
+    line_dft16<INV>(x);
+    buf[t * C] = x[0];
+#pragma unroll
+    for (int j = 1; j < 16; ++j) buf[(j * P + t) * C] = cmul(x[j], make_float2(w[j - 1].x, INV ? -w[j - 1].y : w[j - 1].y));
+    __syncthreads();
+    if constexpr (LOGL == 8) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = buf[(t * P + k) * C];
+        line_dft16<INV>(x);
+    } else {  // T = 8: rows t and t + 8, whose outputs interleave
+        float2 a[8], b[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            a[k] = buf[(t * P + k) * C];
+            b[k] = buf[((t + 8) * P + k) * C];
+        }
+        line_dft8<INV>(a);
+        line_dft8<INV>(b);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            x[2 * k] = a[k];
+            x[2 * k + 1] = b[k];
+        }
+    }
+}
+
+// dcol_body (without the second product) for LOGL = 7, 8 and 128 threads a block
+template <int LOGL, class Wait>
+__device__ __forceinline__ void dcol_wide_body(const DColArgs& a, const ColMap& m, int tile, float2* sm,
+                                               const float2* __restrict__ tw, Wait wait) {
+    using G = Wide<LOGL>;
+    constexpr int L = G::L, T = G::T, C = G::C;
+    const int c = threadIdx.x & (C - 1), t = threadIdx.x / C;
+    const int l = tile * C + c;
+    const bool on = l < m.ncols;
+    const uint32_t base = (uint32_t)(l >> m.lq) * m.P + (l & ((1 << m.lq) - 1)) + (uint32_t)t * m.S;
+    const uint32_t step = (uint32_t)T * m.S;
+    float2 w[15];
+#pragma unroll
+    for (int j = 1; j < 16; ++j) w[j - 1] = __ldg(&tw[t * j * (REG_TW_N / L)]);
+    wait();
+    float2 x[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) x[k] = make_float2(0.f, 0.f);
+    if (on) {
+        const float2* f = reinterpret_cast<const float2*>(a.f) + base;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = f[k * step];
+        if (a.mul) {
+            const float2* g = reinterpret_cast<const float2*>(a.mul) + base;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const float2 y = g[k * step];
+                x[k] = make_float2(__fmul_rn(x[k].x, y.x), __fmul_rn(x[k].y, y.y));
+            }
+        }
+    }
+    wide_fft<LOGL, false>(x, t, sm + c, w);
+    const float f = (float)t * (1.0f / (float)L);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        float kk = f + (k < 8 ? (float)(k * T) : (float)(k * T - L)) * (1.0f / (float)L);
+        if (k == 8 && t == 0) kk = 0.f;
+        x[k] = make_float2(__fmul_rn(-kk, x[k].y), __fmul_rn(kk, x[k].x));
+    }
+    wide_fft<LOGL, true>(x, t, sm + 16 * G::P * C + c, w);
+    if (on) {
+        float2* o = reinterpret_cast<float2*>(a.out) + base;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) o[k * step] = x[k];
+    }
+}
+
 // shared memory of dcol_body: two exchange buffers of C columns
 inline size_t dcol_smem(int C, int L) { return 2 * (size_t)C * fft_buf(L) * sizeof(float2); }
 

@@ -65,12 +65,18 @@ struct D12Args {
     ColMap m1, m2;
     int log1, log2, tiles1;
 };
+template <int LOGL, bool WIDE>
+__device__ __forceinline__ void d12_role(const DColArgs& a, const ColMap& m, int tile, float2* sm, const float2* __restrict__ tw) {
+    if constexpr (WIDE && LOGL >= 7) dcol_wide_body<LOGL>(a, m, tile, sm, tw, pdl_entry);
+    else dcol_body<LOGL, 10 - LOGL, true>(a, m, tile, sm, tw, pdl_entry);
+}
+template <bool WIDE>
 __global__ void __launch_bounds__(128, 4) k3_d12(D12Args a, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
     if ((int)blockIdx.x < a.tiles1) {
-        DISPATCH3(a.log1, dcol_body<LG, 10 - LG, true>(a.a1, a.m1, blockIdx.x, sm, tw, pdl_entry));
+        DISPATCH3(a.log1, d12_role<LG, WIDE>(a.a1, a.m1, blockIdx.x, sm, tw));
     } else {
-        DISPATCH3(a.log2, dcol_body<LG, 10 - LG, true>(a.a2, a.m2, blockIdx.x - a.tiles1, sm, tw, pdl_entry));
+        DISPATCH3(a.log2, d12_role<LG, WIDE>(a.a2, a.m2, blockIdx.x - a.tiles1, sm, tw));
     }
 }
 
@@ -410,10 +416,17 @@ void d12(reg3_ctx* c, const float* f, const float* mul1, const float* mul2) {
     a.m2 = ColMap{D.l3 - 1, D.n2 * D.n3 / 2, D.n3 / 2, nc2};
     a.log1 = D.l1;
     a.log2 = D.l2;
-    const int C1 = 1024 / D.n1, C2 = 1024 / D.n2;  // columns of a block
+    // 16 entries a thread on axes of 128 and 256 points where that leaves several blocks per SM
+    const bool wide = D.N >= (1 << 20);
+    auto cols = [&](int n) { return (wide && n >= 128 ? 2048 : 1024) / n; };  // columns of a block
+    auto smem = [&](int n) {
+        return wide && n >= 128 ? (n == 128 ? Wide<7>::SMEM : Wide<8>::SMEM) : dcol_smem(1024 / n, n);
+    };
+    const int C1 = cols(D.n1), C2 = cols(D.n2);
     a.tiles1 = (nc1 + C1 - 1) / C1;
     const int tiles2 = (nc2 + C2 - 1) / C2;
-    launch3(c, k3_d12, a.tiles1 + tiles2, 128, dcol_smem(C1, D.n1), a, c->tw);
+    const size_t sh = smem(D.n1) > smem(D.n2) ? smem(D.n1) : smem(D.n2);
+    launch3(c, wide ? k3_d12<true> : k3_d12<false>, a.tiles1 + tiles2, 128, sh, a, c->tw);
 }
 
 // row kernels: 128 threads a block (64 for small boxes), at most the box's pairs of rows

@@ -1,6 +1,7 @@
 """Three-dimensional transport through axis-wise derivatives (csrc/deriv.cuh, csrc/reg3d.cu) at the
 sizes where its launch rules change: the smallest box, one column block per axis; the box sizes at
-which the column and row blocks grow (2^17, 2^18, 2^20 points); columns shorter than a block.
+which the column and row blocks grow (2^17, 2^18, 2^20 points) and axes of 128 and 256 points take 16 entries a thread; columns
+shorter than a block.
 
 Tolerance as in test_gpu_reg3d: max(1, c) (2e-5 + 2 u (n / 2) log2(n)), n the longest axis, c the
 conditioning of the sums g and H v~."""
@@ -26,7 +27,7 @@ def _cuda():
 
 @pytest.mark.parametrize("shape,nt,beta_w", [
     ((8, 8, 8), 1, math.inf), ((8, 16, 8), 2, 0.0), ((64, 64, 32), 1, 1e-3), ((32, 64, 128), 1, math.inf),
-    ((64, 128, 128), 1, 1e-3),
+    ((64, 128, 128), 1, 1e-3), ((256, 128, 32), 1, math.inf),
 ])
 def test_block_size_edges_match_oracle(shape, nt, beta_w):
     import torch
