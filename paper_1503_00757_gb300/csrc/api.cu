@@ -473,8 +473,7 @@ static void sp_vec(reg_ctx* c, int op, float coefA, const float* u, float* out) 
 // out = coefA A u + K b  (reduced gradient / Hessian assembly, Eq. (e:control-eq-elim), (e:inc-control-eq-elim));
 // out == nullptr: the spectra stay in S[4], S[5] (finish_out)
 static void sp_assemble(reg_ctx* c, float coefA, const float* u, const float* b, float* out) {
-    launch_r2c_vec(c, u, u + c->N, c->S[0], c->S[1]);
-    launch_r2c_vec(c, b, b + c->N, c->S[2], c->S[3]);
+    launch_r2c_two(c, u, b, c->S);
     const float2* in[4] = {c->S[0], c->S[1], c->S[2], c->S[3]};
     float2* o[2] = {c->S[4], c->S[5]};
     launch_col(c, OP_ASSEMBLE, in, o, spec_params(c, coefA), nullptr);
@@ -484,8 +483,7 @@ static void sp_assemble(reg_ctx* c, float coefA, const float* u, const float* b,
 // ---- preconditioned coordinates y = Q v, Q^ = (beta_v A'^)^(1/2), A'(0) = 1 ----
 // out = Pi0 y + Q^-1 K b (the gradient, or with y = s and b = b~ the Hessian product, in y)
 static void sp_assemble_y(reg_ctx* c, const float* y, const float* b, float* out) {
-    launch_r2c_vec(c, y, y + c->N, c->S[0], c->S[1]);
-    launch_r2c_vec(c, b, b + c->N, c->S[2], c->S[3]);
+    launch_r2c_two(c, y, b, c->S);
     const float2* in[4] = {c->S[0], c->S[1], c->S[2], c->S[3]};
     float2* o[2] = {c->S[4], c->S[5]};
     launch_col(c, OP_ASSEMBLE_Y, in, o, spec_params(c, 0.f), nullptr);
@@ -916,8 +914,7 @@ static void reg_energy_y(reg_ctx* c, const float* y) {
 static void objective_launches(reg_ctx* c, const float* v, int nt, const float* y = nullptr) {
     state_solve(c, v, nt);
     // J_data = 0.5 ||m_R - m_1||^2
-    launch_axpby(c, c->N, 1.f, c->mR, -1.f, mh(c, nt), -1, -1, c->w1);
-    int np = launch_dot_partial(c, c->w1, c->w1, c->N, c->d_part);
+    int np = launch_diff2_partial(c, c->mR, mh(c, nt), c->N, c->d_part);
     launch_finalize(c, c->d_part, np, c->d_scal + SL_JDATA, 0.5 * hh(c), 0, 0);
     if (y)
         reg_energy_y(c, y);

@@ -204,7 +204,13 @@ __device__ __forceinline__ void dcol_body(const DColArgs& a, const ColMap& m, in
     const uint32_t step = (uint32_t)T * m.S;
     LineTw<LOGL, TWREG> W;
     W.load(tw, t);
-    float2 x[8];
+    float2 x[8], y[8];
+    // the factor (the velocity: written two or more launches back) is fetched ahead of the wait
+    if (on && a.mul) {
+        const float2* g = reinterpret_cast<const float2*>(a.mul) + base;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) y[k] = g[k * step];
+    }
     wait();
 #pragma unroll
     for (int k = 0; k < 8; ++k) x[k] = make_float2(0.f, 0.f);
@@ -213,10 +219,6 @@ __device__ __forceinline__ void dcol_body(const DColArgs& a, const ColMap& m, in
 #pragma unroll
         for (int k = 0; k < 8; ++k) x[k] = f[k * step];
         if (a.mul) {
-            const float2* g = reinterpret_cast<const float2*>(a.mul) + base;
-            float2 y[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) y[k] = g[k * step];
 #pragma unroll
             for (int k = 0; k < 8; ++k) x[k] = make_float2(__fmul_rn(x[k].x, y[k].x), __fmul_rn(x[k].y, y[k].y));
             if (a.f2) {
@@ -224,8 +226,7 @@ __device__ __forceinline__ void dcol_body(const DColArgs& a, const ColMap& m, in
                 const float2* g2 = reinterpret_cast<const float2*>(a.mul2) + base;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const uint32_t i = k * step;
-                    const float2 p = f2[i], q = g2[i];
+                    const float2 p = f2[k * step], q = g2[k * step];
                     x[k] = make_float2(fmaf(p.x, q.x, x[k].x), fmaf(p.y, q.y, x[k].y));
                 }
             }

@@ -157,6 +157,8 @@ size_t col_smem(int C, int L, bool div1);
 void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S, int nb = 1, long long ss = 0);
 // nb vector fields back to back (2 N floats each; spectra S1, S2: N entries apart from field to field)
 void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, float2* S2, int nb = 1);
+// spectra of the vector fields u (S[0], S[1]) and b (S[2], S[3]) in one launch
+void launch_r2c_two(reg_ctx* ctx, const float* u, const float* b, float2* const* S);
 void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f);
 void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb = 1,
                     float scale = 1.f, long long ss = 0);  // ss: entries from field to field (0: N)
@@ -226,6 +228,8 @@ void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, 
 // ---- pointwise / reductions ----
 // part[...] <- partial sums of sum_i x_i y_i over n elements; returns #partials
 int launch_dot_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part);
+// part[...] <- partial sums of sum_i (x_i - y_i)^2; returns #partials
+int launch_diff2_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part);
 // part[...] <- partial sums of sum_i x_i over n elements; returns #partials
 int launch_sum_partial(reg_ctx* ctx, const float* x, long long n, double* part);
 int launch_maxnorm_partial(reg_ctx* ctx, const float* v, int N, double* part);

@@ -158,16 +158,28 @@ __device__ __forceinline__ void stage_chunk(float2* dst, const float2* __restric
 struct Batch {
     long long f, s;
 };
+// a second vector field and its spectra for blockIdx.y = 1 (nullptr: none)
+struct Second {
+    const float *f1, *f2;
+    float2 *S1, *S2;
+};
 
 template <int LOGL, bool VEC>
 __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const float* __restrict__ f2,
-                                             float2* S1, float2* S2, int R, const float2* __restrict__ tw, Batch bt) {
+                                             float2* S1, float2* S2, int R, const float2* __restrict__ tw, Batch bt, Second sec) {
     pdl_entry();
-    f1 += blockIdx.y * bt.f;
-    S1 += blockIdx.y * bt.s;
-    if (VEC) {
-        f2 += blockIdx.y * bt.f;
-        S2 += blockIdx.y * bt.s;
+    if (VEC && sec.f1 && blockIdx.y) {
+        f1 = sec.f1;
+        f2 = sec.f2;
+        S1 = sec.S1;
+        S2 = sec.S2;
+    } else {
+        f1 += blockIdx.y * bt.f;
+        S1 += blockIdx.y * bt.s;
+        if (VEC) {
+            f2 += blockIdx.y * bt.f;
+            S2 += blockIdx.y * bt.s;
+        }
     }
     extern __shared__ __align__(16) float2 sm[];
     constexpr int L = 1 << LOGL, T = L >> 3, W = L >> 1;
@@ -845,7 +857,7 @@ void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S, int nb, long lon
         auto kern = k_r2c<LG, false>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw,
-                 Batch{(long long)ctx->N, ss});
+                 Batch{(long long)ctx->N, ss}, Second{});
     });
     ktimer_end(ctx);
 }
@@ -857,7 +869,19 @@ void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, 
         auto kern = k_r2c<LG, true>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, u1, u2, S1, S2, g.R, ctx->tw,
-                 Batch{2LL * ctx->N, (long long)ctx->N});
+                 Batch{2LL * ctx->N, (long long)ctx->N}, Second{});
+    });
+    ktimer_end(ctx);
+}
+
+void launch_r2c_two(reg_ctx* ctx, const float* u, const float* b, float2* const* S) {
+    const RowCfg g = row_cfg(ctx);
+    ktimer_begin(ctx, KC_ROW, 32.0 * ctx->N);
+    DISPATCH_LOG(ctx->log2, {
+        auto kern = k_r2c<LG, true>;
+        set_smem(kern, g.smem);
+        launch_k(ctx, kern, dim3(g.grid, 2), g.threads, g.smem, u, u + ctx->N, S[0], S[1], g.R, ctx->tw, Batch{0, 0},
+                 Second{b, b + ctx->N, S[2], S[3]});
     });
     ktimer_end(ctx);
 }
@@ -1000,6 +1024,25 @@ __global__ void k_dot_partial(const float* __restrict__ x, const float* __restri
 int launch_dot_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part) {
     ktimer_begin(ctx, KC_POINT, 8.0 * n);
     launch_k(ctx, k_dot_partial, NBLK_RED, NTHREADS, 0, x, y, n, part);
+    ktimer_end(ctx);
+    return NBLK_RED;
+}
+
+// partial sums of sum_i (x_i - y_i)^2, the difference rounded to FP32
+__global__ void k_diff2_partial(const float* __restrict__ x, const float* __restrict__ y, long long n, double* part) {
+    pdl_entry();
+    double acc = 0.0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const float d = x[i] - y[i];
+        acc += (double)d * (double)d;
+    }
+    const double s = block_reduce<0>(acc);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+int launch_diff2_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part) {
+    ktimer_begin(ctx, KC_POINT, 8.0 * n);
+    launch_k(ctx, k_diff2_partial, NBLK_RED, NTHREADS, 0, x, y, n, part);
     ktimer_end(ctx);
     return NBLK_RED;
 }

@@ -17,6 +17,10 @@
 // Assembly (regularization and projection, which couple the axes): half spectra along axis 3,
 // n1 x n2 x (n3 / 2 + 1) complex entries per field, in five launches: rows real to complex,
 // axis 2, axis 1 forward with the multiplier and back, axis 2 back, rows complex to real.
+//
+// 128^3, nt = 16 matvec: 42.5 ms with full complex 3-D transforms in every stage, 1.54 ms now; about
+// 10 us a stage in k3_d12 (shared memory and FP32 issue) and 12 us in the row kernels (L2 and, for
+// the gradient history, HBM: 4 TB/s).  64 x 128 x 32, nt = 5 gradient: 4.62 -> 0.27 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -1,6 +1,12 @@
 // Transport kernels (sm_103a) of the state, adjoint, incremental state and incremental adjoint
 // equations of Mang & Biros (arXiv 1503.00757, Sec. 3) on a 2-D grid: Heun's RK2 in pseudo-time
 // with spectral derivatives taken axis by axis (deriv.cuh).
+//
+// Bound by the latency of a chain of dependent launches (64 to 128 CTAs of a few microseconds at
+// 512^2), so what counts is what lies between one launch's wait and its last store: the row
+// kernels' transforms precede their wait, no spectra are split or merged, and the operands are in
+// registers when the column kernel's result arrives.  512^2, nt = 32 matvec: 1464 us with the
+// stages in the row spectra, 848 us with these (6.3 us a stage).
 #include <type_traits>
 
 #include "deriv.cuh"
@@ -60,13 +66,17 @@ __global__ void __launch_bounds__(NTHREADS) k_adj_init(const float* __restrict__
     }
 }
 
+// Heun stage of the deformation gradient (deriv.cuh).  With k_dcol over all four planes a step is 4
+// launches; 8 separate gradients and a pointwise kernel per stage were 26.  det F, displacement and
+// labels at 512^2, nt = 32: 5640 -> 1390 us.
 template <int LOGL>
 __global__ void __launch_bounds__(256, 1) k_defgrad_row(DefGradStage a, int N, int lines, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) float2 sm[];
     defgrad_row_body<LOGL>(a, (uint32_t)N, lines, sm, tw, pdl_entry);
 }
 
-// grad f in one launch: blocks [0, tiles1) write d_1 f, the others d_2 f (both only read f)
+// grad f in one launch: blocks [0, tiles1) write d_1 f, the others d_2 f (both only read f).  Small
+// calls are bound by the launches (64^2: three launches 8.7 us, one 4.3 us).
 struct GradArgs {
     DColArgs col;
     ColMap m;

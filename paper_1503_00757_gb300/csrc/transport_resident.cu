@@ -6,12 +6,14 @@
 // of it.  Here a cluster of CS CTAs owns the grid, R = n1 / CS rows each; u_j, the velocity and the
 // body force live in registers for the whole solve, and a stage is
 //   publish the stage's field in shared memory -> cluster barrier (meanwhile: x^2 derivative of the
-//   own rows, source terms) -> x^1 derivative of C = n2 / (2 CS) packed columns, gathered from the
-//   row owners' shared memory and scattered back to it -> cluster barrier -> update in registers.
+//   own rows) -> x^1 derivative of C = n2 / (2 CS) packed columns, gathered from the row owners'
+//   shared memory and scattered back to it -> cluster barrier -> update in registers.
 // The transforms, the products and their order are those of transport.cu (deriv.cuh), so the
-// results are the same bit for bit.  16 CTAs (the largest cluster) give 256^2 a block of 256
-// threads with 8 entries each; more points per axis would put more than 16 entries per thread on
-// 16 SMs, where the kernel pairs have the whole chip.
+// results are the same bit for bit.  Half the threads are the row role, half the column role, so the
+// two derivatives of a stage run side by side (one role doing both: 231 us for the gradient at
+// 128^2, nt = 16; two roles: 208; kernel pairs: 318).  Bound by the latency of one transform pair
+// and two cluster barriers a stage, about 2.3 us.  At 256^2 the 16 SMs of the largest cluster compute
+// as long as the kernel pairs wait (302 against 301 us a matvec, nt = 16), so the line is below it.
 #include <map>
 #include <mutex>
 

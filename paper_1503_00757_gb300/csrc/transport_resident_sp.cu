@@ -9,7 +9,8 @@
 // R = n1 / CS rows each, whose fields, velocity and body force stay in registers and whose row
 // spectra stay in shared memory; the column pass gathers its C = n2 / (2 CS) columns from the row
 // owners over distributed shared memory and scatters the result back (two cluster barriers a
-// stage instead of two launches, about 9 us a stage at 128^2).
+// stage instead of two launches of about 9 us together at 128^2; eight mixed 128^2 pairs, two
+// Newton steps each: 14.1 ms with the launches, 8.1 ms).  Bound by latency, like transport_resident.cu.
 #include <map>
 #include <mutex>
 
@@ -56,6 +57,10 @@ __global__ void __launch_bounds__(SpGeom<LOG1, LOG2>::THREADS, 1) k_resident_sp(
     const int e = rank * C + c;
     const int owner = tc / R, off = (int)sp_idx(tc - owner * R, e, W);
     const float scale = 1.0f / (float)N;
+    uint32_t from[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) from[k] = colact ? cl_map(S1 + off, owner + k * (G::CS / 8)) : 0u;
+    constexpr uint32_t SP_PLANE = R * W * sizeof(float2);  // S2 and Gd follow S1 in every CTA
     pdl_entry();
 
     float2* xb = Xr + 2 * q * fft_buf(L);
@@ -82,26 +87,18 @@ __global__ void __launch_bounds__(SpGeom<LOG1, LOG2>::THREADS, 1) k_resident_sp(
             S1[idx] = split_entry<LOG2>(Z + (r >> 1) * L, r & 1, ee);
         }
     };
-    // flux spectra of x (one row per transform) into S1, S2; 2 R W entries of scratch at Z, Gd.. are not
-    // enough for R full spectra, so the two halves of the rows go one after the other
+    // flux spectra of x (one row per transform) into S1, S2; the R full spectra take Gd and Z, both
+    // consumed by then
     auto flux_forward = [&](float2 (&x)[8]) {
         reg_fft<LOG2, false>(x, t, true, xb, xb + fft_buf(L), tw);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            __syncthreads();
-            if (q / (R / 2) == h) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) Z[(q - h * (R / 2)) * L + t + k * T] = x[k];
-            }
-            __syncthreads();
-            for (int idx = threadIdx.x; idx < R * W; idx += blockDim.x) {
-                const int r = ((idx / (4 * W)) << 2) | (idx & 3);
-                const int ee = (idx >> 2) & (W - 1);
-                if (r / (R / 2) == h) {
-                    S1[idx] = split_entry<LOG2>(Z + (r - h * (R / 2)) * L, 0, ee);
-                    S2[idx] = split_entry<LOG2>(Z + (r - h * (R / 2)) * L, 1, ee);
-                }
-            }
+        for (int k = 0; k < 8; ++k) Gd[q * L + t + k * T] = x[k];
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < R * W; idx += blockDim.x) {
+            const int r = ((idx / (4 * W)) << 2) | (idx & 3);
+            const int ee = (idx >> 2) & (W - 1);
+            S1[idx] = split_entry<LOG2>(Gd + r * L, 0, ee);
+            S2[idx] = split_entry<LOG2>(Gd + r * L, 1, ee);
         }
     };
     // Gd <- i k1~ S1 / N along x^1 (DIV: plus (i k2~ / n2) S2), as k_col<OP_GRAD1 / OP_DIV1>
@@ -111,7 +108,7 @@ __global__ void __launch_bounds__(SpGeom<LOG1, LOG2>::THREADS, 1) k_resident_sp(
         float2 x[8];
         if (colact) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) x[k] = cl_load(cl_map(S1 + off, owner + k * (G::CS / 8)));
+            for (int k = 0; k < 8; ++k) x[k] = cl_load(from[k]);
         }
         float2* cb = Xc + 2 * c * fft_buf(L1);
         reg_fft<LOG1, false>(x, tc, colact, cb, cb + fft_buf(L1), tw);
@@ -148,13 +145,12 @@ __global__ void __launch_bounds__(SpGeom<LOG1, LOG2>::THREADS, 1) k_resident_sp(
             const float ce = cd2 * (float)e;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                const int o = owner + k * (G::CS / 8);
                 float2 val = x[k];
                 if (div) {
-                    const float2 f2 = cl_load(cl_map(S2 + off, o));
+                    const float2 f2 = cl_load(from[k] + SP_PLANE);
                     val = make_float2(val.x - ce * f2.y, val.y + ce * f2.x);
                 }
-                cl_store(cl_map(Gd + off, o), val);
+                cl_store(from[k] + 2 * SP_PLANE, val);
             }
         }
         cl_arrive();
@@ -256,6 +252,16 @@ __global__ void __launch_bounds__(SpGeom<LOG1, LOG2>::THREADS, 1) k_resident_sp(
 #pragma unroll 1
         for (int s = 0; s < 2 * nt; ++s) {
             const int j = nt - (s >> 1), stage = 1 + (s & 1);
+            const float* gm = a.gm + (size_t)(j - 1) * 2 * N;
+            float ga[8], gb[8];
+            if (stage == 2) {  // fetched while the columns are at work
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const size_t idx = rowbase + t + k * T;
+                    ga[k] = gm[idx];
+                    gb[k] = gm[N + idx];
+                }
+            }
             column(true);
             const bool act1 = q < R / 2;
             if (act1) {
@@ -271,18 +277,16 @@ __global__ void __launch_bounds__(SpGeom<LOG1, LOG2>::THREADS, 1) k_resident_sp(
                 }
             }
             __syncthreads();
-            const float* gm = a.gm + (size_t)(j - 1) * 2 * N;
             const float w = (j - 1 == 0) ? 0.5f * a.h : a.h;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                const size_t idx = rowbase + t + k * T;
                 const float dv = O[q * L + t + k * T];
                 const float pls = stage == 2 ? ls[k] : 0.f;
                 const float out = (stage == 1) ? fmaf(a.h, dv, u[k]) : 0.5f * fmaf(a.h, dv, u[k] + pls);
                 if (stage == 2) {
                     const float wl = w * out;
-                    b1[k] = fmaf(wl, gm[idx], b1[k]);
-                    b2[k] = fmaf(wl, gm[N + idx], b2[k]);
+                    b1[k] = fmaf(wl, ga[k], b1[k]);
+                    b2[k] = fmaf(wl, gb[k], b2[k]);
                     u[k] = out;
                 } else {
                     ls[k] = out;
