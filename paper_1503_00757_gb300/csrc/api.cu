@@ -8,6 +8,8 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
+#include <utility>
+#include <vector>
 
 #include "deriv.cuh"
 #include "fft.cuh"
@@ -110,18 +112,11 @@ static int alloc_hist(reg_ctx* c, int nt) {
 
 extern "C" void reg_destroy(reg_ctx* c) {
     if (!c) return;
-    float** fl[] = {&c->mT, &c->mR, &c->v_lin, &c->E_lin, &c->eta_lin, &c->w0, &c->w1, &c->w2, &c->w3,
-                    &c->bvec, &c->vtmp, &c->vtmp2, &c->gtmp, &c->T3, &c->T3b, &c->vx, &c->g, &c->r, &c->z, &c->s, &c->Hs,
-                    &c->vt, &c->vtrial, &c->F, &c->Fs, &c->gF, &c->gv, &c->ybuf, &c->ytrial, &c->vtil};
-    for (auto p : fl) cudaFree(*p);
-    cudaFree(c->S[0]);
     free_hist(c);
     clear_graphs(c);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (auto g : c->timing_graphs) cudaGraphExecDestroy(g);
-    cudaFree(c->d_scal);
-    cudaFree(c->d_part);
-    cudaFree(c->tw);
+    cudaFree(c->slab);
     cudaFreeHost(c->h_scal);
     for (auto e : c->event_pool) cudaEventDestroy(e);
     delete c;
@@ -192,8 +187,14 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     for (int k = 0; k < KC_COUNT; ++k) { c->tcount[k] = 0; c->tms[k] = 0.0; c->tbytes[k] = 0.0; }
 
     const size_t N = c->N;
-    bool ok = true;
-    auto A = [&](float** p, size_t n) { if (ok && cudaMalloc(p, sizeof(float) * n) != cudaSuccess) ok = false; };
+    // the fixed-size workspace is one allocation (some 35 cudaMalloc calls were most of reg_create)
+    size_t used = 0;
+    std::vector<std::pair<void**, size_t>> parts;
+    auto take = [&](void** p, size_t bytes) {
+        parts.emplace_back(p, used);
+        used += (bytes + 255) & ~(size_t)255;
+    };
+    auto A = [&](float** p, size_t n) { take((void**)p, sizeof(float) * n); };
     A(&c->mT, N); A(&c->mR, N); A(&c->v_lin, 2 * N); A(&c->E_lin, 3 * N); A(&c->eta_lin, N);
     A(&c->w0, N); A(&c->w1, N); A(&c->w2, N); A(&c->w3, N);
     A(&c->bvec, 2 * N); A(&c->vtmp, 2 * N); A(&c->vtmp2, 2 * N); A(&c->gtmp, 4 * N); A(&c->T3, 3 * N);
@@ -202,12 +203,16 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     A(&c->vt, 2 * N); A(&c->vtrial, 2 * N);
     A(&c->ybuf, 2 * N); A(&c->ytrial, 2 * N); A(&c->vtil, 2 * N);
     A(&c->F, 4 * N); A(&c->Fs, 4 * N); A(&c->gF, 8 * N); A(&c->gv, 4 * N);
-    if (ok && cudaMalloc(&c->S[0], sizeof(float2) * 6 * (N / 2)) != cudaSuccess) ok = false;
-    for (int i = 1; i < 6 && ok; ++i) c->S[i] = c->S[0] + i * (N / 2);  // one block: batched passes stride through it
     c->npart = 5 * 304 + 4096;
-    if (ok && cudaMalloc(&c->d_scal, sizeof(double) * SL_COUNT) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc(&c->d_part, sizeof(double) * c->npart) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc(&c->tw, sizeof(float2) * REG_TW_TOTAL) != cudaSuccess) ok = false;
+    take((void**)&c->S[0], sizeof(float2) * 6 * (N / 2));
+    take((void**)&c->d_scal, sizeof(double) * (SL_COUNT + 1));
+    take((void**)&c->d_part, sizeof(double) * c->npart);
+    take((void**)&c->tw, sizeof(float2) * REG_TW_TOTAL);
+    bool ok = cudaMalloc(&c->slab, used) == cudaSuccess;
+    if (ok) {
+        for (auto& q : parts) *q.first = static_cast<char*>(c->slab) + q.second;
+        for (int i = 1; i < 6; ++i) c->S[i] = c->S[0] + i * (N / 2);  // one block: batched passes stride through it
+    }
     if (ok && cudaMallocHost(&c->h_scal, sizeof(double) * SL_COUNT) != cudaSuccess) ok = false;
     if (!ok) {
         cudaGetLastError();
@@ -223,6 +228,7 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
         reg_destroy(c);
         return st;
     }
+    cudaMemset(c->d_scal + SL_COUNT, 0, sizeof(double));  // the reductions' block counter
     cudaMemset(c->mT, 0, sizeof(float) * N);
     cudaMemset(c->mR, 0, sizeof(float) * N);
     {
@@ -914,8 +920,7 @@ static void reg_energy_y(reg_ctx* c, const float* y) {
 static void objective_launches(reg_ctx* c, const float* v, int nt, const float* y = nullptr) {
     state_solve(c, v, nt);
     // J_data = 0.5 ||m_R - m_1||^2
-    int np = launch_diff2_partial(c, c->mR, mh(c, nt), c->N, c->d_part);
-    launch_finalize(c, c->d_part, np, c->d_scal + SL_JDATA, 0.5 * hh(c), 0, 0);
+    launch_diff2(c, c->mR, mh(c, nt), c->N, SL_JDATA, 0.5 * hh(c));
     if (y)
         reg_energy_y(c, y);
     else
@@ -1171,8 +1176,7 @@ extern "C" int reg_hessian_matvec(reg_ctx* c, const float* vt, float* Hvt) {
 // Newton-Krylov solve (Algorithm 1) with PCG (Algorithm 2)
 // ---------------------------------------------------------------------------
 static int dot_dev(reg_ctx* c, const float* x, const float* y, int slot) {
-    int np = launch_dot_partial(c, x, y, 2 * (long long)c->N, c->d_part);
-    launch_finalize(c, c->d_part, np, c->d_scal + slot, hh(c), 0, 0);
+    launch_dot(c, x, y, 2 * (long long)c->N, slot, hh(c));
     return REG_OK;
 }
 
@@ -1230,13 +1234,12 @@ static int pcg_dev(reg_ctx* c, double gnorm, double eta, int maxit, int* hit_max
             else
                 matvec_launches(c, c->s, c->Hs);
             dot_dev(c, c->s, c->Hs, SL_SHS);
-            int np = launch_pcg_update(c, n2N, c->vt, c->s, c->r, c->Hs, c->d_part);
+            launch_pcg_update(c, n2N, c->vt, c->s, c->r, c->Hs, yp ? -1 : SL_RNORM2, scale);
             if (yp) {
                 sp_qnorm(c, c->r, SL_RNORM2);
                 dot_dev(c, c->r, c->r, SL_RZNEW);
                 launch_pcg_dir(c, n2N, c->r, c->s);
             } else {
-                launch_finalize(c, c->d_part, np, c->d_scal + SL_RNORM2, scale, 0, 0);
                 precond_dev(c, c->r, c->z);
                 dot_dev(c, c->z, c->r, SL_RZNEW);
                 launch_pcg_dir(c, n2N, c->z, c->s);
@@ -1398,11 +1401,7 @@ extern "C" int reg_solve(reg_ctx* c, float* v, const reg_solve_opts* opts, reg_s
         if (!std::isfinite(J) || !std::isfinite(gnorm)) status = REG_ERR_NAN;
     }
     // mismatch measure (Appendix F): ||m_R - m_1||^2 / ||m_R - m_T||^2
-    launch_axpby(c, c->N, 1.f, c->mR, -1.f, c->mT, -1, -1, c->w0);
-    {
-        int np = launch_dot_partial(c, c->w0, c->w0, c->N, c->d_part);
-        launch_finalize(c, c->d_part, np, c->d_scal + SL_DOT0, hh(c), 0, 0);
-    }
+    launch_diff2(c, c->mR, c->mT, c->N, SL_DOT0, hh(c));
     RET(read_scalars(c));
     const double r0 = c->h_scal[SL_DOT0];
     const double r1 = 2.0 * c->h_scal[SL_JDATA];

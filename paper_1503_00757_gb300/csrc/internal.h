@@ -80,6 +80,7 @@ struct reg_ctx {
     cudaStream_t stream;
     cudaStream_t cap;  // launch sequences are captured here when `stream` is the legacy default stream
 
+    void* slab;  // the allocation behind every buffer below but the histories and h_scal
     // images and history
     float *mT, *mR;
     float *m_hist;   // (nt_cap + 1) * N
@@ -106,7 +107,7 @@ struct reg_ctx {
     // det F workspace
     float *F, *Fs, *gF, *gv;  // 4N, 4N, 8N (F of the next step, D), 4N
 
-    double* d_scal;  // SL_COUNT
+    double* d_scal;  // SL_COUNT, then the block counter of the reductions
     double* d_part;  // partial sums
     int npart;
     double* h_scal;  // pinned host mirror
@@ -226,10 +227,9 @@ void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, 
                      const float* lsrc = nullptr, const float* vt = nullptr, const float* gmt = nullptr);
 
 // ---- pointwise / reductions ----
-// part[...] <- partial sums of sum_i x_i y_i over n elements; returns #partials
-int launch_dot_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part);
-// part[...] <- partial sums of sum_i (x_i - y_i)^2; returns #partials
-int launch_diff2_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part);
+// d_scal[slot] = scale * sum_i x_i y_i over n elements; the same of (x_i - y_i)^2
+void launch_dot(reg_ctx* ctx, const float* x, const float* y, long long n, int slot, double scale);
+void launch_diff2(reg_ctx* ctx, const float* x, const float* y, long long n, int slot, double scale);
 // part[...] <- partial sums of sum_i x_i over n elements; returns #partials
 int launch_sum_partial(reg_ctx* ctx, const float* x, long long n, double* part);
 int launch_maxnorm_partial(reg_ctx* ctx, const float* v, int N, double* part);
@@ -238,9 +238,10 @@ void launch_finalize(reg_ctx* ctx, const double* part, int np, double* out, doub
 // y = a * x + b * y, with optional device-scalar factor: if (num >= 0) a *= d_scal[num] / d_scal[den]
 void launch_axpby(reg_ctx* ctx, long long n, float a, const float* x, float b, float* y, int num, int den,
                   float* out);
-// PCG step: vt += kappa s; r -= kappa Hs; partial sum r^2; kappa = d_scal[SL_RZ] / d_scal[SL_SHS];
+// PCG step: vt += kappa s; r -= kappa Hs; d_scal[slot] = scale * sum r^2 (slot < 0: not taken); kappa = d_scal[SL_RZ] / d_scal[SL_SHS];
 // no update when d_scal[SL_SHS] <= 0
-int launch_pcg_update(reg_ctx* ctx, long long n, float* vt, const float* s, float* r, const float* Hs, double* part);
+void launch_pcg_update(reg_ctx* ctx, long long n, float* vt, const float* s, float* r, const float* Hs, int slot,
+                       double scale);
 // s = z + (d_scal[SL_RZNEW] / d_scal[SL_RZ]) s
 void launch_pcg_dir(reg_ctx* ctx, long long n, const float* z, float* s);
 void launch_fill(reg_ctx* ctx, long long n, float* y, float val);

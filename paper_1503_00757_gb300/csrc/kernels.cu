@@ -1012,39 +1012,66 @@ void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* ou
 // ---------------------------------------------------------------------------
 // pointwise and reduction kernels
 // ---------------------------------------------------------------------------
-__global__ void k_dot_partial(const float* __restrict__ x, const float* __restrict__ y, long long n, double* part) {
+// The last block to finish sums the blocks' partials in k_finalize's order (the same result as that
+// launch of its own, about 2 us less on the chain): out = scale * sum.  The counter wraps to 0 by
+// itself.  out == nullptr: partials only.
+struct Total {
+    double* out;
+    double scale;
+    unsigned* counter;
+};
+__device__ __forceinline__ void block_total(double s, double* part, const Total& t) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = s;
+        last = false;
+        if (t.out) {
+            __threadfence();
+            last = atomicInc(t.counter, gridDim.x - 1) == gridDim.x - 1;
+        }
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) acc += __ldcg(part + i);
+    const double sum = block_reduce<0>(acc);
+    if (threadIdx.x == 0) *t.out = t.scale * sum;
+}
+static Total total(reg_ctx* ctx, int slot, double scale) {
+    return Total{slot >= 0 ? ctx->d_scal + slot : nullptr, scale, reinterpret_cast<unsigned*>(ctx->d_scal + SL_COUNT)};
+}
+
+__global__ void k_dot_partial(const float* __restrict__ x, const float* __restrict__ y, long long n, double* part,
+                              Total tot) {
     pdl_entry();
     double acc = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         acc += (double)x[i] * (double)y[i];
-    const double s = block_reduce<0>(acc);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    block_total(block_reduce<0>(acc), part, tot);
 }
 
-int launch_dot_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part) {
+void launch_dot(reg_ctx* ctx, const float* x, const float* y, long long n, int slot, double scale) {
     ktimer_begin(ctx, KC_POINT, 8.0 * n);
-    launch_k(ctx, k_dot_partial, NBLK_RED, NTHREADS, 0, x, y, n, part);
+    launch_k(ctx, k_dot_partial, NBLK_RED, NTHREADS, 0, x, y, n, ctx->d_part, total(ctx, slot, scale));
     ktimer_end(ctx);
-    return NBLK_RED;
 }
 
-// partial sums of sum_i (x_i - y_i)^2, the difference rounded to FP32
-__global__ void k_diff2_partial(const float* __restrict__ x, const float* __restrict__ y, long long n, double* part) {
+// sum_i (x_i - y_i)^2, the difference rounded to FP32
+__global__ void k_diff2(const float* __restrict__ x, const float* __restrict__ y, long long n, double* part, Total tot) {
     pdl_entry();
     double acc = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float d = x[i] - y[i];
         acc += (double)d * (double)d;
     }
-    const double s = block_reduce<0>(acc);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    block_total(block_reduce<0>(acc), part, tot);
 }
 
-int launch_diff2_partial(reg_ctx* ctx, const float* x, const float* y, long long n, double* part) {
+void launch_diff2(reg_ctx* ctx, const float* x, const float* y, long long n, int slot, double scale) {
     ktimer_begin(ctx, KC_POINT, 8.0 * n);
-    launch_k(ctx, k_diff2_partial, NBLK_RED, NTHREADS, 0, x, y, n, part);
+    launch_k(ctx, k_diff2, NBLK_RED, NTHREADS, 0, x, y, n, ctx->d_part, total(ctx, slot, scale));
     ktimer_end(ctx);
-    return NBLK_RED;
 }
 
 __global__ void k_sum_partial(const float* __restrict__ x, long long n, double* part) {
@@ -1117,30 +1144,27 @@ void launch_axpby(reg_ctx* ctx, long long n, float a, const float* x, float b, f
 }
 
 __global__ void k_pcg_update(long long n, float* vt, const float* __restrict__ s, float* r, const float* __restrict__ Hs,
-                             const double* __restrict__ scal, double* part) {
+                             const double* scal, double* part, Total tot) {
     pdl_entry();
     const double shs = scal[SL_SHS];
     const float kappa = (float)(scal[SL_RZ] / shs);
     double acc = 0.0;
-    if (!(shs > 0.0)) {  // non-positive curvature: leave vt and r unchanged (the host stops PCG)
-        if (threadIdx.x == 0) part[blockIdx.x] = 0.0;
-        return;
-    }
+    if (!(shs > 0.0)) n = 0;  // non-positive curvature: leave vt and r unchanged (the host stops PCG)
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         vt[i] = fmaf(kappa, s[i], vt[i]);
         const float ri = fmaf(-kappa, Hs[i], r[i]);
         r[i] = ri;
         acc += (double)ri * (double)ri;
     }
-    const double t = block_reduce<0>(acc);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
+    block_total(block_reduce<0>(acc), part, tot);
 }
 
-int launch_pcg_update(reg_ctx* ctx, long long n, float* vt, const float* s, float* r, const float* Hs, double* part) {
+void launch_pcg_update(reg_ctx* ctx, long long n, float* vt, const float* s, float* r, const float* Hs, int slot,
+                       double scale) {
     ktimer_begin(ctx, KC_POINT, 4.0 * n * 6);
-    launch_k(ctx, k_pcg_update, NBLK_RED, NTHREADS, 0, n, vt, s, r, Hs, ctx->d_scal, part);
+    launch_k(ctx, k_pcg_update, NBLK_RED, NTHREADS, 0, n, vt, s, r, Hs, ctx->d_scal, ctx->d_part,
+             total(ctx, slot, scale));
     ktimer_end(ctx);
-    return NBLK_RED;
 }
 
 __global__ void k_pcg_dir(long long n, const float* __restrict__ z, float* s, const double* __restrict__ scal) {

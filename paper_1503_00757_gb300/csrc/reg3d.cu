@@ -26,6 +26,8 @@
 #include <cmath>
 #include <cstdint>
 #include <string>
+#include <utility>
+#include <vector>
 
 #include "deriv.cuh"
 #include "internal.h"
@@ -380,6 +382,7 @@ struct reg3_ctx {
     int kmode;  // 0: K = I (gamma = 0), 1: incompressible (gamma = inf), 2: mass source
     cudaStream_t stream;
     cudaStream_t cap;  // the stream the launch sequences are captured on (created on first use)
+    void* slab;  // the allocation behind the device buffers
     float *mT, *mR, *v, *vt, *gm, *y, *ys, *lam, *src, *D1, *D2, *bt;
     float2* S;   // six half spectra: 0..2 of b (and the results), 3..5 of v
     float2* tw;
@@ -648,9 +651,7 @@ extern "C" void reg3_destroy(reg3_ctx* c) {
     for (cudaGraphExec_t g : c->graphs)
         if (g) cudaGraphExecDestroy(g);
     if (c->cap) cudaStreamDestroy(c->cap);
-    void* ptrs[] = {c->mT, c->mR, c->v, c->vt, c->gm, c->y, c->ys, c->lam, c->src, c->D1, c->D2, c->bt,
-                    c->S, c->tw, c->d_part, c->d_sum};
-    for (void* p : ptrs) cudaFree(p);
+    cudaFree(c->slab);
     cudaFreeHost(c->h_sum);
     delete c;
 }
@@ -673,8 +674,13 @@ extern "C" int reg3_create(int n1, int n2, int n3, int nt, double beta, double g
     c->stream = 0;
     c->npart = R3_BLOCKS + col3(c->D.l1, n2 * c->D.W1).grid;
     const size_t N = (size_t)c->D.N;
-    bool ok = true;
-    auto M = [&](void** p, size_t bytes) { if (ok && cudaMalloc(p, bytes) != cudaSuccess) ok = false; };
+    // one allocation for all buffers
+    size_t used = 0;
+    std::vector<std::pair<void**, size_t>> parts;
+    auto M = [&](void** p, size_t bytes) {
+        parts.emplace_back(p, used);
+        used += (bytes + 255) & ~(size_t)255;
+    };
     M((void**)&c->mT, sizeof(float) * N);
     M((void**)&c->mR, sizeof(float) * N);
     M((void**)&c->v, sizeof(float) * 3 * N);
@@ -691,6 +697,9 @@ extern "C" int reg3_create(int n1, int n2, int n3, int nt, double beta, double g
     M((void**)&c->tw, sizeof(float2) * REG_TW_TOTAL);
     M((void**)&c->d_part, sizeof(double) * 3 * c->npart);
     M((void**)&c->d_sum, sizeof(double) * 3);
+    bool ok = cudaMalloc(&c->slab, used) == cudaSuccess;
+    if (ok)
+        for (auto& q : parts) *q.first = static_cast<char*>(c->slab) + q.second;
     if (ok && cudaMallocHost((void**)&c->h_sum, sizeof(double) * 3) != cudaSuccess) ok = false;
     if (!ok) {
         cudaGetLastError();
