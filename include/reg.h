@@ -297,14 +297,15 @@ int reg_set_tiles(reg_ctx* ctx, int rows_per_cta, int cols_per_cta, int prefetch
  *     the row spectra of the transported field in shared memory and exchange
  *     column slabs through distributed shared memory (square grids n x n,
  *     16 <= n <= 512, on devices with thread-block clusters);
- *   cluster == 0: a row kernel and a column kernel per Heun stage, the spectra
- *     passing through global memory (every grid).
- * Default: the two-kernel path (faster on a GB300 at every grid size and
- * concurrency measured: the cluster kernel keeps 16 warps per SM, too few to
- * hide the latency of its per-stage operand loads).  Results
- * agree to FP32 rounding (the transforms are the same; the order of a few
- * additions differs).  REG_ERR_ARG if cluster != 0 and this grid or device
- * cannot run it. */
+ *   cluster == 0: a row kernel and a column kernel per Heun stage (every grid).
+ * Default (until this call): grids of 64 to 256 points per axis with n1 n2 < 256^2 run every
+ * Gauss-Newton transport solve as one launch resident in a cluster of 8 or 16 CTAs, with the
+ * arithmetic of the kernel pairs (results equal bit for bit); larger and smaller grids, and full
+ * Newton, the kernel pairs.  H1 problems take derivatives axis by axis, H2 and H3 problems
+ * through the row spectra (their Krylov iteration amplifies a change of rounding, so they keep
+ * the arithmetic they have always had).  The cluster != 0 kernel agrees with either to FP32
+ * rounding (the order of a few additions differs) and is slower at every grid size and
+ * concurrency measured.  REG_ERR_ARG if cluster != 0 and this grid or device cannot run it. */
 int reg_set_transport(reg_ctx* ctx, int cluster);
 
 /* The transport path of a context: *cluster = 1 for the cluster-resident
@@ -509,7 +510,7 @@ int reg3_solve(reg3_ctx* ctx, float* v, double tol, int maxit_newton, int maxit_
  * every output written once) since the last enable (host pointers, each
  * nullable).  Classes: 0 column FFT + multiplier kernels, 1 row FFT + RK2
  * stage kernels (advection / adjoint), 2 other row FFT kernels,
- * 3 pointwise / reduction kernels, 4 cluster-resident transport kernels (one
+ * 3 pointwise / reduction kernels, 4 resident transport kernels (one
  * launch per transport solve, or per matvec for both of its solves). */
 int reg_kernel_timing(reg_ctx* ctx, int enable);
 int reg_kernel_time(reg_ctx* ctx, int kclass, long long* launches, double* ms, double* bytes);
