@@ -707,6 +707,9 @@ extern "C" int reg3_create(int n1, int n2, int n3, int nt, double beta, double g
         return reg_fail(REG_ERR_NOMEM, "3-D context allocation failed");
     }
     upload_twiddles(c->tw);
+    // A copy from pageable memory may return once its data is staged, and a working stream need not be
+    // ordered after the legacy stream (cudaStreamNonBlocking): wait until the table is on the device.
+    cudaStreamSynchronize(0);
     const int st = r3_err("3-D context set-up");
     if (st != REG_OK) {
         reg3_destroy(c);
