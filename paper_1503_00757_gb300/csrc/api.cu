@@ -332,6 +332,12 @@ enum GraphKind {
     GK_GRADIENT_Y = 7, GK_PCG_ITER_Y = 8, GK_PCG_INIT_Y = 9, GK_DISPLACEMENT = 10, GK_LABELS = 11
 };
 
+// whether the caller is capturing the working stream
+static bool capturing(const reg_ctx* c) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    return c->stream != 0 && cudaStreamIsCapturing(c->stream, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+
 template <typename F>
 static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt, F&& body) {
     if (c->timing && c->stream != 0) {
@@ -1449,8 +1455,9 @@ extern "C" int reg_displacement(reg_ctx* c, const float* v, float* u_out) {
     const int nt = c->nt;
     const size_t N = c->N;
     CK(cudaMemcpyAsync(c->vtil, v, sizeof(float) * 2 * N, cudaMemcpyDeviceToDevice, c->stream));
-    RET(run_seq(c, GK_DISPLACEMENT, nullptr, nullptr, nt,
-                [&] { displacement_solve(c, c->vtil, nt, c->vtmp, c->vx, c->gtmp); }));
+    auto body = [&] { displacement_solve(c, c->vtil, nt, c->vtmp, c->vx, c->gtmp); };
+    if (capturing(c)) body();  // into the graph the caller is capturing
+    else RET(run_seq(c, GK_DISPLACEMENT, nullptr, nullptr, nt, body));
     CK(cudaMemcpyAsync(u_out, c->vtmp, sizeof(float) * 2 * N, cudaMemcpyDeviceToDevice, c->stream));
     CKL();
     return REG_OK;
