@@ -65,6 +65,8 @@ extern "C" void reg_default_opts(reg_solve_opts* o) {
 // allocation
 // ---------------------------------------------------------------------------
 static void clear_graphs(reg_ctx* c) {
+    if (c->graphs.empty()) return;
+    const GraphCalls allow;
     for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);
     c->graphs.clear();
 }
@@ -369,6 +371,7 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
             return REG_OK;
         }
     }
+    const GraphCalls allow;
     const long long l0 = c->launches;
     const cudaStream_t user = c->stream;
     if (user == 0) {

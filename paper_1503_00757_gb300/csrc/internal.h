@@ -267,6 +267,17 @@ void ktimer_end(reg_ctx* ctx);
 
 int reg_fail(int status, const std::string& msg);
 
+// While it lives, this thread may instantiate and destroy graphs although another stream is being
+// captured (by any thread, in the default global mode): nothing here depends on captured work, and
+// without it the call would fail and invalidate that capture.
+struct GraphCalls {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    GraphCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~GraphCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    GraphCalls(const GraphCalls&) = delete;
+    GraphCalls& operator=(const GraphCalls&) = delete;
+};
+
 // out = scale exp(-a |k|^2) P_L b on the context's grid for nb velocity fields back to back (device):
 // the output map of the warm-start network (Gaussian low-pass, then Leray).  spec: nb N spectrum
 // entries of scratch.

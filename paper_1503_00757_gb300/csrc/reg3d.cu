@@ -616,6 +616,7 @@ int run3(reg3_ctx* c, int kind, F&& body) {
         return r3_err("launch");
     }
     if (!c->graphs[kind]) {
+        const GraphCalls allow;
         if (!c->cap && cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess)
             return r3_err("capture stream");
         if (cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed) != cudaSuccess) return r3_err("capture");

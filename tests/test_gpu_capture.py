@@ -52,3 +52,56 @@ def test_displacement_inside_a_callers_capture(regnorm, called_before):
     torch.cuda.synchronize()
     ctx.close()
     assert torch.equal(u, replayed)
+
+
+@pytest.mark.parametrize("working_stream", [False, True])
+def test_first_calls_while_another_stream_is_captured(working_stream):
+    """A context's first calls, which capture and instantiate its launch sequences, neither fail nor
+    spoil a capture on another stream in the default (global) mode; the results are the usual ones."""
+    import ctypes
+    import torch
+    from paper_1503_00757_gb300.binding import Context, Context3D, lib
+    L = lib()
+    mT, mR, v, vt = _inputs()
+    rng = np.random.default_rng(6)
+    m3 = [to_gpu(rng.random((16, 16, 16))) for _ in range(2)]
+    v3, t3 = (to_gpu(0.1 * rng.standard_normal((3, 16, 16, 16))) for _ in range(2))
+    E = lambda k: torch.zeros(k, N, N, device="cuda")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+
+    def calls():
+        s = torch.cuda.Stream() if working_stream else None
+        ctx, c3 = Context(N, N, NT, stream=s), Context3D(16, 16, 16, 2, stream=s)
+        u, det, m1, g, H, H3 = E(2), E(1), E(1), E(2), E(2), torch.zeros_like(v3)
+        torch.cuda.synchronize()
+        ctx.set_images(mT, mR)
+        c3.set_images(*m3)
+        c3.gradient(v3, H3)
+        todo = [lambda: L.reg_displacement(ctx.h, p(v), p(u)), lambda: L.reg3_hessian_matvec(c3.h, p(t3), p(H3)),
+                lambda: L.reg_detgrad(ctx.h, p(v), p(det), None), lambda: L.reg_objective(ctx.h, p(v), p(m1), None),
+                lambda: L.reg_gradient(ctx.h, p(v), p(g), None), lambda: L.reg_hessian_matvec(ctx.h, p(vt), p(H))]
+        # dropping captured sequences counts as well
+        todo += [lambda: L.reg_set_params(ctx.h, NT, 1, 2e-2, math.inf, 0.0)]
+        torch.cuda.synchronize()
+        return ctx, c3, todo, (u, det, m1, g, H, H3)
+
+    ctx, c3, todo, ref = calls()
+    assert [f() for f in todo] == [0] * len(todo)
+    torch.cuda.synchronize()
+    ctx.close()
+    c3.close()
+    ctx, c3, todo, out = calls()
+    x, other, graph = torch.zeros(4, device="cuda"), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=other):
+        x.add_(1)
+        rcs = [f() for f in todo]
+        x.add_(1)
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    ctx.close()
+    c3.close()
+    assert rcs == [0] * len(todo)
+    assert bool((x == 2).all())
+    assert all(torch.equal(a, b) for a, b in zip(ref, out))
