@@ -154,26 +154,31 @@ __device__ __forceinline__ void stage_chunk(float2* dst, const float2* __restric
     for (int i = threadIdx.x; i < n / 2; i += blockDim.x) d4[i] = s4[i];
 }
 
-// blockIdx.y: independent fields, f floats and s spectrum entries apart
+// Fields of a launch: one, many equally spaced ones, or two anywhere (blockIdx.y picks the field).
+// Kinds of their own: with the strides in the one-field kernels a solve's small launches were 1 to
+// 6 % slower (preconditioner at 256^2: 14.9 us with them, 14.4 without).
+enum Fields { ONE = 0, MANY = 1, TWO = 2 };
+// MANY: f floats and s spectrum entries apart
 struct Batch {
     long long f, s;
 };
-// a second vector field and its spectra for blockIdx.y = 1 (nullptr: none)
+// TWO: the second vector field and its spectra
 struct Second {
     const float *f1, *f2;
     float2 *S1, *S2;
 };
 
-template <int LOGL, bool VEC>
+template <int LOGL, bool VEC, int FIELDS>
 __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const float* __restrict__ f2,
                                              float2* S1, float2* S2, int R, const float2* __restrict__ tw, Batch bt, Second sec) {
     pdl_entry();
-    if (VEC && sec.f1 && blockIdx.y) {
+    if (FIELDS == TWO && blockIdx.y) {
         f1 = sec.f1;
         f2 = sec.f2;
         S1 = sec.S1;
         S2 = sec.S2;
-    } else {
+    }
+    if (FIELDS == MANY) {
         f1 += blockIdx.y * bt.f;
         S1 += blockIdx.y * bt.s;
         if (VEC) {
@@ -222,16 +227,19 @@ __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const
     }
 }
 
-template <int LOGL, bool VEC>
+// FIELDS == MANY also scales the result
+template <int LOGL, bool VEC, int FIELDS>
 __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, const float2* __restrict__ S2,
                                              float* __restrict__ f1, float* __restrict__ f2, int R,
                                              const float2* __restrict__ tw, Batch bt, float scale) {
     pdl_entry();
-    f1 += blockIdx.y * bt.f;
-    S1 += blockIdx.y * bt.s;
-    if (VEC) {
-        f2 += blockIdx.y * bt.f;
-        S2 += blockIdx.y * bt.s;
+    if (FIELDS == MANY) {
+        f1 += blockIdx.y * bt.f;
+        S1 += blockIdx.y * bt.s;
+        if (VEC) {
+            f2 += blockIdx.y * bt.f;
+            S2 += blockIdx.y * bt.s;
+        }
     }
     extern __shared__ __align__(16) float2 sm[];
     constexpr int L = 1 << LOGL, T = L >> 3, W = L >> 1;
@@ -257,14 +265,15 @@ __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, cons
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int j = t + k * T;
+            if (FIELDS == MANY) x[k] = cscale(x[k], scale);
             if (VEC) {
                 const size_t idx = (size_t)(row0 + q) * L + j;
-                f1[idx] = scale * x[k].x;
-                f2[idx] = scale * x[k].y;
+                f1[idx] = x[k].x;
+                f2[idx] = x[k].y;
             } else {
                 const size_t idx = (size_t)(row0 + 2 * q) * L + j;
-                f1[idx] = scale * x[k].x;
-                f1[idx + L] = scale * x[k].y;
+                f1[idx] = x[k].x;
+                f1[idx + L] = x[k].y;
             }
         }
     }
@@ -558,7 +567,7 @@ __global__ void __launch_bounds__(512) k_adj_init_sp(const float* __restrict__ a
 // the partner entry at -k1 before the multiplier is applied.
 // ---------------------------------------------------------------------------
 struct ColArgs {
-    long long bs;   // blockIdx.y: stride of independent fields (0: one field)
+    long long bs;   // MANY: spectrum entries from field to field
     const float2* in[5];
     float2* out[2];
     SpecParams P;
@@ -692,7 +701,7 @@ __device__ __forceinline__ void spec_apply(const SpecParams& P, float k1o, float
     }
 }
 
-template <int LOGL, int NIN, int NOUT, int OP>
+template <int LOGL, int NIN, int NOUT, int OP, int FIELDS>
 __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict__ tw) {
     pdl_entry();
     extern __shared__ __align__(16) float2 sm[];
@@ -709,7 +718,7 @@ __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict
     float2 xin[NIN][8];
 #pragma unroll
     for (int f = 0; f < NIN; ++f) {
-        const float2* src = a.in[f] + blockIdx.y * a.bs;
+        const float2* src = FIELDS == MANY ? a.in[f] + blockIdx.y * a.bs : a.in[f];
         for (int idx = threadIdx.x; idx < C * L; idx += blockDim.x) {
             const int g = idx >> g_shift;
             const int rem = idx & g_mask;
@@ -778,7 +787,7 @@ __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict
 #pragma unroll
         for (int k = 0; k < 8; ++k) A[c * L + t + k * T] = y[o][k];
         __syncthreads();
-        float2* dst = a.out[o] + blockIdx.y * a.bs;
+        float2* dst = FIELDS == MANY ? a.out[o] + blockIdx.y * a.bs : a.out[o];
         const float cd2 = 1.0f / (float)a.n2;
         for (int idx = threadIdx.x; idx < C * L; idx += blockDim.x) {
             const int g = idx >> g_shift;
@@ -854,7 +863,7 @@ void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S, int nb, long lon
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 8.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = k_r2c<LG, false>;
+        auto kern = nb > 1 ? k_r2c<LG, false, MANY> : k_r2c<LG, false, ONE>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw,
                  Batch{(long long)ctx->N, ss}, Second{});
@@ -866,7 +875,7 @@ void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, 
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = k_r2c<LG, true>;
+        auto kern = nb > 1 ? k_r2c<LG, true, MANY> : k_r2c<LG, true, ONE>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, u1, u2, S1, S2, g.R, ctx->tw,
                  Batch{2LL * ctx->N, (long long)ctx->N}, Second{});
@@ -878,7 +887,7 @@ void launch_r2c_two(reg_ctx* ctx, const float* u, const float* b, float2* const*
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 32.0 * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = k_r2c<LG, true>;
+        auto kern = k_r2c<LG, true, TWO>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, 2), g.threads, g.smem, u, u + ctx->N, S[0], S[1], g.R, ctx->tw, Batch{0, 0},
                  Second{b, b + ctx->N, S[2], S[3]});
@@ -890,7 +899,7 @@ void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f) {
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 8.0 * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = k_c2r<LG, false>;
+        auto kern = k_c2r<LG, false, ONE>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, g.grid, g.threads, g.smem, S, nullptr, f, nullptr, g.R, ctx->tw, Batch{0, 0}, 1.f);
     });
@@ -902,7 +911,7 @@ void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1,
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = k_c2r<LG, true>;
+        auto kern = nb > 1 || scale != 1.f ? k_c2r<LG, true, MANY> : k_c2r<LG, true, ONE>;
         set_smem(kern, g.smem);
         launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, S1, S2, u1, u2, g.R, ctx->tw,
                  Batch{2LL * ctx->N, ss > 0 ? ss : (long long)ctx->N}, scale);
@@ -956,7 +965,7 @@ void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, 
     ktimer_end(ctx);
 }
 
-template <int NIN, int NOUT, int OP>
+template <int NIN, int NOUT, int OP, int FIELDS = ONE>
 static void launch_col_t(reg_ctx* ctx, const float2* const* in, float2* const* out, const SpecParams& P,
                          double* part, int nb = 1, long long bs = 0) {
     const int L = ctx->n1, W = ctx->n2 / 2;
@@ -975,7 +984,7 @@ static void launch_col_t(reg_ctx* ctx, const float2* const* in, float2* const* o
     a.n2 = ctx->n2;
     ktimer_begin(ctx, KC_COL, 4.0 * nb * (NIN + NOUT + (OP == OP_DIV1 ? 1 : 0)) * ctx->N);
     DISPATCH_LOG(ctx->log1, {
-        auto kern = k_col<LG, NIN, NOUT, OP>;
+        auto kern = k_col<LG, NIN, NOUT, OP, FIELDS>;
         set_smem(kern, smem);
         launch_k(ctx, kern, dim3(W / cpb, nb), cpb * (L / 8), smem, a, ctx->tw);
     });
@@ -987,7 +996,10 @@ int col_blocks(reg_ctx* ctx) { return (ctx->n2 / 2) / spec_cols_per_cta(ctx); }
 void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* out, const SpecParams& P,
                 double* part, int nb, long long bs) {
     switch (op) {
-        case OP_GRAD: launch_col_t<1, 2, OP_GRAD>(ctx, in, out, P, part, nb, bs); break;
+        case OP_GRAD:
+            if (nb > 1) launch_col_t<1, 2, OP_GRAD, MANY>(ctx, in, out, P, part, nb, bs);
+            else launch_col_t<1, 2, OP_GRAD>(ctx, in, out, P, part);
+            break;
         case OP_DIV: launch_col_t<2, 1, OP_DIV>(ctx, in, out, P, part); break;
         case OP_REG: launch_col_t<2, 2, OP_REG>(ctx, in, out, P, part); break;
         case OP_PROJ: launch_col_t<2, 2, OP_PROJ>(ctx, in, out, P, part); break;
@@ -997,7 +1009,10 @@ void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* ou
         case OP_DIVT_PROJ: launch_col_t<5, 2, OP_DIVT_PROJ>(ctx, in, out, P, part); break;
         case OP_GRAD1: launch_col_t<1, 1, OP_GRAD1>(ctx, in, out, P, part); break;
         case OP_DIV1: launch_col_t<1, 1, OP_DIV1>(ctx, in, out, P, part); break;
-        case OP_SMOOTH_PROJ: launch_col_t<2, 2, OP_SMOOTH_PROJ>(ctx, in, out, P, part, nb, bs); break;
+        case OP_SMOOTH_PROJ:
+            if (nb > 1) launch_col_t<2, 2, OP_SMOOTH_PROJ, MANY>(ctx, in, out, P, part, nb, bs);
+            else launch_col_t<2, 2, OP_SMOOTH_PROJ>(ctx, in, out, P, part);
+            break;
         case OP_SMOOTH: launch_col_t<1, 1, OP_SMOOTH>(ctx, in, out, P, part); break;
         case OP_MASSP: launch_col_t<2, 2, OP_MASSP>(ctx, in, out, P, part); break;
         case OP_QINV: launch_col_t<2, 2, OP_QINV>(ctx, in, out, P, part); break;
