@@ -58,14 +58,15 @@ enum Slot {
 
 struct EventPair { cudaEvent_t a, b; int kclass; double bytes; };
 
-// A captured launch sequence, replayed with cudaGraphLaunch.  Keyed by the
-// kind of sequence, the caller pointers it was captured with and nt.
+// A launch sequence, once captured replayed with cudaGraphLaunch.  Keyed by the
+// kind of sequence, the pointers it was captured with and nt.
 struct GraphEntry {
     int kind;
     const void* p0;
     const void* p1;
     int nt;
-    cudaGraphExec_t exec;
+    int direct;            // times it was launched directly, before a capture
+    cudaGraphExec_t exec;  // nullptr: not captured (yet)
     long long nkern;
 };
 
