@@ -347,6 +347,12 @@ static bool capturing(const reg_ctx* c) {
 // first objective of a fresh context, 256^2, H1, nt = 8: 262 us captured, 135 us directly
 constexpr int DIRECT_CALLS = 4;
 
+// Calls that replay a captured sequence cannot go into a caller's capture: refused before anything of
+// the context, or of the caller's graph, changes.
+static int refuse_capture(const reg_ctx* c) {
+    return capturing(c) ? reg_fail(REG_ERR_CUDA, "the context's stream is being captured") : REG_OK;
+}
+
 template <typename F>
 static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt, F&& body) {
     if (c->timing && c->stream != 0) {
@@ -1065,6 +1071,7 @@ static void matvec_launches(reg_ctx* c, const float* vt, float* Hvt) {
 
 static int matvec_dev(reg_ctx* c, const float* vt, float* Hvt) {
     if (!c->have_lin) return reg_fail(REG_ERR_STATE, "reg_hessian_matvec called before reg_gradient");
+    RET(refuse_capture(c));
     CK(cudaMemcpyAsync(c->vtil, vt, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
     RET(run_seq(c, GK_MATVEC, nullptr, nullptr, c->nt_lin, [&] { matvec_launches(c, c->vtil, nullptr); }));
     return finish_out(c, Hvt);
@@ -1161,6 +1168,7 @@ extern "C" int reg_objective(reg_ctx* c, const float* v, float* m1, double* J) {
     CTX_CHECK(c);
     RET(check_ptr(v, "v"));
     if (m1) RET(check_ptr(m1, "m1"));
+    RET(refuse_capture(c));
     if (v != c->vtrial)
         CK(cudaMemcpyAsync(c->vtrial, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
     RET(objective_dev(c, c->vtrial, c->nt));
@@ -1177,6 +1185,7 @@ extern "C" int reg_objective(reg_ctx* c, const float* v, float* m1, double* J) {
 extern "C" int reg_gradient(reg_ctx* c, const float* v, float* g, double* J) {
     CTX_CHECK(c);
     RET(check_ptr(v, "v")); RET(check_ptr(g, "g"));
+    RET(refuse_capture(c));
     RET(gradient_dev(c, v, g, c->nt));
     if (J) {
         RET(read_scalars(c));
@@ -1550,6 +1559,7 @@ extern "C" int reg_detgrad(reg_ctx* c, const float* v, float* detF, double* stat
     CTX_CHECK(c);
     RET(check_ptr(v, "v"));
     if (detF) RET(check_ptr(detF, "detF"));
+    RET(refuse_capture(c));
     const int nt = c->nt;
     CK(cudaMemcpyAsync(c->vtil, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
     RET(run_seq(c, GK_DETGRAD, nullptr, nullptr, nt, [&] { detgrad_launches(c, c->vtil, nt); }));

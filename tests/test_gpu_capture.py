@@ -105,3 +105,42 @@ def test_first_calls_while_another_stream_is_captured(working_stream):
     assert rcs == [0] * len(todo)
     assert bool((x == 2).all())
     assert all(torch.equal(a, b) for a, b in zip(ref, out))
+
+
+@pytest.mark.parametrize("called_before", [False, True])
+def test_refused_calls_leave_the_context_and_the_capture_as_they_were(called_before):
+    """Objective, gradient, matvec and det F are refused on a stream that is being captured; the
+    linearization point and the caller's graph do not notice."""
+    import ctypes
+    import torch
+    from paper_1503_00757_gb300.binding import Context, lib
+    L = lib()
+    mT, mR, v, vt = _inputs()
+    s = torch.cuda.Stream()
+    ctx = Context(N, N, NT, stream=s)
+    E = lambda k: torch.zeros(k, N, N, device="cuda")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    g, H, H2, w, x = E(2), E(2), E(2), (0.5 * v).contiguous(), torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    ctx.set_images(mT, mR)
+    if called_before:
+        ctx.detgrad(v)
+        ctx.objective(v)
+    ctx.gradient(v, g)
+    ctx.hessian_matvec(vt, H)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        x.add_(1)
+        rcs = [L.reg_gradient(ctx.h, p(w), p(g), None), L.reg_objective(ctx.h, p(w), None, None),
+               L.reg_hessian_matvec(ctx.h, p(w), p(H)), L.reg_detgrad(ctx.h, p(w), None, None)]
+        x.add_(1)
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert rcs == [2, 2, 2, 2]  # REG_ERR_CUDA
+    assert bool((x == 2).all())
+    ctx.hessian_matvec(vt, H2)
+    torch.cuda.synchronize()
+    ctx.close()
+    assert torch.equal(H, H2)
