@@ -64,11 +64,15 @@ extern "C" void reg_default_opts(reg_solve_opts* o) {
 // ---------------------------------------------------------------------------
 // allocation
 // ---------------------------------------------------------------------------
+static void drop_graph(GraphEntry& g) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (g.graph) cudaGraphDestroy(g.graph);
+}
+
 static void clear_graphs(reg_ctx* c) {
     if (c->graphs.empty()) return;
     const GraphCalls allow;
-    for (auto& g : c->graphs)
-        if (g.exec) cudaGraphExecDestroy(g.exec);
+    for (auto& g : c->graphs) drop_graph(g);
     c->graphs.clear();
 }
 
@@ -323,20 +327,70 @@ extern "C" int reg_set_stream(reg_ctx* c, void* stream) {
 // ---------------------------------------------------------------------------
 // CUDA graphs: each fixed launch sequence (objective, gradient tail, matvec,
 // one PCG iteration, det F, displacement) is captured once per (kind, internal
-// pointers, nt) and replayed.  The sequences touch the context's buffers only:
-// a caller's field is copied in before and the last kernel (spectra to the
-// caller's buffer) is launched after, so new buffers cost nothing.  The legacy
+// pointers, nt) and replayed.  The sequences work on the context's buffers: a
+// caller's field is copied in by the first node, or before, and the caller's
+// buffer is written by the last node, or after; the two nodes are pointed at the
+// buffers of each call (Io), so new buffers cost nothing.  The legacy
 // default stream cannot be captured: its sequences are captured on a stream of
 // the context's own and replayed on the legacy stream.  Capture and instantiation
-// cost 60 to 150 us, as much as several calls gain, so on that stream (and for
-// the displacement and label solves on any) a sequence is launched directly the
-// first DIRECT_CALLS times.  While per-kernel timing is on sequences run directly
+// cost 60 to 150 us and a replay gains 5 to 20 us over direct launches, so on that
+// stream (and for the displacement and label solves on any) a sequence is launched
+// directly the first DIRECT_CALLS times.  While per-kernel timing is on sequences run directly
 // (legacy stream) or with event nodes.
 // ---------------------------------------------------------------------------
 enum GraphKind {
     GK_OBJECTIVE = 1, GK_GRADIENT = 2, GK_MATVEC = 3, GK_PCG_ITER = 4, GK_PCG_INIT = 5, GK_DETGRAD = 6,
-    GK_GRADIENT_Y = 7, GK_PCG_ITER_Y = 8, GK_PCG_INIT_Y = 9, GK_DISPLACEMENT = 10, GK_LABELS = 11
+    GK_GRADIENT_Y = 7, GK_PCG_ITER_Y = 8, GK_PCG_INIT_Y = 9, GK_DISPLACEMENT = 10, GK_LABELS = 11,
+    GK_OBJECTIVE_IN = 12
 };
+
+// The caller's fields of a sequence (each nullable): its first launch copies 2 N floats from `in` to
+// `dst`, its last one writes `out` (launch_c2r_vec, or a copy of 2 N floats from `src`).
+struct Io {
+    const float* in;
+    float* dst;
+    float* out;
+    const float* src;
+};
+
+// after a capture with io: the sequence is a chain, so the nodes are its root and its leaf
+static bool find_io(GraphEntry& g, const Io& io) {
+    size_t n = 1;
+    if (io.in && (cudaGraphGetRootNodes(g.graph, &g.in_node, &n) != cudaSuccess || n != 1)) return false;
+    if (io.out) {
+        if (cudaGraphGetNodes(g.graph, nullptr, &n) != cudaSuccess) return false;
+        std::vector<cudaGraphNode_t> nodes(n);
+        if (cudaGraphGetNodes(g.graph, nodes.data(), &n) != cudaSuccess) return false;
+        for (cudaGraphNode_t v : nodes) {
+            cudaGraphNode_t after[2];
+            cudaGraphEdgeData edge[2];  // the programmatic edges carry data, which a query has to take
+            size_t next = 2;
+            if (cudaGraphNodeGetDependentNodes(v, after, edge, &next) != cudaSuccess) return false;
+            if (next == 0) g.out_node = v;
+        }
+    }
+    g.in = io.in;
+    g.out = io.out;
+    return true;
+}
+
+// points the nodes of a captured sequence at this call's fields
+static bool bind_io(reg_ctx* c, GraphEntry& g, const Io& io) {
+    const size_t bytes = sizeof(float) * 2 * c->N;
+    if (io.in != g.in) {
+        if (cudaGraphExecMemcpyNodeSetParams1D(g.exec, g.in_node, io.dst, io.in, bytes, cudaMemcpyDeviceToDevice) != cudaSuccess)
+            return false;
+        g.in = io.in;
+    }
+    if (io.out != g.out) {
+        const cudaError_t e = io.src ? cudaGraphExecMemcpyNodeSetParams1D(g.exec, g.out_node, io.out, io.src, bytes,
+                                                                          cudaMemcpyDeviceToDevice)
+                                     : rebind_c2r_vec(g.exec, g.out_node, io.out, io.out + c->N);
+        if (e != cudaSuccess) return false;
+        g.out = io.out;
+    }
+    return true;
+}
 
 // whether the caller is capturing the working stream
 static bool capturing(const reg_ctx* c) {
@@ -345,7 +399,7 @@ static bool capturing(const reg_ctx* c) {
 }
 
 // first objective of a fresh context, 256^2, H1, nt = 8: 262 us captured, 135 us directly
-constexpr int DIRECT_CALLS = 4;
+constexpr int DIRECT_CALLS = 10;
 
 // Calls that replay a captured sequence cannot go into a caller's capture: refused before anything of
 // the context, or of the caller's graph, changes.
@@ -353,8 +407,9 @@ static int refuse_capture(const reg_ctx* c) {
     return capturing(c) ? reg_fail(REG_ERR_CUDA, "the context's stream is being captured") : REG_OK;
 }
 
-template <typename F>
-static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt, F&& body) {
+// direct: the same launches without the copies that only a replay needs
+template <typename F, typename G>
+static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt, const Io& io, F&& body, G&& direct) {
     if (c->timing && c->stream != 0) {
         // per-kernel timing: capture the sequence with its event records as graph nodes, so
         // the events bracket the kernels on the device without host launch gaps in between
@@ -380,23 +435,30 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
     GraphEntry* seq = nullptr;
     for (auto& g : c->graphs)
         if (g.kind == kind && g.p0 == p0 && g.p1 == p1 && g.nt == nt) seq = &g;
+    const GraphCalls allow;
     if (seq && seq->exec) {
-        CK(cudaGraphLaunch(seq->exec, c->stream));
-        c->launches += seq->nkern;
+        if (bind_io(c, *seq, io)) {
+            CK(cudaGraphLaunch(seq->exec, c->stream));
+            c->launches += seq->nkern;
+        } else {  // memory of a kind the nodes cannot be pointed at
+            cudaGetLastError();
+            body();
+            CKL();
+        }
         return REG_OK;
     }
-    const GraphCalls allow;
     if (!seq) {
         if (c->graphs.size() >= 64) {  // callers that pass many distinct pointers: drop the oldest capture
-            if (c->graphs.front().exec) cudaGraphExecDestroy(c->graphs.front().exec);
+            drop_graph(c->graphs.front());
             c->graphs.erase(c->graphs.begin());
         }
-        c->graphs.push_back(GraphEntry{kind, p0, p1, nt, 0, nullptr, 0});
+        c->graphs.emplace_back();
         seq = &c->graphs.back();
+        seq->kind = kind; seq->p0 = p0; seq->p1 = p1; seq->nt = nt;
     }
     if ((c->stream == 0 || kind == GK_DISPLACEMENT || kind == GK_LABELS) && seq->direct < DIRECT_CALLS) {
         ++seq->direct;
-        body();
+        direct();
         CKL();
         return REG_OK;
     }
@@ -422,15 +484,24 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         return reg_fail(REG_ERR_CUDA, std::string("stream capture failed: ") + cudaGetErrorString(e));
     }
     seq->nkern = nk;
+    seq->graph = graph;
     e = cudaGraphInstantiate(&seq->exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-        seq->exec = nullptr;
-        return reg_fail(REG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) seq->exec = nullptr;
+    const bool found = e != cudaSuccess || find_io(*seq, io);
+    if (e != cudaSuccess || !found || !(io.in || io.out)) {
+        cudaGraphDestroy(seq->graph);
+        seq->graph = nullptr;
     }
+    if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    if (!found) return reg_fail(REG_ERR_CUDA, "graph nodes of the caller's fields");
     CK(cudaGraphLaunch(seq->exec, c->stream));
     c->launches += nk;
     return REG_OK;
+}
+
+template <typename F>
+static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt, F&& body, const Io& io = Io{}) {
+    return run_seq(c, kind, p0, p1, nt, io, body, body);
 }
 
 static int check_ptr(const void* p, const char* what) {
@@ -599,15 +670,14 @@ static void sp_divt_proj(reg_ctx* c, float coefA, const float* T, const float* b
 }
 
 // the result of gradient_launches / matvec_launches with a null output, into the caller's buffer
-static int finish_out(reg_ctx* c, float* out) {
-    if (!c->shear_model)
-        launch_c2r_vec(c, c->S[4], c->S[5], out, out + c->N);
-    else if (c->pmode == PROJ_LERAY)
+static const float* out_src(const reg_ctx* c) { return c->shear_model && c->pmode != PROJ_LERAY ? c->vtmp2 : nullptr; }
+static void finish_out(reg_ctx* c, float* out) {
+    if (out_src(c))
+        cudaMemcpyAsync(out, out_src(c), sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+    else if (c->shear_model)
         launch_c2r_vec(c, c->S[5], c->S[0], out, out + c->N);
     else
-        CK(cudaMemcpyAsync(out, c->vtmp2, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    CKL();
-    return REG_OK;
+        launch_c2r_vec(c, c->S[4], c->S[5], out, out + c->N);
 }
 
 // regularization energy into d_scal[SL_JREG]
@@ -965,6 +1035,19 @@ static int objective_dev(reg_ctx* c, const float* v, int nt, const float* y = nu
     RET(ensure_nt(c, nt));
     return run_seq(c, GK_OBJECTIVE, v, y, nt, [&] { objective_launches(c, v, nt, y); });
 }
+// the same at a caller's v, which is copied to the context's field `at` first (keep: it is read later on)
+static int objective_at(reg_ctx* c, const float* v, float* at, int nt, bool keep, const float* y = nullptr) {
+    if (v == at) return objective_dev(c, at, nt, y);
+    RET(ensure_nt(c, nt));
+    auto body = [&] {
+        cudaMemcpyAsync(at, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        objective_launches(c, at, nt, y);
+    };
+    return run_seq(c, GK_OBJECTIVE_IN, at, y, nt, Io{v, at, nullptr, nullptr}, body, [&] {
+        if (keep) body();
+        else objective_launches(c, v, nt, y);
+    });
+}
 
 static void gradient_launches(reg_ctx* c, const float* v, float* g, int nt) {
     adjoint_solve(c, v, nt, c->mR, 1.f, mh(c, nt), -1.f, c->bvec, c->full_newton ? c->lam_hist : nullptr);
@@ -986,19 +1069,14 @@ static void gradient_launches(reg_ctx* c, const float* v, float* g, int nt) {
 }
 
 // the velocity becomes the context's linearization point first: the sequences read it from there
-static int set_lin(reg_ctx* c, const float* v) {
-    c->have_lin = false;
-    if (v != c->v_lin)
-        CK(cudaMemcpyAsync(c->v_lin, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    return REG_OK;
-}
-
 static int gradient_dev(reg_ctx* c, const float* v, float* g, int nt) {
-    RET(set_lin(c, v));
-    RET(objective_dev(c, c->v_lin, nt));
-    float* out = g == c->g ? g : nullptr;  // reg_solve's own buffer, or finished outside the sequence
-    RET(run_seq(c, GK_GRADIENT, out, nullptr, nt, [&] { gradient_launches(c, c->v_lin, out, nt); }));
-    if (!out) RET(finish_out(c, g));
+    RET(objective_at(c, v, c->v_lin, nt, true));
+    c->have_lin = false;
+    float* own = g == c->g ? g : nullptr;  // reg_solve's own buffer, or a caller's
+    RET(run_seq(c, GK_GRADIENT, own, nullptr, nt, [&] {
+        gradient_launches(c, c->v_lin, own, nt);
+        if (!own) finish_out(c, g);
+    }, Io{nullptr, nullptr, own ? nullptr : g, out_src(c)}));
     c->nt_lin = nt;
     c->have_lin = true;
     return REG_OK;
@@ -1006,8 +1084,8 @@ static int gradient_dev(reg_ctx* c, const float* v, float* g, int nt) {
 
 // Gradient in preconditioned coordinates: g_y = Q^-1 g_v = Pi0 y + Q^-1 K b, at v = Q^-1 y
 static int gradient_dev_y(reg_ctx* c, const float* v, const float* y, float* gy, int nt) {
-    RET(set_lin(c, v));
-    RET(objective_dev(c, c->v_lin, nt, y));
+    RET(objective_at(c, v, c->v_lin, nt, true, y));
+    c->have_lin = false;
     RET(run_seq(c, GK_GRADIENT_Y, y, nullptr, nt, [&] {  // gy is always c->g
         adjoint_solve(c, c->v_lin, nt, c->mR, 1.f, mh(c, nt), -1.f, c->bvec, c->full_newton ? c->lam_hist : nullptr);
         sp_assemble_y(c, y, c->bvec, gy);
@@ -1072,9 +1150,14 @@ static void matvec_launches(reg_ctx* c, const float* vt, float* Hvt) {
 static int matvec_dev(reg_ctx* c, const float* vt, float* Hvt) {
     if (!c->have_lin) return reg_fail(REG_ERR_STATE, "reg_hessian_matvec called before reg_gradient");
     RET(refuse_capture(c));
-    CK(cudaMemcpyAsync(c->vtil, vt, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    RET(run_seq(c, GK_MATVEC, nullptr, nullptr, c->nt_lin, [&] { matvec_launches(c, c->vtil, nullptr); }));
-    return finish_out(c, Hvt);
+    // Hvt may be vt: the direct launches, too, have read vt before the first store to Hvt
+    auto body = [&] {
+        cudaMemcpyAsync(c->vtil, vt, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        matvec_launches(c, c->vtil, nullptr);
+        finish_out(c, Hvt);
+    };
+    return run_seq(c, GK_MATVEC, nullptr, nullptr, c->nt_lin, Io{vt, c->vtil, Hvt, out_src(c)}, body,
+                   [&] { matvec_launches(c, vt, Hvt); });
 }
 
 static void precond_dev(reg_ctx* c, const float* r, float* z) {
@@ -1169,9 +1252,7 @@ extern "C" int reg_objective(reg_ctx* c, const float* v, float* m1, double* J) {
     RET(check_ptr(v, "v"));
     if (m1) RET(check_ptr(m1, "m1"));
     RET(refuse_capture(c));
-    if (v != c->vtrial)
-        CK(cudaMemcpyAsync(c->vtrial, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream));
-    RET(objective_dev(c, c->vtrial, c->nt));
+    RET(objective_at(c, v, c->vtrial, c->nt, false));
     c->have_lin = false;  // history now belongs to this v, but grad/adjoint data do not
     if (m1) CK(cudaMemcpyAsync(m1, mh(c, c->nt), sizeof(float) * c->N, cudaMemcpyDeviceToDevice, c->stream));
     if (J) {

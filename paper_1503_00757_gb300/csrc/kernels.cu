@@ -919,6 +919,18 @@ void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1,
     ktimer_end(ctx);
 }
 
+cudaError_t rebind_c2r_vec(cudaGraphExec_t exec, cudaGraphNode_t node, float* u1, float* u2) {
+    cudaKernelNodeParams p;
+    const cudaError_t e = cudaGraphKernelNodeGetParams(node, &p);
+    if (e != cudaSuccess) return e;
+    void* args[8];  // k_c2r's parameters
+    for (int i = 0; i < 8; ++i) args[i] = p.kernelParams[i];
+    args[2] = &u1;
+    args[3] = &u2;
+    p.kernelParams = args;
+    return cudaGraphExecKernelNodeSetParams(exec, node, &p);
+}
+
 void launch_row_adv(reg_ctx* ctx, const AdvArgs& a) {
     const RowCfg g = row_cfg(ctx);
     // floats per node read/written: G 2 (complex half spectra = 1 float per node each), u_j 1,

@@ -43,13 +43,15 @@ def test_every_call_of_a_sequence_gives_the_same_result(n, regnorm, shear, worki
         torch.cuda.synchronize()
         J1, J2 = ctx.objective(a, m1), ctx.gradient(a, g)
         ctx.hessian_matvec(b, H)
+        ctx.hessian_matvec(b, b)  # in place
         ctx.displacement(a, u)
         ctx.label_overlap(a, lT, lR, lab)
         s = ctx.detgrad(a, det)
         torch.cuda.synchronize()
+        assert torch.equal(b, H)
         return (m1, g, H, u, lab, det), (J1, J2, s), (a, b)
 
-    calls = [once() for _ in range(7)]
+    calls = [once() for _ in range(13)]
     ctx.set_params(nt + 1, regnorm, 2 * beta, math.inf, shear)
     other = once()
     ctx.set_params(nt, regnorm, beta, 1e-3, shear)
