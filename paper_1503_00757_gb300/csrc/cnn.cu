@@ -1683,6 +1683,7 @@ extern "C" int reg_net_forward_fine(reg_net* n, const float* images, int B, floa
     if (B < 1 || B > n->maxB) return reg_fail(REG_ERR_ARG, "batch out of range");
     const int H = n->H, W = n->W, Hf = 2 * H, Wf = 2 * W;
     if (Hf > 1024 || Wf > 1024) return reg_fail(REG_ERR_ARG, "the fine grid (2H, 2W) must fit [16, 1024]");
+    if (((uintptr_t)v_out) & 15) return reg_fail(REG_ERR_ARG, "out is not 16-byte aligned");
     if (!n->proj_fine) {
         reg_ctx* pf = nullptr;
         int st = reg_create(reg_grid{Hf, Wf}, 1, REG_H1, 1.0, INFINITY, 0.0, &pf);

@@ -38,3 +38,18 @@ def test_output_map_of_a_batch_equals_its_members(H, W):
     net.close()
     assert torch.equal(scaled, out * torch.tensor(0.3, dtype=torch.float32, device="cuda"))
     assert torch.equal(scaled, scaled_one)
+
+
+def test_fine_warm_start_refuses_a_misaligned_output():
+    import ctypes
+    import torch
+    from paper_1503_00757_gb300.binding import Net, lib
+    net = Net(32, 32, 1)
+    images, buf = torch.rand(1, 2, 64, 64, device="cuda"), torch.zeros(2 * 64 * 64 + 4, device="cuda")
+    torch.cuda.synchronize()
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert lib().reg_net_forward_fine(net.h, p(images), 1, p(buf[1:])) == 1  # REG_ERR_ARG
+    assert b"16-byte aligned" in lib().reg_last_error()
+    assert lib().reg_net_forward_fine(net.h, p(images), 1, p(buf)) == 0
+    torch.cuda.synchronize()
+    net.close()
