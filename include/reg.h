@@ -298,8 +298,9 @@ int reg_set_tiles(reg_ctx* ctx, int rows_per_cta, int cols_per_cta, int prefetch
  *     column slabs through distributed shared memory (square grids n x n,
  *     16 <= n <= 512, on devices with thread-block clusters);
  *   cluster == 0: a row kernel and a column kernel per Heun stage (every grid).
- * Default (until this call): grids of 64 to 256 points per axis with n1 n2 < 256^2 run every
- * Gauss-Newton transport solve as one launch resident in a cluster of 8 or 16 CTAs, with the
+ * Default (until this call, and after reg_reset_transport): grids of 64 to
+ * 256 points per axis with n1 n2 < 256^2 run every Gauss-Newton transport
+ * solve as one launch resident in a cluster of 8 or 16 CTAs, with the
  * arithmetic of the kernel pairs (results equal bit for bit); larger and smaller grids, and full
  * Newton, the kernel pairs.  H1 problems take derivatives axis by axis, H2 and H3 problems
  * through the row spectra (their Krylov iteration amplifies a change of rounding, so they keep
@@ -308,9 +309,14 @@ int reg_set_tiles(reg_ctx* ctx, int rows_per_cta, int cols_per_cta, int prefetch
  * concurrency measured.  REG_ERR_ARG if cluster != 0 and this grid or device cannot run it. */
 int reg_set_transport(reg_ctx* ctx, int cluster);
 
-/* The transport path of a context: *cluster = 1 for the cluster-resident
- * kernel; *ctas_per_cluster = its cluster size on this grid (0 if it cannot
- * run); *max_active_clusters = how many such clusters fit on the device at
+/* Back to the default described above. */
+int reg_reset_transport(reg_ctx* ctx);
+
+/* The transport path of a context: *cluster = 1 for the kernel that
+ * reg_set_transport(ctx, 1) selects, 0 otherwise (also where the default runs
+ * the resident solves of the small grids); *ctas_per_cluster = that kernel's
+ * cluster size on this grid (0 if it cannot run); *max_active_clusters = how
+ * many such clusters fit on the device at
  * once (cudaOccupancyMaxActiveClusters; independent solves on separate
  * streams run concurrently up to that number).  Host pointers, each nullable. */
 int reg_transport_config(reg_ctx* ctx, int* cluster, int* ctas_per_cluster, int* max_active_clusters);

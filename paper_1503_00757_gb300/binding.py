@@ -87,6 +87,7 @@ _SIGS = {
     "reg_set_tiles": ([_P, _I, _I, _I], _I),
     "reg_set_pdl": ([_P, _I], _I),
     "reg_set_transport": ([_P, _I], _I),
+    "reg_reset_transport": ([_P], _I),
     "reg_set_hessian": ([_P, _I], _I),
     "reg_displacement": ([_P, _P, _P], _I),
     "reg_label_overlap": ([_P, _P, _P, _P, _P, ctypes.POINTER(_D)], _I),
@@ -544,8 +545,12 @@ class Context:
         _check(lib().reg_set_tiles(self.h, R, C, P))
 
     def set_transport(self, cluster):
-        """Transport solves in the cluster-resident kernel (True) or the row/column kernel pairs (False)."""
-        _check(lib().reg_set_transport(self.h, 1 if cluster else 0))
+        """Transport solves in the cluster-resident kernel (True), the row/column kernel pairs (False)
+        or the default for the grid (None)."""
+        if cluster is None:
+            _check(lib().reg_reset_transport(self.h))
+        else:
+            _check(lib().reg_set_transport(self.h, 1 if cluster else 0))
 
     def transport_config(self):
         """(cluster path in use, CTAs per cluster, clusters that fit on the device at once)."""

@@ -177,7 +177,8 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->tileR = c->tileC = c->tileP = 0;
     c->pdl = true;
     c->tc_ok = tc_max_active_clusters(c->n1, c->n2) > 0;
-    c->use_rs = rs_available(c->log1, c->log2) && rs_sp_available(c->log1, c->log2);
+    c->rs_ok = rs_available(c->log1, c->log2) && rs_sp_available(c->log1, c->log2);
+    c->use_rs = c->rs_ok;
     c->use_tc = false;  // the row / column kernel pairs unless the autotuner measured the cluster kernel faster
     {
         int dev = 0, R, C, P, D, T;
@@ -276,14 +277,23 @@ extern "C" int reg_set_tiles(reg_ctx* c, int rows_per_cta, int cols_per_cta, int
     return REG_OK;
 }
 
+static void set_transport(reg_ctx* c, bool tc, bool rs) {
+    if (tc != c->use_tc || rs != c->use_rs) clear_graphs(c);  // captures bake in the kernels
+    c->use_tc = tc;
+    c->use_rs = rs;
+}
+
 extern "C" int reg_set_transport(reg_ctx* c, int cluster) {
     if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
     if (cluster && !c->tc_ok)
         return reg_fail(REG_ERR_ARG, "the cluster-resident transport kernel does not run on this grid or device");
-    const bool on = cluster != 0;
-    if (on != c->use_tc || c->use_rs) clear_graphs(c);  // captures bake in the kernels
-    c->use_tc = on;
-    c->use_rs = false;
+    set_transport(c, cluster != 0, false);
+    return REG_OK;
+}
+
+extern "C" int reg_reset_transport(reg_ctx* c) {
+    if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
+    set_transport(c, false, c->rs_ok);
     return REG_OK;
 }
 

@@ -127,6 +127,7 @@ struct reg_ctx {
     float *lam_hist;   // (nt_cap + 1) * N
     float *gmt_hist;   // (nt_cap + 1) * 2N
     bool tc_ok;        // the cluster-resident transport kernel can run on this grid and device
+    bool rs_ok;        // the resident kernels run on this grid and device
     bool use_rs;       // Gauss-Newton transport solves in the resident kernel (small grids)
     bool use_tc;       // transport solves run in the cluster-resident kernel (else the two-pass kernels)
     int tileR, tileC;  // rows per row-kernel CTA, spectrum columns per column-kernel CTA (0: default)
