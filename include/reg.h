@@ -300,7 +300,8 @@ int reg_set_tiles(reg_ctx* ctx, int rows_per_cta, int cols_per_cta, int prefetch
  *   cluster == 0: a row kernel and a column kernel per Heun stage (every grid).
  * Default (until this call, and after reg_reset_transport): grids of 64 to
  * 256 points per axis with n1 n2 < 256^2 run every Gauss-Newton transport
- * solve as one launch resident in a cluster of 8 or 16 CTAs, with the
+ * solve (H2 and H3 problems: with n1 n2 <= 2^14) as one launch resident in a
+ * cluster of 8 or 16 CTAs, with the
  * arithmetic of the kernel pairs (results equal bit for bit); larger and smaller grids, and full
  * Newton, the kernel pairs.  H1 problems take derivatives axis by axis, H2 and H3 problems
  * through the row spectra (their Krylov iteration amplifies a change of rounding, so they keep

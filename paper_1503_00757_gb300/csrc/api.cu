@@ -177,8 +177,9 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->tileR = c->tileC = c->tileP = 0;
     c->pdl = true;
     c->tc_ok = tc_max_active_clusters(c->n1, c->n2) > 0;
-    c->rs_ok = rs_available(c->log1, c->log2) && rs_sp_available(c->log1, c->log2);
-    c->use_rs = c->rs_ok;
+    c->rs_ok = rs_available(c->log1, c->log2);
+    c->rs_sp_ok = rs_sp_available(c->log1, c->log2);
+    c->use_rs = true;
     c->use_tc = false;  // the row / column kernel pairs unless the autotuner measured the cluster kernel faster
     {
         int dev = 0, R, C, P, D, T;
@@ -293,7 +294,7 @@ extern "C" int reg_set_transport(reg_ctx* c, int cluster) {
 
 extern "C" int reg_reset_transport(reg_ctx* c) {
     if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
-    set_transport(c, false, c->rs_ok);
+    set_transport(c, false, true);
     return REG_OK;
 }
 
@@ -859,7 +860,9 @@ static void d1_of(reg_ctx* c, const float* f, const float* mul = nullptr, const 
 }
 
 // whole solves in one launch (transport_resident.cu)
-static bool resident(const reg_ctx* c) { return c->use_rs && !c->full_newton; }
+static bool resident(const reg_ctx* c) {
+    return c->use_rs && !c->full_newton && (sp_transport(c) ? c->rs_sp_ok : c->rs_ok);
+}
 
 // State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[nt] and gm_hist[0..nt]
 // (the kernel pairs also m_hist[1..nt-1]).

@@ -57,13 +57,19 @@ bool cluster_prepare(K k, const cudaLaunchConfig_t& cfg) {
     return ok;
 }
 
-// the grids of the resident kernels: 64 to 256 points per axis, fewer than 256 x 256
+// the grids of the resident kernels: 64 to 256 points per axis, up to 2^15 points (spectral stages: 2^14)
 #define RS_CASE(L1, L2, ...) \
     case (L1)*16 + (L2): { constexpr int B1 = L1, B2 = L2; __VA_ARGS__; } break;
+#define RS_SP_CASES(...)                                                                      \
+    RS_CASE(6, 6, __VA_ARGS__) RS_CASE(6, 7, __VA_ARGS__) RS_CASE(6, 8, __VA_ARGS__)          \
+    RS_CASE(7, 6, __VA_ARGS__) RS_CASE(7, 7, __VA_ARGS__) RS_CASE(8, 6, __VA_ARGS__)
 #define RS_DISPATCH(L1, L2, ...)                                                              \
     switch ((L1)*16 + (L2)) {                                                                 \
-        RS_CASE(6, 6, __VA_ARGS__) RS_CASE(6, 7, __VA_ARGS__) RS_CASE(6, 8, __VA_ARGS__)      \
-        RS_CASE(7, 6, __VA_ARGS__) RS_CASE(7, 7, __VA_ARGS__) RS_CASE(7, 8, __VA_ARGS__)      \
-        RS_CASE(8, 6, __VA_ARGS__) RS_CASE(8, 7, __VA_ARGS__)                                 \
+        RS_SP_CASES(__VA_ARGS__) RS_CASE(7, 8, __VA_ARGS__) RS_CASE(8, 7, __VA_ARGS__)        \
+        default: break;                                                                       \
+    }
+#define RS_SP_DISPATCH(L1, L2, ...)                                                           \
+    switch ((L1)*16 + (L2)) {                                                                 \
+        RS_SP_CASES(__VA_ARGS__)                                                              \
         default: break;                                                                       \
     }

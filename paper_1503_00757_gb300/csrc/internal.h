@@ -127,8 +127,8 @@ struct reg_ctx {
     float *lam_hist;   // (nt_cap + 1) * N
     float *gmt_hist;   // (nt_cap + 1) * 2N
     bool tc_ok;        // the cluster-resident transport kernel can run on this grid and device
-    bool rs_ok;        // the resident kernels run on this grid and device
-    bool use_rs;       // Gauss-Newton transport solves in the resident kernel (small grids)
+    bool rs_ok, rs_sp_ok;  // the resident kernels (with the spectral stages) are used on this grid and device
+    bool use_rs;       // Gauss-Newton transport solves in the resident kernel where it is used
     bool use_tc;       // transport solves run in the cluster-resident kernel (else the two-pass kernels)
     int tileR, tileC;  // rows per row-kernel CTA, spectrum columns per column-kernel CTA (0: default)
     int tileP;         // 1: RK2 row kernels prefetch their operands (used when tileR > 0)
@@ -309,7 +309,8 @@ struct RsArgs {
     float ca, cb;
     float* b;            // body force (2N): written
 };
-// grids of 64 to 256 points per axis on a device that fits the clusters (prepares the kernels)
+// grids of 64 to 256 points per axis, up to 2^15 (spectral stages: 2^14) points, on a device that fits
+// the clusters (prepares the kernels)
 bool rs_available(int log1, int log2);
 void launch_resident(reg_ctx* ctx, int mode, const RsArgs& a);
 // the same with the spectral stages (transport_resident_sp.cu)

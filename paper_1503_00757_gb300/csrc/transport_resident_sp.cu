@@ -1,6 +1,6 @@
 // The spectral RK2 stages of kernels.cu (k_row_adv_sp, k_row_adj_sp and the OP_GRAD1 / OP_DIV1
 // column passes) resident in a thread-block cluster: whole transport solves of the H2 and H3
-// problems on grids of 64 to 256 points per axis in one launch.
+// problems on grids of 64 to 256 points per axis, up to 2^14 points, in one launch.
 //
 // Those problems keep the spectral stages because their Krylov iteration amplifies a change of
 // rounding (kernels.cu), so this kernel does their arithmetic, expression by expression (products
@@ -321,7 +321,12 @@ bool sp_prepare() {
 }  // namespace
 
 bool rs_sp_available(int log1, int log2) {
-    if (log1 < 6 || log1 > 8 || log2 < 6 || log2 > 8 || log1 + log2 > 15) return false;
+    // 2^15 points: faster alone (matvec, nt = 16: 393 us against 449 at 256 x 128, 459 against 564 at
+    // 128 x 256) but not with many solves at once, whose clusters take turns on the chip: 8 solves 83
+    // against 79 us each, 32 solves 61 against 39 (128 x 256: 96 against 91, 70 against 36).  On 2^14
+    // points it is ahead at every number of solves: 128 x 128 alone 314 against 538, 32 at once 30.0
+    // against 30.9.
+    if (log1 < 6 || log1 > 8 || log2 < 6 || log2 > 8 || log1 + log2 > 14) return false;
     static std::mutex mu;
     static std::map<int, bool> known;  // per device and grid: the attributes apply to the current device
     int dev = 0;
@@ -331,7 +336,7 @@ bool rs_sp_available(int log1, int log2) {
     auto it = known.find(key);
     if (it != known.end()) return it->second;
     bool ok = false;
-    RS_DISPATCH(log1, log2, ok = sp_prepare<B1, B2, RS_STATE>() && sp_prepare<B1, B2, RS_ADJOINT>() &&
+    RS_SP_DISPATCH(log1, log2, ok = sp_prepare<B1, B2, RS_STATE>() && sp_prepare<B1, B2, RS_ADJOINT>() &&
                                  sp_prepare<B1, B2, RS_MATVEC>());
     return known[key] = ok;
 }
@@ -340,7 +345,7 @@ void launch_resident_sp(reg_ctx* ctx, int mode, const RsArgs& a) {
     const double fields = mode == RS_STATE ? 3 + 1 + 2.0 * (a.nt + 1)
                                            : (mode == RS_ADJOINT ? 6 + 2.0 * (a.nt + 1) : 6 + 4.0 * (a.nt + 1));
     ktimer_begin(ctx, KC_TRANSPORT, 4.0 * fields * ctx->N);
-    RS_DISPATCH(ctx->log1, ctx->log2, {
+    RS_SP_DISPATCH(ctx->log1, ctx->log2, {
         cudaLaunchAttribute attr[2];
         if (mode == RS_STATE) {
             cudaLaunchConfig_t cfg = sp_config<B1, B2, RS_STATE>(ctx->stream, attr, ctx->pdl);
