@@ -236,7 +236,7 @@ typedef struct {
  * concurrently.  Pairs are taken largest grid first.  Before the first pair
  * of a grid size is solved, reg_autotune picks that size's FFT tiles for
  * min(nworkers, 8) concurrent solves at the largest nt of the batch's pairs
- * of that size (once per process and device).  Every pair's result is identical to reg_solve on
+ * of that size and kind, H1 or H2 / H3 (once per process and device).  Every pair's result is identical to reg_solve on
  * that pair alone with a context created after that tuning.  Synchronous.  Returns REG_OK if
  * every pair returned REG_OK, else the first failing pair's status (each
  * item's own status is in item.status); REG_ERR_ARG for invalid arguments. */
@@ -263,7 +263,12 @@ void reg_executor_destroy(reg_executor* ex);
  * (D, see reg_set_pdl), on the current device with zero images and velocity
  * and private streams, and records the fastest in a process-wide table;
  * contexts created afterwards on this device and grid use it (existing
- * contexts keep theirs).  Valid: R a multiple of 4 dividing n1,
+ * contexts keep theirs until reg_set_params changes between H1 and H2 / H3).
+ * H1 problems and H2 / H3 problems run different kernels (reg_set_transport):
+ * both kinds are timed and recorded, the outputs are the H1 kind's, and the
+ * batch functions measure the kinds that their pairs need.  The matvec is
+ * timed as contexts run it: where its solves are resident in one launch, R, C
+ * and D are those of the kernels around them and P keeps its default.  Valid: R a multiple of 4 dividing n1,
  * 32 <= R n2 / 8 <= 512 threads; C a power of two >= 2 dividing n2 / 2,
  * 32 <= C n1 / 8 <= 256 threads; at most 227 KB of shared memory; P = 1 only
  * for n2 <= 512.  Every candidate is timed in two passes and keeps its faster
@@ -278,7 +283,10 @@ int reg_autotune(reg_grid grid, int nt, int concurrency, int force, int* rows_pe
 
 /* The tiles and launch mode a context launches with (tuned, else the default
  * rule: the smallest R with R n2 / 8 >= 64, the smallest C >= 4 (2 for
- * n1 = 1024) with C n1 / 8 >= 64, P = 1 for n2 <= 512, D = 1). */
+ * n1 = 1024) with C n1 / 8 >= 64, P = 1 for n2 <= 512, D = 1).  C is that of
+ * the axis-wise column kernel; by default the spectral one takes the smallest
+ * C >= 2 with C n1 / 8 >= 64.  The axis-wise kernels for rows of 1024 points
+ * prefetch whatever P is. */
 int reg_tile_config(reg_ctx* ctx, int* rows_per_cta, int* cols_per_cta, int* prefetch, int* pdl);
 
 /* Sets a context's tiles (validity as for reg_autotune; R = C = 0 restores

@@ -153,6 +153,19 @@ static void set_params(reg_ctx* c, int nt, int regnorm, double beta, double gamm
     c->have_lin = false;
 }
 
+// the tuned tiles and launch mode for the context's kind of problem, else the defaults
+static void apply_tuned(reg_ctx* c) {
+    int dev = 0;
+    Tuned t = {0, 0, 0, 1};
+    if (cudaGetDevice(&dev) == cudaSuccess) tuned_tiles(dev, c->n1, c->n2, tune_kind(c->regnorm), &t);
+    if (!c->tiles_set) {
+        c->tileR = t.R;
+        c->tileC = t.C;
+        c->tileP = t.P;
+    }
+    if (!c->pdl_set) c->pdl = t.D != 0;
+}
+
 extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, double gamma, double shear, reg_ctx** out) {
     if (!out) return reg_fail(REG_ERR_ARG, "out is NULL");
     *out = nullptr;
@@ -174,23 +187,13 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->stream = 0;
     c->cap = nullptr;
     c->launches = 0;
-    c->tileR = c->tileC = c->tileP = 0;
-    c->pdl = true;
+    c->tiles_set = c->pdl_set = false;
     c->tc_ok = tc_max_active_clusters(c->n1, c->n2) > 0;
     c->rs_ok = rs_available(c->log1, c->log2);
     c->rs_sp_ok = rs_sp_available(c->log1, c->log2);
     c->use_rs = true;
-    c->use_tc = false;  // the row / column kernel pairs unless the autotuner measured the cluster kernel faster
-    {
-        int dev = 0, R, C, P, D, T;
-        if (cudaGetDevice(&dev) == cudaSuccess && tuned_tiles(dev, c->n1, c->n2, &R, &C, &P, &D, &T)) {
-            c->tileR = R;
-            c->tileC = C;
-            c->tileP = P;
-            c->pdl = D != 0;
-            c->use_tc = T != 0 && c->tc_ok;
-        }
-    }
+    c->use_tc = false;
+    apply_tuned(c);
     c->use_graphs = true;
     c->timing = false;
     for (int k = 0; k < KC_COUNT; ++k) { c->tcount[k] = 0; c->tms[k] = 0.0; c->tbytes[k] = 0.0; }
@@ -257,13 +260,16 @@ extern "C" int reg_set_params(reg_ctx* c, int nt, int regnorm, double beta, doub
     const bool same = nt == c->nt && regnorm == c->regnorm && beta == c->beta_v && gamma == c->beta_w &&
                       shear == c->shear;
     if (!same) clear_graphs(c);  // captured sequences bake in nt and the Fourier-multiplier parameters
+    const bool other = tune_kind(regnorm) != tune_kind(c->regnorm);
     set_params(c, nt, regnorm, beta, gamma, shear);
+    if (other) apply_tuned(c);
     return alloc_hist(c, nt);
 }
 
 extern "C" int reg_set_tiles(reg_ctx* c, int rows_per_cta, int cols_per_cta, int prefetch) {
     if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
     if (rows_per_cta == 0 && cols_per_cta == 0) {
+        c->tiles_set = true;
         if (c->tileR != 0 || c->tileC != 0) clear_graphs(c);
         c->tileR = c->tileC = c->tileP = 0;
         return REG_OK;
@@ -272,6 +278,7 @@ extern "C" int reg_set_tiles(reg_ctx* c, int rows_per_cta, int cols_per_cta, int
         return reg_fail(REG_ERR_ARG, "tiles outside the launch limits of this grid");
     if (rows_per_cta != c->tileR || cols_per_cta != c->tileC || prefetch != c->tileP)
         clear_graphs(c);  // captures bake in launch shapes and kernels
+    c->tiles_set = true;
     c->tileR = rows_per_cta;
     c->tileC = cols_per_cta;
     c->tileP = prefetch;
@@ -324,6 +331,7 @@ extern "C" int reg_set_pdl(reg_ctx* c, int enable) {
     if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
     const bool on = enable != 0;
     if (on != c->pdl) clear_graphs(c);  // captures bake in the launch attribute
+    c->pdl_set = true;
     c->pdl = on;
     return REG_OK;
 }
@@ -863,6 +871,8 @@ static void d1_of(reg_ctx* c, const float* f, const float* mul = nullptr, const 
 static bool resident(const reg_ctx* c) {
     return c->use_rs && !c->full_newton && (sp_transport(c) ? c->rs_sp_ok : c->rs_ok);
 }
+
+bool resident_transport(const reg_ctx* c) { return resident(c); }
 
 // State equation (Eq. (e:state-eq-elim)), Heun in time: fills m_hist[nt] and gm_hist[0..nt]
 // (the kernel pairs also m_hist[1..nt-1]).

@@ -8,6 +8,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -62,17 +63,18 @@ extern "C" int reg_executor_solve(reg_executor* ex, reg_batch_item* items, int c
         items[i].status = -1;
     }
     const int nworkers = std::min<int>((int)ex->workers.size(), count);
-    // FFT tiles of every grid size in the batch (measured once per process and device)
+    // FFT tiles of every grid size and kind of stages in the batch (measured once per process and device)
     {
         cudaSetDevice(ex->dev);
-        std::map<std::pair<int, int>, int> sizes;  // grid -> largest nt of its pairs
+        std::map<std::tuple<int, int, int>, int> sizes;  // grid and kind -> largest nt of its pairs
         for (int i = 0; i < count; ++i) {
-            int& nt = sizes[std::make_pair(items[i].grid.n1, items[i].grid.n2)];
+            int& nt = sizes[std::make_tuple(items[i].grid.n1, items[i].grid.n2, (int)tune_kind(items[i].regnorm))];
             nt = std::max(nt, std::min(items[i].nt, 4096));
         }
         for (const auto& kv : sizes) {
-            const int st = reg_autotune(reg_grid{kv.first.first, kv.first.second}, std::max(kv.second, 1),
-                                        std::min(nworkers, 8), 0, nullptr, nullptr, nullptr, nullptr, nullptr);
+            Tuned t;
+            const int st = autotune_kind(reg_grid{std::get<0>(kv.first), std::get<1>(kv.first)}, std::max(kv.second, 1),
+                                         std::min(nworkers, 8), false, (TuneKind)std::get<2>(kv.first), &t, nullptr);
             if (st != REG_OK) return st;
         }
     }

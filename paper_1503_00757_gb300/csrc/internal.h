@@ -132,6 +132,7 @@ struct reg_ctx {
     bool use_tc;       // transport solves run in the cluster-resident kernel (else the two-pass kernels)
     int tileR, tileC;  // rows per row-kernel CTA, spectrum columns per column-kernel CTA (0: default)
     int tileP;         // 1: RK2 row kernels prefetch their operands (used when tileR > 0)
+    bool tiles_set, pdl_set;  // tiles / launch mode set by the caller: kept when the kind of problem changes
 
     long long launches;
     bool pdl;         // launch with programmatic dependent launch (default on)
@@ -149,9 +150,17 @@ struct reg_ctx {
 // ---- FFT tile choices (kernels.cu: defaults and limits; tune.cu: autotuner table) ----
 void default_tiles(int n1, int n2, int* R, int* C, int* P);
 bool tiles_valid(int n1, int n2, int R, int C, int P);
-// tuned (R, C, P, D, T) for this device and grid, if reg_autotune has measured it (D: launch with
-// PDL; T: transports in the cluster-resident kernel; T nullable)
-bool tuned_tiles(int dev, int n1, int n2, int* R, int* C, int* P, int* D, int* T);
+// The kernels a Gauss-Newton solve runs in, tuned separately: axis-wise stages (H1, shear) or stages in
+// the row spectra (H2, H3).
+enum TuneKind { TUNE_AXIS = 0, TUNE_SPECTRAL = 1 };
+inline TuneKind tune_kind(int regnorm) { return regnorm == REG_H1 ? TUNE_AXIS : TUNE_SPECTRAL; }
+struct Tuned { int R, C, P, D; };  // D: launch with PDL
+// the choice for this device, grid and kind, if it has been measured
+bool tuned_tiles(int dev, int n1, int n2, TuneKind kind, Tuned* t);
+// whether the context's Gauss-Newton transport solves are resident in one launch
+bool resident_transport(const reg_ctx* c);
+// reg_autotune of one kind; ms (nullable): < 0 for a choice measured earlier
+int autotune_kind(reg_grid grid, int nt, int concurrency, bool force, TuneKind kind, Tuned* t, double* ms);
 
 // ---- launchers (kernels.cu); all asynchronous on ctx->stream ----
 // copies the REG_TW_TOTAL twiddle entries to the device
