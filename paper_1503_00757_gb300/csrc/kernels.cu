@@ -158,32 +158,38 @@ __device__ __forceinline__ void stage_chunk(float2* dst, const float2* __restric
 // Kinds of their own: with the strides in the one-field kernels a solve's small launches were 1 to
 // 6 % slower (preconditioner at 256^2: 14.9 us with them, 14.4 without).
 enum Fields { ONE = 0, MANY = 1, TWO = 2 };
-// MANY: f floats and s spectrum entries apart
-struct Batch {
-    long long f, s;
+template <int FIELDS>
+struct Rest {};  // where the other fields are
+template <>
+struct Rest<MANY> {
+    long long f, s;  // floats and spectrum entries from field to field
+    float scale;     // of the result (k_c2r)
 };
-// TWO: the second vector field and its spectra
-struct Second {
+template <>
+struct Rest<TWO> {  // the second vector field and its spectra
     const float *f1, *f2;
     float2 *S1, *S2;
 };
 
 template <int LOGL, bool VEC, int FIELDS>
 __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const float* __restrict__ f2,
-                                             float2* S1, float2* S2, int R, const float2* __restrict__ tw, Batch bt, Second sec) {
+                                             float2* S1, float2* S2, int R, const float2* __restrict__ tw,
+                                             Rest<FIELDS> rest) {
     pdl_entry();
-    if (FIELDS == TWO && blockIdx.y) {
-        f1 = sec.f1;
-        f2 = sec.f2;
-        S1 = sec.S1;
-        S2 = sec.S2;
+    if constexpr (FIELDS == TWO) {
+        if (blockIdx.y) {
+            f1 = rest.f1;
+            f2 = rest.f2;
+            S1 = rest.S1;
+            S2 = rest.S2;
+        }
     }
-    if (FIELDS == MANY) {
-        f1 += blockIdx.y * bt.f;
-        S1 += blockIdx.y * bt.s;
+    if constexpr (FIELDS == MANY) {
+        f1 += blockIdx.y * rest.f;
+        S1 += blockIdx.y * rest.s;
         if (VEC) {
-            f2 += blockIdx.y * bt.f;
-            S2 += blockIdx.y * bt.s;
+            f2 += blockIdx.y * rest.f;
+            S2 += blockIdx.y * rest.s;
         }
     }
     extern __shared__ __align__(16) float2 sm[];
@@ -231,14 +237,14 @@ __global__ void __launch_bounds__(512) k_r2c(const float* __restrict__ f1, const
 template <int LOGL, bool VEC, int FIELDS>
 __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, const float2* __restrict__ S2,
                                              float* __restrict__ f1, float* __restrict__ f2, int R,
-                                             const float2* __restrict__ tw, Batch bt, float scale) {
+                                             const float2* __restrict__ tw, Rest<FIELDS> rest) {
     pdl_entry();
-    if (FIELDS == MANY) {
-        f1 += blockIdx.y * bt.f;
-        S1 += blockIdx.y * bt.s;
+    if constexpr (FIELDS == MANY) {
+        f1 += blockIdx.y * rest.f;
+        S1 += blockIdx.y * rest.s;
         if (VEC) {
-            f2 += blockIdx.y * bt.f;
-            S2 += blockIdx.y * bt.s;
+            f2 += blockIdx.y * rest.f;
+            S2 += blockIdx.y * rest.s;
         }
     }
     extern __shared__ __align__(16) float2 sm[];
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, cons
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int j = t + k * T;
-            if (FIELDS == MANY) x[k] = cscale(x[k], scale);
+            if constexpr (FIELDS == MANY) x[k] = cscale(x[k], rest.scale);
             if (VEC) {
                 const size_t idx = (size_t)(row0 + q) * L + j;
                 f1[idx] = x[k].x;
@@ -863,10 +869,12 @@ void launch_r2c_scalar(reg_ctx* ctx, const float* f, float2* S, int nb, long lon
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 8.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = nb > 1 ? k_r2c<LG, false, MANY> : k_r2c<LG, false, ONE>;
-        set_smem(kern, g.smem);
-        launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw,
-                 Batch{(long long)ctx->N, ss}, Second{});
+        auto go = [&](auto kern, auto rest) {
+            set_smem(kern, g.smem);
+            launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, f, nullptr, S, nullptr, g.R, ctx->tw, rest);
+        };
+        if (nb > 1) go(k_r2c<LG, false, MANY>, Rest<MANY>{ctx->N, ss, 1.f});
+        else go(k_r2c<LG, false, ONE>, Rest<ONE>{});
     });
     ktimer_end(ctx);
 }
@@ -875,10 +883,12 @@ void launch_r2c_vec(reg_ctx* ctx, const float* u1, const float* u2, float2* S1, 
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = nb > 1 ? k_r2c<LG, true, MANY> : k_r2c<LG, true, ONE>;
-        set_smem(kern, g.smem);
-        launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, u1, u2, S1, S2, g.R, ctx->tw,
-                 Batch{2LL * ctx->N, (long long)ctx->N}, Second{});
+        auto go = [&](auto kern, auto rest) {
+            set_smem(kern, g.smem);
+            launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, u1, u2, S1, S2, g.R, ctx->tw, rest);
+        };
+        if (nb > 1) go(k_r2c<LG, true, MANY>, Rest<MANY>{2LL * ctx->N, ctx->N, 1.f});
+        else go(k_r2c<LG, true, ONE>, Rest<ONE>{});
     });
     ktimer_end(ctx);
 }
@@ -889,8 +899,8 @@ void launch_r2c_two(reg_ctx* ctx, const float* u, const float* b, float2* const*
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_r2c<LG, true, TWO>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, dim3(g.grid, 2), g.threads, g.smem, u, u + ctx->N, S[0], S[1], g.R, ctx->tw, Batch{0, 0},
-                 Second{b, b + ctx->N, S[2], S[3]});
+        launch_k(ctx, kern, dim3(g.grid, 2), g.threads, g.smem, u, u + ctx->N, S[0], S[1], g.R, ctx->tw,
+                 Rest<TWO>{b, b + ctx->N, S[2], S[3]});
     });
     ktimer_end(ctx);
 }
@@ -901,7 +911,7 @@ void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f) {
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_c2r<LG, false, ONE>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, S, nullptr, f, nullptr, g.R, ctx->tw, Batch{0, 0}, 1.f);
+        launch_k(ctx, kern, g.grid, g.threads, g.smem, S, nullptr, f, nullptr, g.R, ctx->tw, Rest<ONE>{});
     });
     ktimer_end(ctx);
 }
@@ -911,10 +921,12 @@ void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1,
     const RowCfg g = row_cfg(ctx);
     ktimer_begin(ctx, KC_ROW, 16.0 * nb * ctx->N);
     DISPATCH_LOG(ctx->log2, {
-        auto kern = nb > 1 || scale != 1.f ? k_c2r<LG, true, MANY> : k_c2r<LG, true, ONE>;
-        set_smem(kern, g.smem);
-        launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, S1, S2, u1, u2, g.R, ctx->tw,
-                 Batch{2LL * ctx->N, ss > 0 ? ss : (long long)ctx->N}, scale);
+        auto go = [&](auto kern, auto rest) {
+            set_smem(kern, g.smem);
+            launch_k(ctx, kern, dim3(g.grid, nb), g.threads, g.smem, S1, S2, u1, u2, g.R, ctx->tw, rest);
+        };
+        if (nb > 1 || scale != 1.f) go(k_c2r<LG, true, MANY>, Rest<MANY>{2LL * ctx->N, ss > 0 ? ss : ctx->N, scale});
+        else go(k_c2r<LG, true, ONE>, Rest<ONE>{});
     });
     ktimer_end(ctx);
 }
@@ -923,8 +935,8 @@ cudaError_t rebind_c2r_vec(cudaGraphExec_t exec, cudaGraphNode_t node, float* u1
     cudaKernelNodeParams p;
     const cudaError_t e = cudaGraphKernelNodeGetParams(node, &p);
     if (e != cudaSuccess) return e;
-    void* args[8];  // k_c2r's parameters
-    for (int i = 0; i < 8; ++i) args[i] = p.kernelParams[i];
+    void* args[7];  // k_c2r's parameters
+    for (int i = 0; i < 7; ++i) args[i] = p.kernelParams[i];
     args[2] = &u1;
     args[3] = &u2;
     p.kernelParams = args;
