@@ -245,7 +245,10 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     cudaMemset(c->mR, 0, sizeof(float) * N);
     {
         const double one = 1.0;  // the unit denominator of device-scalar-scaled updates
-        if (cudaMemcpy(c->d_scal + SL_ONE, &one, sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
+        // a copy from pageable memory may return once its data is staged, and the first kernels may run
+        // on a stream that is not ordered after the legacy stream: wait for all of the set-up
+        if (cudaMemcpy(c->d_scal + SL_ONE, &one, sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaStreamSynchronize(0) != cudaSuccess) {
             reg_destroy(c);
             return reg_fail(REG_ERR_CUDA, "scalar upload failed");
         }

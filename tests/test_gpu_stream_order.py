@@ -43,3 +43,30 @@ def test_3d_context_is_ready_when_created():
         assert idle, "the set-up's copy was still in flight"
         assert torch.equal(g, again)
     assert all(torch.equal(outs[0], o) for o in outs[1:])
+
+
+def test_2d_context_is_ready_when_created():
+    """The same for 2-D contexts: the shear model with a mass source reads a scalar that the
+    constructor uploads last."""
+    import torch
+    from paper_1503_00757_gb300.binding import Context
+    n, nt = 32, 1
+    rng = np.random.default_rng(12)
+    mT, mR = (to_gpu(rng.random((n, n))) for _ in range(2))
+    v = to_gpu(0.05 * rng.standard_normal((2, n, n)))
+    s = torch.cuda.Stream()
+    outs = []
+    for _ in range(16):
+        g, again = torch.empty(2, n, n, device="cuda"), torch.empty(2, n, n, device="cuda")
+        torch.cuda.synchronize()
+        ctx = Context(n, n, nt, beta=1e-2, gamma=1e-3, shear=0.5, stream=s)
+        idle = torch.cuda.default_stream().query()
+        ctx.set_images(mT, mR)
+        ctx.gradient(v, g)
+        ctx.gradient(v, again)
+        torch.cuda.synchronize()
+        ctx.close()
+        assert idle, "the set-up's copy was still in flight"
+        assert torch.equal(g, again)
+        outs.append(g)
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
