@@ -375,22 +375,17 @@ struct Io {
     const float* src;
 };
 
-// after a capture with io: the sequence is a chain, so the nodes are its root and its leaf
-static bool find_io(GraphEntry& g, const Io& io) {
-    size_t n = 1;
-    if (io.in && (cudaGraphGetRootNodes(g.graph, &g.in_node, &n) != cudaSuccess || n != 1)) return false;
-    if (io.out) {
-        if (cudaGraphGetNodes(g.graph, nullptr, &n) != cudaSuccess) return false;
-        std::vector<cudaGraphNode_t> nodes(n);
-        if (cudaGraphGetNodes(g.graph, nodes.data(), &n) != cudaSuccess) return false;
-        for (cudaGraphNode_t v : nodes) {
-            cudaGraphNode_t after[2];
-            cudaGraphEdgeData edge[2];  // the programmatic edges carry data, which a query has to take
-            size_t next = 2;
-            if (cudaGraphNodeGetDependentNodes(v, after, edge, &next) != cudaSuccess) return false;
-            if (next == 0) g.out_node = v;
-        }
-    }
+// at the end of a capture with io: the sequence is a chain, so the nodes are its root and the one that
+// the next launch would depend on
+static bool find_io(GraphEntry& g, const Io& io, cudaStream_t capture) {
+    cudaStreamCaptureStatus s;
+    cudaGraph_t graph = nullptr;
+    const cudaGraphNode_t* last = nullptr;
+    const cudaGraphEdgeData* edge = nullptr;  // the programmatic edges carry data, which the query has to take
+    size_t n = 0;
+    if (cudaStreamGetCaptureInfo(capture, &s, nullptr, &graph, &last, &edge, &n) != cudaSuccess || n != 1) return false;
+    g.out_node = *last;
+    if (io.in && (cudaGraphGetRootNodes(graph, &g.in_node, &n) != cudaSuccess || n != 1)) return false;
     g.in = io.in;
     g.out = io.out;
     return true;
@@ -496,6 +491,7 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         return reg_fail(REG_ERR_CUDA, std::string("stream capture: ") + cudaGetErrorString(e));
     }
     body();
+    const bool bound = io.in || io.out, found = !bound || find_io(*seq, io, c->stream);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(c->stream, &graph);
     c->stream = user;
@@ -506,16 +502,13 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         return reg_fail(REG_ERR_CUDA, std::string("stream capture failed: ") + cudaGetErrorString(e));
     }
     seq->nkern = nk;
-    seq->graph = graph;
-    e = cudaGraphInstantiate(&seq->exec, graph, 0);
-    if (e != cudaSuccess) seq->exec = nullptr;
-    const bool found = e != cudaSuccess || find_io(*seq, io);
-    if (e != cudaSuccess || !found || !(io.in || io.out)) {
-        cudaGraphDestroy(seq->graph);
-        seq->graph = nullptr;
+    e = found ? cudaGraphInstantiate(&seq->exec, graph, 0) : cudaErrorInvalidValue;
+    if (e == cudaSuccess && bound) seq->graph = graph;
+    else cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+        seq->exec = nullptr;
+        return reg_fail(REG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
     }
-    if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    if (!found) return reg_fail(REG_ERR_CUDA, "graph nodes of the caller's fields");
     CK(cudaGraphLaunch(seq->exec, c->stream));
     c->launches += nk;
     return REG_OK;
