@@ -749,7 +749,7 @@ static void state_solve_sp(reg_ctx* c, const float* v, int nt, const float* m0) 
     for (int j = 0; j < nt; ++j) {
         launch_col(c, OP_GRAD1, in, G, P, nullptr);
         AdvArgs a = {};
-        a.G1 = c->S[1]; a.G2 = nullptr; a.Sd2 = c->S[0];
+        a.G1 = c->S[1]; a.Sd2 = c->S[0];
         a.uj = mh(c, j); a.us = nullptr; a.v = v;
         a.gm = nullptr; a.vt = nullptr;
         a.u_out = c->w0; a.grad_out = gmh(c, j); a.S_out = c->S[0];
@@ -771,7 +771,7 @@ static void adjoint_solve_sp(reg_ctx* c, const float* v, int nt, const float* a,
     const float h = 1.0f / (float)nt;
     float* lst = c->w2;
     auto lam_at = [&](int j) { return lhist ? lhist + (size_t)j * c->N : c->w1; };
-    launch_adj_init_sp(c, a, ca, cf, cb, v, lam_at(nt), bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2], nullptr);
+    launch_adj_init_sp(c, a, ca, cf, cb, v, lam_at(nt), bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2]);
     const float2* Fin[2] = {c->S[1], c->S[2]};
     float2* D[1] = {c->S[0]};
     const SpecParams P = spec_params(c, 0.f);
@@ -798,7 +798,7 @@ static void inc_adjoint_full_sp(reg_ctx* c, const float* v, const float* vt, int
     const float h = 1.0f / (float)nt;
     float* lam = c->w1;
     float* lst = c->w2;
-    launch_adj_init_sp(c, nullptr, 0.f, c->w3, -1.f, v, lam, bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2], nullptr,
+    launch_adj_init_sp(c, nullptr, 0.f, c->w3, -1.f, v, lam, bout, gmh(c, nt), 0.5f * h, c->S[1], c->S[2],
                     lamh(c, nt), vt, gmth(c, nt));
     const float2* Fin[2] = {c->S[1], c->S[2]};
     float2* D[1] = {c->S[0]};

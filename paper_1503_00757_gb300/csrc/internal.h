@@ -204,8 +204,8 @@ void launch_adj_init(reg_ctx* ctx, const float* a, float ca, const float* c, flo
 
 // RK2 stages in the row spectra (kernels.cu)
 struct AdvArgs {
-    const float2 *G1, *G2;  // spectra of d1 u_s, d2 u_s; G1 == nullptr -> zero gradient
-    const float2* Sd2;      // G2 == nullptr: row spectrum of u_s, d2 u_s = (i k2~ / n2) Sd2
+    const float2* G1;       // spectrum of d1 u_s; nullptr -> zero gradient
+    const float2* Sd2;      // row spectrum of u_s: d2 u_s = (i k2~ / n2) Sd2
     const float *uj, *us;   // u_j (nullptr: u_j = 0) and the stage-2 input u* (stage 1: us unused)
     const float* v;         // velocity (2N)
     const float* gm;        // grad m at the source time (2N); nullptr -> no source
@@ -238,12 +238,11 @@ struct AdjArgs {
 };
 void launch_row_adj(reg_ctx* ctx, const AdjArgs& a);
 
-// lam = ca * a + cb * c (a nullable); b = w lam gm; flux spectra of lam v;
-// optional FP64 partials of 0.5 * sum(lam^2) * h1 h2.  Full Newton (lsrc != nullptr):
-// b += w lsrc gmt and the flux is lam v + lsrc vt.
+// lam = ca * a + cb * c (a nullable); b = w lam gm; flux spectra of lam v.  Full Newton
+// (lsrc != nullptr): b += w lsrc gmt and the flux is lam v + lsrc vt.
 void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, const float* v,
-                     float* lam, float* b, const float* gm, float w, float2* F1, float2* F2, double* part,
-                     const float* lsrc = nullptr, const float* vt = nullptr, const float* gmt = nullptr);
+                        float* lam, float* b, const float* gm, float w, float2* F1, float2* F2,
+                        const float* lsrc = nullptr, const float* vt = nullptr, const float* gmt = nullptr);
 
 // ---- pointwise / reductions ----
 // d_scal[slot] = scale * sum_i x_i y_i over n elements; the same of (x_i - y_i)^2

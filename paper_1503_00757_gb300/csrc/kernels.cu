@@ -1,9 +1,13 @@
 // CUDA kernels (sm_103a) for the pseudospectral Gauss-Newton-Krylov
 // registration solver of Mang & Biros (arXiv 1503.00757).
 //
+// The operators that couple the axes (regularization, projection, preconditioner, filters, energies) and
+// the transport stages of H2 and H3 problems; the transport of H1 problems takes its derivatives axis
+// by axis (transport.cu).
+//
 // A 2-D transform of an n1 x n2 real field is split into two passes over HBM:
 //   * row kernels: one CTA owns R consecutive rows; real FFTs along x^2
-//     (two real rows, or two real fields of one row, per complex FFT), fused
+//     (two real rows, or two real fields of one row, per complex FFT), in the H2 / H3 stages fused
 //     with the pointwise work of an RK2 stage (Sec. 4) on the physical side;
 //   * column kernels: one CTA owns C consecutive columns of the packed half
 //     spectra (row-quad tiled layout, see fft_reg.cuh); forward FFT along x^1,
@@ -291,13 +295,13 @@ __global__ void __launch_bounds__(512) k_c2r(const float2* __restrict__ S1, cons
 // amplify a change of rounding by 10^3 to 10^5 (the velocities of two 128^2 H2 solves, beta_v =
 // 1e-3, stopped after the same two Newton steps, differ by 1e-5 to 1e-1 when the last bits of b~
 // do), so they keep the arithmetic that their users' results came from.
-// ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
+//
 // RK2 (Heun) advection stage of the state and incremental state equations
 // (Eq. (e:state-eq-elim), (e:inc-state-eq-elim)):
 //   k = -v . grad u_s - v~ . grad m(t)         (source only for the incremental state)
 //   stage 1: u* = u_j + h k ;  stage 2: u_{j+1} = (u_j + u* + h k) / 2
-// grad u_s arrives as packed spectra (G1, G2) from the column pass; the stage
+// d1 u_s arrives as a packed spectrum (G1) from the column pass, d2 u_s is diagonal
+// in the row spectrum of u_s (Sd2); the stage
 // result u_out leaves as its packed spectrum S_out for the next column pass.
 // ---------------------------------------------------------------------------
 template <int LOGL, bool PRE>
@@ -334,16 +338,11 @@ __global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adv_sp(AdvAr
     float2 x[8];
     if (a.G1) {
         stage_chunk<LOGL>(A, a.G1 + base, R * W);
-        stage_chunk<LOGL>(A + R * W, (a.G2 ? a.G2 : a.Sd2) + base, R * W);
+        stage_chunk<LOGL>(A + R * W, a.Sd2 + base, R * W);
         __syncthreads();
-        if (a.G2) {
+        const float c = 1.0f / (float)L;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) x[k] = merged_entry<LOGL>(A, q, A + R * W, q, t + k * T);
-        } else {
-            const float c = 1.0f / (float)L;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) x[k] = merged_entry_d2<LOGL>(A, q, A + R * W, q, t + k * T, c);
-        }
+        for (int k = 0; k < 8; ++k) x[k] = merged_entry_d2<LOGL>(A, q, A + R * W, q, t + k * T, c);
         reg_fft<LOGL, true>(x, t, true, X + 2 * q * fft_buf(L), X + 2 * q * fft_buf(L) + fft_buf(L), tw);
     } else {
 #pragma unroll
@@ -520,13 +519,13 @@ __global__ void __launch_bounds__(512, RowBlocks<PRE>::value) k_row_adj_sp(AdjAr
     flux_fft_store<LOGL>(x, q, t, R, row0, A, X, a.F1, a.F2, tw);
 }
 
-// lam = ca*a + cb*c; b = w lam gm; flux spectra; partial 0.5*sum(lam^2).  With lsrc (full
+// lam = ca*a + cb*c; b = w lam gm; flux spectra.  With lsrc (full
 // Newton): b += w lsrc gmt and the flux is lam v + lsrc v~.
 template <int LOGL>
 __global__ void __launch_bounds__(512) k_adj_init_sp(const float* __restrict__ a, float ca, const float* __restrict__ c,
                                                   float cb, const float* __restrict__ v, float* lam, float* b,
                                                   const float* __restrict__ gm, float w, float2* F1, float2* F2,
-                                                  double* part, int N, int R, const float2* __restrict__ tw,
+                                                  int N, int R, const float2* __restrict__ tw,
                                                   const float* __restrict__ lsrc, const float* __restrict__ vt,
                                                   const float* __restrict__ gmt) {
     pdl_entry();
@@ -537,7 +536,6 @@ __global__ void __launch_bounds__(512) k_adj_init_sp(const float* __restrict__ a
     const int q = threadIdx.x / T, t = threadIdx.x - q * T;
     const int row0 = blockIdx.x * R;
     const size_t rowbase = (size_t)(row0 + q) * L;
-    double acc = 0.0;
     float2 x[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -545,7 +543,6 @@ __global__ void __launch_bounds__(512) k_adj_init_sp(const float* __restrict__ a
         float l = cb * c[idx];
         if (a) l = fmaf(ca, a[idx], l);
         lam[idx] = l;
-        acc += 0.5 * (double)l * (double)l;
         if (lsrc) {
             const float ls = lsrc[idx];
             b[idx] = fmaf(w * ls, gmt[idx], w * l * gm[idx]);
@@ -556,10 +553,6 @@ __global__ void __launch_bounds__(512) k_adj_init_sp(const float* __restrict__ a
             b[N + idx] = w * l * gm[N + idx];
             x[k] = make_float2(l * v[idx], l * v[N + idx]);
         }
-    }
-    if (part) {
-        const double s = block_reduce<0>(acc);
-        if (threadIdx.x == 0) part[blockIdx.x] = s;
     }
     flux_fft_store<LOGL>(x, q, t, R, row0, A, X, F1, F2, tw);
 }
@@ -816,7 +809,7 @@ __global__ void __launch_bounds__(256) k_col(ColArgs a, const float2* __restrict
 // launch helpers
 // ---------------------------------------------------------------------------
 // Default tile choices.  R rows per row CTA: a multiple of 4 with at least 64
-// transform entries in flight per 8 (T = L/8 per row); C columns per column CTA: at least 4 where
+// threads (L / 8 per row); C columns per column CTA: at least 4 where
 // that fits 256 threads (32-byte sectors of the transport's fields; 512^2 matvec, nt = 16: 364 us
 // against 395 us with 2, 256^2: 281 against 285) and 64 threads.  reg_autotune may replace both per
 // grid.
@@ -975,16 +968,16 @@ void launch_row_adj(reg_ctx* ctx, const AdjArgs& a) {
 }
 
 void launch_adj_init_sp(reg_ctx* ctx, const float* a, float ca, const float* c, float cb, const float* v, float* lam,
-                     float* b, const float* gm, float w, float2* F1, float2* F2, double* part, const float* lsrc,
-                     const float* vt, const float* gmt) {
+                        float* b, const float* gm, float w, float2* F1, float2* F2, const float* lsrc,
+                        const float* vt, const float* gmt) {
     const RowCfg g = row_cfg(ctx);
     // a 1 (optional), c 1, v 2, lam 1, b 2 + gm 2, flux spectra 2; full Newton: lsrc 1, v~ 2, grad m~ 2
     ktimer_begin(ctx, KC_ROW, 4.0 * ((a ? 1 : 0) + 1 + 2 + 1 + 4 + 2 + (lsrc ? 5 : 0)) * ctx->N);
     DISPATCH_LOG(ctx->log2, {
         auto kern = k_adj_init_sp<LG>;
         set_smem(kern, g.smem);
-        launch_k(ctx, kern, g.grid, g.threads, g.smem, a, ca, c, cb, v, lam, b, gm, w, F1, F2, part, ctx->N, g.R,
-                 ctx->tw, lsrc, vt, gmt);
+        launch_k(ctx, kern, g.grid, g.threads, g.smem, a, ca, c, cb, v, lam, b, gm, w, F1, F2, ctx->N, g.R, ctx->tw,
+                 lsrc, vt, gmt);
     });
     ktimer_end(ctx);
 }

@@ -31,17 +31,12 @@
 
 #include "deriv.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 namespace {
 
 constexpr int R3_THREADS = 256;
 constexpr int R3_BLOCKS = 608;  // 4 per SM of a GB300 for the grid-stride kernels
-
-// see kernels.cu: wait for the preceding kernel, then let the next one start launching
-__device__ __forceinline__ void pdl_entry() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 
 struct Dims3 {
     int n1, n2, n3;
@@ -441,8 +436,7 @@ struct Row3 { int lines, threads, grid; size_t smem; };
 Row3 row3(const Dims3& D) {
     Row3 r;
     const int T = D.n3 / 8, pairs = D.n1 * D.n2 / 2;
-    int th = D.N >= (1 << 18) ? 128 : 64;
-    if (th < 32) th = 32;
+    const int th = D.N >= (1 << 18) ? 128 : 64;
     r.lines = th / T;
     if (r.lines > pairs) r.lines = pairs;
     r.threads = r.lines * T;
