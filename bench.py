@@ -84,9 +84,16 @@ def matvec_models(n1, n2, nt, ms, hbm_gbs, fp32_tflops):
     time steps, against two byte models and an FFT flop model (N = n1 n2 nodes, FP32):
       streaming  (24 nt + 40) N bytes: a time step fully on chip, so that each of the two
                  sweeps reads the state history once and round-trips one state per step;
+      axis_pass  168 nt N bytes: what the axis-wise stages of H1 problems move, every launch's
+                 inputs and outputs through memory: per step 42 fields, namely 2 per column
+                 launch of the incremental state and 3 of the adjoint (its factor v_1), 6 and 4 per
+                 stage-1 row launch, 11 and 11 per stage-2 row launch (the launchers' tallies);
+      axis_flops the transforms of those stages: a pair over n2/2 packed columns and one over
+                 n1/2 packed pairs of rows per stage, 5 N (log2 n1 + log2 n2);
       fft_pass   280 nt N bytes: every 2-D FFT pass (about 15 real 2-D transforms per step,
-                 16 N bytes each) and the pointwise work (about 40 N) through memory;
-      flops      the transforms of the 4 nt RK2 stages (incremental state and adjoint, two
+                 16 N bytes each) and the pointwise work (about 40 N) through memory, as the
+                 stages in the row spectra (H2, H3) do;
+      flops      those stages' transforms: the transforms of the 4 nt RK2 stages (incremental state and adjoint, two
                  stages per step), 5 n log2 n flop per complex transform of length n: per
                  stage one column transform pair over n2/2 spectrum columns (5 N log2 n1)
                  and 1.5 row transforms' worth over the n1 rows (7.5 N log2 n2).
@@ -94,12 +101,13 @@ def matvec_models(n1, n2, nt, ms, hbm_gbs, fp32_tflops):
     N = n1 * n2
     sec = ms * 1e-3
     out = {"ms_per_matvec": ms}
-    for name, byt in (("streaming", (24 * nt + 40) * N), ("fft_pass", 280 * nt * N)):
+    for name, byt in (("streaming", (24 * nt + 40) * N), ("axis_pass", 168 * nt * N), ("fft_pass", 280 * nt * N)):
         gbs = byt / sec / 1e9
         out[name] = {"bytes": byt, "GB/s": gbs, "frac_hbm": gbs / hbm_gbs}
-    fl = 4 * nt * (5 * math.log2(n1) + 7.5 * math.log2(n2)) * N
-    tf = fl / sec / 1e12
-    out["flops"] = {"flop": fl, "TFLOP/s": tf, "frac_fp32": (tf / fp32_tflops) if fp32_tflops else None}
+    for name, rows in (("axis_flops", 5.0), ("flops", 7.5)):
+        fl = 4 * nt * (5 * math.log2(n1) + rows * math.log2(n2)) * N
+        tf = fl / sec / 1e12
+        out[name] = {"flop": fl, "TFLOP/s": tf, "frac_fp32": (tf / fp32_tflops) if fp32_tflops else None}
     return out
 
 
@@ -112,10 +120,10 @@ def stream_bytes(n1, n2, nt):
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per Gauss-Newton matvec at 512^2,
-# nt = 32, summed over its 260 launches from one ncu capture of the current kernels (ncu flushes
+# nt = 32, summed over its 259 kernel launches from one ncu capture (axis-wise kernel pairs; ncu flushes
 # the caches before each launch, so this is the cold-cache traffic; command in the profiles
 # folder's matvec traffic summary).
-MATVEC_TRAFFIC_512 = 1.2932e9
+MATVEC_TRAFFIC_512 = 1.0577e9
 
 
 def roofline(bytes_per_matvec, conc, ms_single, peak, peak_kind):

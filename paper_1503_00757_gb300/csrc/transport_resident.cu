@@ -14,6 +14,9 @@
 // 128^2, nt = 16; two roles: 208; kernel pairs: 318).  Bound by the latency of one transform pair
 // and two cluster barriers a stage, about 2.3 us.  At 256^2 the 16 SMs of the largest cluster compute
 // as long as the kernel pairs wait (302 against 301 us a matvec, nt = 16), so the line is below it.
+// Matvecs, nt = 16, us each, resident against pairs, for one solve and for 32 at once: 64^2 103 / 213
+// and 5.4 / 28.7, 64 x 256 119 / 275 and 11.7 / 29.6, 256 x 64 146 / 252 and 14.7 / 29.8, 128^2 135 /
+// 277 and 13.6 / 30.6, 128 x 256 160 / 285 and 22.4 / 31.0, 256 x 128 178 / 279 and 26.2 / 31.5.
 #include <map>
 #include <mutex>
 

@@ -10,7 +10,7 @@
 // spectra stay in shared memory; the column pass gathers its C = n2 / (2 CS) columns from the row
 // owners over distributed shared memory and scatters the result back (two cluster barriers a
 // stage instead of two launches of about 9 us together at 128^2; eight mixed 128^2 pairs, two
-// Newton steps each: 14.1 ms with the launches, 8.1 ms).  Bound by latency, like transport_resident.cu.
+// Newton steps each: 13.5 to 16 ms with the launches, 8.2 to 9.5 ms).  Bound by latency, like transport_resident.cu.
 #include <map>
 #include <mutex>
 
