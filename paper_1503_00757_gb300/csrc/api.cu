@@ -14,6 +14,7 @@
 #include "deriv.cuh"
 #include "fft.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 static thread_local std::string g_err = "no error";
 
@@ -77,7 +78,7 @@ static void clear_graphs(reg_ctx* c) {
 }
 
 static void free_hist(reg_ctx* c) {
-    clear_graphs(c);  // captured sequences hold history pointers
+    clear_graphs(c);  // the graphs hold history pointers
     cudaFree(c->m_hist);
     cudaFree(c->gm_hist);
     cudaFree(c->lam_hist);
@@ -121,7 +122,6 @@ extern "C" void reg_destroy(reg_ctx* c) {
     if (!c) return;
     free_hist(c);
     clear_graphs(c);
-    if (c->cap) cudaStreamDestroy(c->cap);
     for (auto g : c->timing_graphs) cudaGraphExecDestroy(g);
     cudaFree(c->slab);
     cudaFreeHost(c->h_scal);
@@ -185,7 +185,7 @@ extern "C" int reg_create(reg_grid grid, int nt, int regnorm, double beta, doubl
     c->nt_cap = 0;
     set_params(c, nt, regnorm, beta, gamma, shear);
     c->stream = 0;
-    c->cap = nullptr;
+    c->build = nullptr;
     c->launches = 0;
     c->tiles_set = c->pdl_set = false;
     c->tc_ok = tc_max_active_clusters(c->n1, c->n2) > 0;
@@ -262,7 +262,7 @@ extern "C" int reg_set_params(reg_ctx* c, int nt, int regnorm, double beta, doub
     RET(check_params(nt, regnorm, beta, gamma, shear));
     const bool same = nt == c->nt && regnorm == c->regnorm && beta == c->beta_v && gamma == c->beta_w &&
                       shear == c->shear;
-    if (!same) clear_graphs(c);  // captured sequences bake in nt and the Fourier-multiplier parameters
+    if (!same) clear_graphs(c);  // the graphs bake in nt and the Fourier-multiplier parameters
     const bool other = tune_kind(regnorm) != tune_kind(c->regnorm);
     set_params(c, nt, regnorm, beta, gamma, shear);
     if (other) apply_tuned(c);
@@ -280,7 +280,7 @@ extern "C" int reg_set_tiles(reg_ctx* c, int rows_per_cta, int cols_per_cta, int
     if (!tiles_valid(c->n1, c->n2, rows_per_cta, cols_per_cta, prefetch))
         return reg_fail(REG_ERR_ARG, "tiles outside the launch limits of this grid");
     if (rows_per_cta != c->tileR || cols_per_cta != c->tileC || prefetch != c->tileP)
-        clear_graphs(c);  // captures bake in launch shapes and kernels
+        clear_graphs(c);  // the graphs bake in launch shapes and kernels
     c->tiles_set = true;
     c->tileR = rows_per_cta;
     c->tileC = cols_per_cta;
@@ -289,7 +289,7 @@ extern "C" int reg_set_tiles(reg_ctx* c, int rows_per_cta, int cols_per_cta, int
 }
 
 static void set_transport(reg_ctx* c, bool tc, bool rs) {
-    if (tc != c->use_tc || rs != c->use_rs) clear_graphs(c);  // captures bake in the kernels
+    if (tc != c->use_tc || rs != c->use_rs) clear_graphs(c);  // the graphs bake in the kernels
     c->use_tc = tc;
     c->use_rs = rs;
 }
@@ -312,7 +312,7 @@ extern "C" int reg_set_hessian(reg_ctx* c, int full) {
     if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
     const bool on = full != 0;
     if (on == c->full_newton) return REG_OK;
-    clear_graphs(c);  // captures bake in the matvec's launch sequence
+    clear_graphs(c);  // the graphs bake in the matvec's launch sequence
     c->have_lin = false;  // the adjoint history belongs to the next reg_gradient
     c->full_newton = on;
     if (on) return alloc_newton_hist(c);
@@ -333,7 +333,7 @@ extern "C" int reg_transport_config(reg_ctx* c, int* cluster, int* ctas_per_clus
 extern "C" int reg_set_pdl(reg_ctx* c, int enable) {
     if (!c) return reg_fail(REG_ERR_ARG, "ctx is NULL");
     const bool on = enable != 0;
-    if (on != c->pdl) clear_graphs(c);  // captures bake in the launch attribute
+    if (on != c->pdl) clear_graphs(c);  // the graphs bake in the launch attribute
     c->pdl_set = true;
     c->pdl = on;
     return REG_OK;
@@ -348,16 +348,14 @@ extern "C" int reg_set_stream(reg_ctx* c, void* stream) {
 
 // ---------------------------------------------------------------------------
 // CUDA graphs: each fixed launch sequence (objective, gradient tail, matvec,
-// one PCG iteration, det F, displacement) is captured once per (kind, internal
+// one PCG iteration, det F, displacement) is built once per (kind, internal
 // pointers, nt) and replayed.  The sequences work on the context's buffers: a
 // caller's field is copied in by the first node, or before, and the caller's
 // buffer is written by the last node, or after; the two nodes are pointed at the
-// buffers of each call (Io), so new buffers cost nothing.  The legacy
-// default stream cannot be captured: its sequences are captured on a stream of
-// the context's own and replayed on the legacy stream.  Capture and instantiation
-// cost 60 to 150 us and a replay gains 5 to 20 us over direct launches, so on that
-// stream (and for the displacement and label solves on any) a sequence is launched
-// directly the first DIRECT_CALLS times.  While per-kernel timing is on sequences run directly
+// buffers of each call (Io), so new buffers cost nothing.  Building and instantiating
+// cost 60 to 150 us and a replay gains 5 to 20 us over direct launches, so on the
+// legacy default stream (and for the displacement and label solves on any) a sequence is
+// launched directly the first DIRECT_CALLS times.  While per-kernel timing is on sequences run directly
 // (legacy stream) or with event nodes.
 // ---------------------------------------------------------------------------
 enum GraphKind {
@@ -375,23 +373,7 @@ struct Io {
     const float* src;
 };
 
-// at the end of a capture with io: the sequence is a chain, so the nodes are its root and the one that
-// the next launch would depend on
-static bool find_io(GraphEntry& g, const Io& io, cudaStream_t capture) {
-    cudaStreamCaptureStatus s;
-    cudaGraph_t graph = nullptr;
-    const cudaGraphNode_t* last = nullptr;
-    const cudaGraphEdgeData* edge = nullptr;  // the programmatic edges carry data, which the query has to take
-    size_t n = 0;
-    if (cudaStreamGetCaptureInfo(capture, &s, nullptr, &graph, &last, &edge, &n) != cudaSuccess || n != 1) return false;
-    g.out_node = *last;
-    if (io.in && (cudaGraphGetRootNodes(graph, &g.in_node, &n) != cudaSuccess || n != 1)) return false;
-    g.in = io.in;
-    g.out = io.out;
-    return true;
-}
-
-// points the nodes of a captured sequence at this call's fields
+// points the first and the last node of a sequence's graph at this call's fields
 static bool bind_io(reg_ctx* c, GraphEntry& g, const Io& io) {
     const size_t bytes = sizeof(float) * 2 * c->N;
     if (io.in != g.in) {
@@ -415,10 +397,10 @@ static bool capturing(const reg_ctx* c) {
     return c->stream != 0 && cudaStreamIsCapturing(c->stream, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
 }
 
-// first objective of a fresh context, 256^2, H1, nt = 8: 262 us captured, 135 us directly
+// first objective of a fresh context, 256^2, H1, nt = 8: 262 us as a graph, 135 us directly
 constexpr int DIRECT_CALLS = 10;
 
-// Calls that replay a captured sequence cannot go into a caller's capture: refused before anything of
+// Calls that replay a graph cannot go into a caller's capture: refused before anything of
 // the context, or of the caller's graph, changes.
 static int refuse_capture(const reg_ctx* c) {
     return capturing(c) ? reg_fail(REG_ERR_CUDA, "the context's stream is being captured") : REG_OK;
@@ -465,7 +447,7 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         return REG_OK;
     }
     if (!seq) {
-        if (c->graphs.size() >= 64) {  // callers that pass many distinct pointers: drop the oldest capture
+        if (c->graphs.size() >= 64) {  // callers that pass many distinct pointers: drop the oldest graph
             drop_graph(c->graphs.front());
             c->graphs.erase(c->graphs.begin());
         }
@@ -480,35 +462,30 @@ static int run_seq(reg_ctx* c, int kind, const void* p0, const void* p1, int nt,
         return REG_OK;
     }
     const long long l0 = c->launches;
-    const cudaStream_t user = c->stream;
-    if (user == 0) {
-        if (!c->cap) CK(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
-        c->stream = c->cap;
-    }
-    cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed);
-    if (e != cudaSuccess) {
-        c->stream = user;
-        return reg_fail(REG_ERR_CUDA, std::string("stream capture: ") + cudaGetErrorString(e));
-    }
+    GraphBuild b;
+    CK(cudaGraphCreate(&b.graph, 0));
+    c->build = &b;
     body();
-    const bool bound = io.in || io.out, found = !bound || find_io(*seq, io, c->stream);
-    cudaGraph_t graph = nullptr;
-    e = cudaStreamEndCapture(c->stream, &graph);
-    c->stream = user;
+    c->build = nullptr;
     const long long nk = c->launches - l0;
     c->launches = l0;
-    if (e != cudaSuccess || graph == nullptr) {
-        cudaGetLastError();
-        return reg_fail(REG_ERR_CUDA, std::string("stream capture failed: ") + cudaGetErrorString(e));
+    cudaError_t e = b.err;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&seq->exec, b.graph, 0);
+    if (e == cudaSuccess && (io.in || io.out)) {
+        seq->graph = b.graph;  // a chain: the copy from the caller's field is its head, the store its tail
+        seq->in_node = b.head;
+        seq->out_node = b.tail;
+        seq->in = io.in;
+        seq->out = io.out;
+    } else {
+        cudaGraphDestroy(b.graph);
     }
-    seq->nkern = nk;
-    e = found ? cudaGraphInstantiate(&seq->exec, graph, 0) : cudaErrorInvalidValue;
-    if (e == cudaSuccess && bound) seq->graph = graph;
-    else cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
         seq->exec = nullptr;
-        return reg_fail(REG_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+        cudaGetLastError();
+        return reg_fail(REG_ERR_CUDA, std::string("graph: ") + cudaGetErrorString(e));
     }
+    seq->nkern = nk;
     CK(cudaGraphLaunch(seq->exec, c->stream));
     c->launches += nk;
     return REG_OK;
@@ -563,7 +540,7 @@ static bool overlap(const float* a, size_t na, const float* b, size_t nb) { retu
 static void sp_grad(reg_ctx* c, const float* f, float* out) {
     const size_t N = c->N;
     if (overlap(f, N, out, 2 * N)) {
-        cudaMemcpyAsync(c->vx, f, sizeof(float) * N, cudaMemcpyDeviceToDevice, c->stream);
+        copy_async(c->build, c->stream, c->vx, f, sizeof(float) * N);
         f = c->vx;
     }
     launch_grad(c, f, out);
@@ -581,7 +558,7 @@ static void sp_grad_spec(reg_ctx* c, const float* f, float* out) {
 static void sp_div(reg_ctx* c, const float* u, float* out) {
     const size_t N = c->N;
     if (overlap(u, 2 * N, out, N)) {  // as above
-        cudaMemcpyAsync(c->vx, u, sizeof(float) * 2 * N, cudaMemcpyDeviceToDevice, c->stream);
+        copy_async(c->build, c->stream, c->vx, u, sizeof(float) * 2 * N);
         u = c->vx;
     }
     launch_dcol(c, DColArgs{u, nullptr, nullptr, nullptr, out});
@@ -688,7 +665,7 @@ static void sp_divt_proj(reg_ctx* c, float coefA, const float* T, const float* b
 static const float* out_src(const reg_ctx* c) { return c->shear_model && c->pmode != PROJ_LERAY ? c->vtmp2 : nullptr; }
 static void finish_out(reg_ctx* c, float* out) {
     if (out_src(c))
-        cudaMemcpyAsync(out, out_src(c), sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        copy_async(c->build, c->stream, out, out_src(c), sizeof(float) * 2 * c->N);
     else if (c->shear_model)
         launch_c2r_vec(c, c->S[5], c->S[0], out, out + c->N);
     else
@@ -741,7 +718,7 @@ static void grad_end_sp(reg_ctx* c, int nt) {
 // spectra and is formed by the row kernel from the stage's own spectrum S[0].
 static void state_solve_sp(reg_ctx* c, const float* v, int nt, const float* m0) {
     const float h = 1.0f / (float)nt;
-    cudaMemcpyAsync(mh(c, 0), m0, sizeof(float) * c->N, cudaMemcpyDeviceToDevice, c->stream);
+    copy_async(c->build, c->stream, mh(c, 0), m0, sizeof(float) * c->N);
     launch_r2c_scalar(c, mh(c, 0), c->S[0]);
     const float2* in[1] = {c->S[0]};
     float2* G[1] = {c->S[1]};
@@ -1059,7 +1036,7 @@ static int objective_at(reg_ctx* c, const float* v, float* at, int nt, bool keep
     if (v == at) return objective_dev(c, at, nt, y);
     RET(ensure_nt(c, nt));
     auto body = [&] {
-        cudaMemcpyAsync(at, v, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        copy_async(c->build, c->stream, at, v, sizeof(float) * 2 * c->N);
         objective_launches(c, at, nt, y);
     };
     return run_seq(c, GK_OBJECTIVE_IN, at, y, nt, Io{v, at, nullptr, nullptr}, body, [&] {
@@ -1079,7 +1056,7 @@ static void gradient_launches(reg_ctx* c, const float* v, float* g, int nt) {
         if (c->pmode == PROJ_LERAY) {
             sp_divt_proj(c, -(float)c->beta_v, c->T3, c->bvec, g);
         } else {
-            cudaMemcpyAsync(c->T3b, c->E_lin, sizeof(float) * 3 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+            copy_async(c->build, c->stream, c->T3b, c->E_lin, sizeof(float) * 3 * c->N);
             shear_mass_assemble(c, c->T3, c->T3b, c->bvec, g ? g : c->vtmp2);
         }
     } else {
@@ -1171,7 +1148,7 @@ static int matvec_dev(reg_ctx* c, const float* vt, float* Hvt) {
     RET(refuse_capture(c));
     // Hvt may be vt: the direct launches, too, have read vt before the first store to Hvt
     auto body = [&] {
-        cudaMemcpyAsync(c->vtil, vt, sizeof(float) * 2 * c->N, cudaMemcpyDeviceToDevice, c->stream);
+        copy_async(c->build, c->stream, c->vtil, vt, sizeof(float) * 2 * c->N);
         matvec_launches(c, c->vtil, nullptr);
         finish_out(c, Hvt);
     };
@@ -1353,11 +1330,11 @@ static int pcg_dev(reg_ctx* c, double gnorm, double eta, int maxit, int* hit_max
         launch_fill(c, n2N, c->vt, 0.f);
         launch_axpby(c, n2N, -1.f, c->g, 0.f, c->r, -1, -1, c->r);  // r = -g
         if (yp) {
-            cudaMemcpyAsync(c->s, c->r, sizeof(float) * n2N, cudaMemcpyDeviceToDevice, c->stream);
+            copy_async(c->build, c->stream, c->s, c->r, sizeof(float) * n2N);
             dot_dev(c, c->r, c->r, SL_RZ);
         } else {
             precond_dev(c, c->r, c->z);
-            cudaMemcpyAsync(c->s, c->z, sizeof(float) * n2N, cudaMemcpyDeviceToDevice, c->stream);
+            copy_async(c->build, c->stream, c->s, c->z, sizeof(float) * n2N);
             dot_dev(c, c->r, c->z, SL_RZ);
         }
     }));
@@ -1381,8 +1358,7 @@ static int pcg_dev(reg_ctx* c, double gnorm, double eta, int maxit, int* hit_max
                 dot_dev(c, c->z, c->r, SL_RZNEW);
                 launch_pcg_dir(c, n2N, c->z, c->s);
             }
-            cudaMemcpyAsync(c->d_scal + SL_RZ, c->d_scal + SL_RZNEW, sizeof(double), cudaMemcpyDeviceToDevice,
-                            c->stream);
+            copy_async(c->build, c->stream, c->d_scal + SL_RZ, c->d_scal + SL_RZNEW, sizeof(double));
         });
         if (st != REG_OK) { *status = st; return it; }
         ++it;

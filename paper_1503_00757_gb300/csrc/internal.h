@@ -58,15 +58,31 @@ enum Slot {
 
 struct EventPair { cudaEvent_t a, b; int kclass; double bytes; };
 
-// A launch sequence, once captured replayed with cudaGraphLaunch.  Keyed by the
-// kind of sequence, the pointers it was captured with and nt.
+// A launch sequence that is being put into a graph instead of onto a stream, as a chain of nodes.  Built
+// node by node, not by stream capture: while a stream is captured no thread may synchronize the
+// device, and one that tries breaks the capture.
+struct GraphBuild {
+    cudaGraph_t graph = nullptr;
+    cudaGraphNode_t head = nullptr, tail = nullptr;
+    bool tail_kernel = false;
+    cudaError_t err = cudaSuccess;
+    void add(cudaError_t e, cudaGraphNode_t node, bool kernel) {
+        if (e != cudaSuccess && err == cudaSuccess) err = e;
+        if (!head) head = node;
+        tail = node;
+        tail_kernel = kernel;
+    }
+};
+
+// A launch sequence, once built as a graph replayed with cudaGraphLaunch.  Keyed by the
+// kind of sequence, the pointers it was built with and nt.
 struct GraphEntry {
     int kind;
     const void* p0;
     const void* p1;
     int nt;
-    int direct;            // times it was launched directly, before a capture
-    cudaGraphExec_t exec;  // nullptr: not captured (yet)
+    int direct;            // times it was launched directly, before a graph was built
+    cudaGraphExec_t exec;  // nullptr: no graph (yet)
     long long nkern;
     // sequences that begin with a copy from, or end with a store to, a caller's field: the graph with
     // those two nodes and the fields they were last pointed at
@@ -85,7 +101,7 @@ struct reg_ctx {
     int pmode;
     bool shear_model;
     cudaStream_t stream;
-    cudaStream_t cap;  // launch sequences are captured here when `stream` is the legacy default stream
+    GraphBuild* build;  // launches go into this graph (nullptr: onto `stream`)
 
     void* slab;  // the allocation behind every buffer below but the histories and h_scal
     // images and history
@@ -285,9 +301,9 @@ void ktimer_end(reg_ctx* ctx);
 
 int reg_fail(int status, const std::string& msg);
 
-// While it lives, this thread may instantiate and destroy graphs although another stream is being
-// captured (by any thread, in the default global mode): nothing here depends on captured work, and
-// without it the call would fail and invalidate that capture.
+// While it lives, this thread may instantiate and destroy graphs although a stream is being captured
+// (by any thread, in the default global mode): nothing here depends on captured work, and without it
+// the call would fail and invalidate that capture.
 struct GraphCalls {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     GraphCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }

@@ -24,6 +24,51 @@ __device__ __forceinline__ void pdl_entry() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Launch onto cfg.stream, or as the next node of the graph that is being built: with a programmatic
+// edge where the configuration asks for programmatic serialization and the node before is a kernel.
+template <typename... KArgs>
+static void launch_cfg(GraphBuild* b, const cudaLaunchConfig_t& cfg, void (*kern)(KArgs...), KArgs... args) {
+    if (!b) {
+        cudaLaunchKernelEx(&cfg, kern, args...);
+        return;
+    }
+    void* params[] = {(void*)&args...};
+    cudaKernelNodeParams p = {};
+    p.func = (void*)kern;
+    p.gridDim = cfg.gridDim;
+    p.blockDim = cfg.blockDim;
+    p.sharedMemBytes = (unsigned)cfg.dynamicSmemBytes;
+    p.kernelParams = params;
+    bool early = false;
+    for (unsigned i = 0; i < cfg.numAttrs; ++i)
+        early = early || (cfg.attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization &&
+                          cfg.attrs[i].val.programmaticStreamSerializationAllowed);
+    early = early && b->tail_kernel;
+    cudaGraphNode_t node = nullptr;
+    cudaError_t e = cudaGraphAddKernelNode(&node, b->graph, &b->tail, b->tail && !early ? 1 : 0, &p);
+    for (unsigned i = 0; e == cudaSuccess && i < cfg.numAttrs; ++i)
+        if (cfg.attrs[i].id == cudaLaunchAttributeClusterDimension)
+            e = cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &cfg.attrs[i].val);
+    if (e == cudaSuccess && early) {
+        cudaGraphEdgeData edge = {};
+        edge.from_port = cudaGraphKernelNodePortProgrammatic;
+        edge.type = cudaGraphDependencyTypeProgrammatic;
+        e = cudaGraphAddDependencies(b->graph, &b->tail, &node, &edge, 1);
+    }
+    b->add(e, node, true);
+}
+// the same for a copy between device buffers
+[[maybe_unused]] static void copy_async(GraphBuild* b, cudaStream_t st, void* dst, const void* src, size_t bytes) {
+    if (!b) {
+        cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st);
+        return;
+    }
+    cudaGraphNode_t node = nullptr;
+    const cudaError_t e = cudaGraphAddMemcpyNode1D(&node, b->graph, &b->tail, b->tail ? 1 : 0, dst, src, bytes,
+                                                   cudaMemcpyDeviceToDevice);
+    b->add(e, node, false);
+}
+
 // Launch with the programmatic-stream-serialization attribute (ctx->pdl) or plainly.
 template <typename... KArgs, typename... Args>
 static void launch_k(reg_ctx* ctx, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
@@ -37,7 +82,7 @@ static void launch_k(reg_ctx* ctx, void (*kern)(KArgs...), dim3 grid, dim3 block
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = ctx->pdl ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+    launch_cfg<KArgs...>(ctx->build, cfg, kern, static_cast<KArgs>(args)...);
 }
 
 [[maybe_unused]] static int rows_per_cta(const reg_ctx* ctx) {

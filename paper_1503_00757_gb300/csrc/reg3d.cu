@@ -376,7 +376,7 @@ struct reg3_ctx {
     double beta, gamma;
     int kmode;  // 0: K = I (gamma = 0), 1: incompressible (gamma = inf), 2: mass source
     cudaStream_t stream;
-    cudaStream_t cap;  // the stream the launch sequences are captured on (created on first use)
+    GraphBuild* build;  // launches go into this graph (nullptr: onto `stream`)
     void* slab;  // the allocation behind the device buffers
     float *mT, *mR, *v, *vt, *gm, *y, *ys, *lam, *src, *D1, *D2, *bt;
     float2* S;   // six half spectra: 0..2 of b (and the results), 3..5 of v
@@ -404,7 +404,7 @@ void launch3(reg3_ctx* c, void (*kern)(KArgs...), dim3 grid, int block, size_t s
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+    launch_cfg<KArgs...>(c->build, cfg, kern, static_cast<KArgs>(args)...);
 }
 
 // D1 = d_1 (f mul1), D2 = d_2 (f mul2) (no factor where mul is nullptr)
@@ -596,9 +596,8 @@ int r3_err(const char* what) {
     return e == cudaSuccess ? REG_OK : reg_fail(REG_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Run a launch sequence that touches the context's own buffers only: captured once per context
-// into a CUDA graph on a stream of the context's own (the legacy default stream cannot be
-// captured) and replayed on its working stream.  While the caller captures that stream the
+// Run a launch sequence that touches the context's own buffers only: built once per context as a
+// CUDA graph and replayed on its working stream.  While the caller captures that stream the
 // launches go into the caller's graph instead.
 enum { G3_GRADIENT = 0, G3_MATVEC = 1, G3_OBJECTIVE = 2 };
 template <typename F>
@@ -611,21 +610,18 @@ int run3(reg3_ctx* c, int kind, F&& body) {
     }
     if (!c->graphs[kind]) {
         const GraphCalls allow;
-        if (!c->cap && cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess)
-            return r3_err("capture stream");
-        if (cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed) != cudaSuccess) return r3_err("capture");
-        const cudaStream_t s = c->stream;
-        c->stream = c->cap;
+        GraphBuild b;
+        if (cudaGraphCreate(&b.graph, 0) != cudaSuccess) return r3_err("graph");
+        c->build = &b;
         body();
-        c->stream = s;
-        cudaGraph_t graph = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(c->cap, &graph);
-        if (e != cudaSuccess || !graph) return r3_err("capture");
-        const cudaError_t ei = cudaGraphInstantiate(&c->graphs[kind], graph, 0);
-        cudaGraphDestroy(graph);
-        if (ei != cudaSuccess) {
+        c->build = nullptr;
+        cudaError_t e = b.err;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graphs[kind], b.graph, 0);
+        cudaGraphDestroy(b.graph);
+        if (e != cudaSuccess) {
             c->graphs[kind] = nullptr;
-            return r3_err("graph");
+            cudaGetLastError();
+            return reg_fail(REG_ERR_CUDA, std::string("graph: ") + cudaGetErrorString(e));
         }
     }
     cudaGraphLaunch(c->graphs[kind], c->stream);
@@ -645,7 +641,6 @@ extern "C" void reg3_destroy(reg3_ctx* c) {
     if (!c) return;
     for (cudaGraphExec_t g : c->graphs)
         if (g) cudaGraphExecDestroy(g);
-    if (c->cap) cudaStreamDestroy(c->cap);
     cudaFree(c->slab);
     cudaFreeHost(c->h_sum);
     delete c;

@@ -39,6 +39,7 @@
 #include "fft.cuh"
 #include "fft_reg.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -736,15 +737,15 @@ void launch_transport_cluster(reg_ctx* ctx, int mode, const TcArgs& args) {
         if (mode == TC_STATE) {
             tc_prepare<LG, TC_STATE>();
             cudaLaunchConfig_t cfg = tc_config<LG, TC_STATE>(ctx->stream, attr);
-            cudaLaunchKernelEx(&cfg, k_transport_cluster<LG, TC_STATE>, a);
+            launch_cfg<TcArgs>(ctx->build, cfg, k_transport_cluster<LG, TC_STATE>, a);
         } else if (mode == TC_ADJOINT) {
             tc_prepare<LG, TC_ADJOINT>();
             cudaLaunchConfig_t cfg = tc_config<LG, TC_ADJOINT>(ctx->stream, attr);
-            cudaLaunchKernelEx(&cfg, k_transport_cluster<LG, TC_ADJOINT>, a);
+            launch_cfg<TcArgs>(ctx->build, cfg, k_transport_cluster<LG, TC_ADJOINT>, a);
         } else {
             tc_prepare<LG, TC_MATVEC>();
             cudaLaunchConfig_t cfg = tc_config<LG, TC_MATVEC>(ctx->stream, attr);
-            cudaLaunchKernelEx(&cfg, k_transport_cluster<LG, TC_MATVEC>, a);
+            launch_cfg<TcArgs>(ctx->build, cfg, k_transport_cluster<LG, TC_MATVEC>, a);
         }
     });
     ktimer_end(ctx);

@@ -279,13 +279,13 @@ void launch_resident(reg_ctx* ctx, int mode, const RsArgs& a) {
         cudaLaunchAttribute attr[2];
         if (mode == RS_STATE) {
             cudaLaunchConfig_t cfg = rs_config<B1, B2, RS_STATE>(ctx->stream, attr, ctx->pdl);
-            cudaLaunchKernelEx(&cfg, k_resident<B1, B2, RS_STATE>, a, (const float2*)ctx->tw);
+            launch_cfg<RsArgs, const float2*>(ctx->build, cfg, k_resident<B1, B2, RS_STATE>, a, ctx->tw);
         } else if (mode == RS_ADJOINT) {
             cudaLaunchConfig_t cfg = rs_config<B1, B2, RS_ADJOINT>(ctx->stream, attr, ctx->pdl);
-            cudaLaunchKernelEx(&cfg, k_resident<B1, B2, RS_ADJOINT>, a, (const float2*)ctx->tw);
+            launch_cfg<RsArgs, const float2*>(ctx->build, cfg, k_resident<B1, B2, RS_ADJOINT>, a, ctx->tw);
         } else {
             cudaLaunchConfig_t cfg = rs_config<B1, B2, RS_MATVEC>(ctx->stream, attr, ctx->pdl);
-            cudaLaunchKernelEx(&cfg, k_resident<B1, B2, RS_MATVEC>, a, (const float2*)ctx->tw);
+            launch_cfg<RsArgs, const float2*>(ctx->build, cfg, k_resident<B1, B2, RS_MATVEC>, a, ctx->tw);
         }
     });
     ktimer_end(ctx);

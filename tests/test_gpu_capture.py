@@ -144,3 +144,60 @@ def test_refused_calls_leave_the_context_and_the_capture_as_they_were(called_bef
     torch.cuda.synchronize()
     ctx.close()
     assert torch.equal(H, H2)
+
+
+@pytest.mark.parametrize("working_stream", [False, True])
+def test_first_calls_while_another_thread_synchronizes_the_device(working_stream):
+    """While a stream is being captured no thread may synchronize the device: a context's first calls
+    capture nothing, so neither side of this fails, and the results are the usual ones."""
+    import threading
+    import torch
+    from paper_1503_00757_gb300.binding import Context, Context3D
+    mT, mR, v, vt = _inputs()
+    rng = np.random.default_rng(6)
+    m3 = [to_gpu(rng.random((16, 16, 16))) for _ in range(2)]
+    v3, t3 = (to_gpu(0.1 * rng.standard_normal((3, 16, 16, 16))) for _ in range(2))
+    s = torch.cuda.Stream() if working_stream else None
+    torch.cuda.synchronize()
+
+    def once():
+        E = lambda k: torch.zeros(k, N, N, device="cuda")
+        out = g, H, u, det, v1, H3 = E(2), E(2), E(2), E(1), E(2), torch.zeros_like(v3)
+        ctx, c3 = Context(N, N, NT, regnorm=2, beta=1e-2, stream=s), Context3D(16, 16, 16, 2, stream=s)
+        ctx.set_images(mT, mR)
+        c3.set_images(*m3)
+        for _ in range(12):
+            ctx.displacement(v, u)
+            ctx.gradient(v, g)
+            ctx.hessian_matvec(vt, H)
+        ctx.detgrad(v, det)
+        c3.gradient(v3, H3)
+        c3.hessian_matvec(t3, H3)
+        from paper_1503_00757_gb300.binding import default_opts
+        ctx.solve(v1, default_opts(maxit_newton=1, maxit_pcg=3), check=False)
+        torch.cuda.synchronize()
+        ctx.close()
+        c3.close()
+        return out
+
+    ref = once()
+    stop, failed, count = threading.Event(), [], [0]
+
+    def other():
+        while not stop.is_set():
+            try:
+                torch.cuda.synchronize()
+                count[0] += 1
+            except Exception as e:  # noqa: BLE001
+                failed.append(str(e))
+
+    t = threading.Thread(target=other)
+    t.start()
+    try:
+        outs = [once() for _ in range(12)]
+    finally:
+        stop.set()
+        t.join()
+    assert not failed and count[0] > 0
+    for o in outs:
+        assert all(torch.equal(a, b) for a, b in zip(o, ref))
