@@ -243,7 +243,7 @@ typedef struct {
 int reg_solve_batch(reg_batch_item* items, int count, const reg_solve_opts* opts, int nworkers);
 
 /* A persistent batch executor: the same scheduling as reg_solve_batch, but
- * its worker streams, per-grid-size contexts and their captured launch
+ * its worker streams, per-grid-size contexts and their graphs of launch
  * sequences stay alive across calls (reg_solve_batch builds and frees one per
  * call).  Create on the device that will run the pairs (nworkers <= 0: 8). */
 typedef struct reg_executor reg_executor;

@@ -196,7 +196,7 @@ void launch_r2c_two(reg_ctx* ctx, const float* u, const float* b, float2* const*
 void launch_c2r_scalar(reg_ctx* ctx, const float2* S, float* f);
 void launch_c2r_vec(reg_ctx* ctx, const float2* S1, const float2* S2, float* u1, float* u2, int nb = 1,
                     float scale = 1.f, long long ss = 0);  // ss: entries from field to field (0: N)
-// points a captured launch_c2r_vec of one field at other outputs
+// points the graph node of a launch_c2r_vec of one field at other outputs
 cudaError_t rebind_c2r_vec(cudaGraphExec_t exec, cudaGraphNode_t node, float* u1, float* u2);
 // nb > 1 (OP_GRAD and OP_SMOOTH_PROJ only): independent fields, bs spectrum entries apart
 void launch_col(reg_ctx* ctx, int op, const float2* const* in, float2* const* out, const SpecParams& P,
