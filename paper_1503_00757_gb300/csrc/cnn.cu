@@ -1162,8 +1162,7 @@ struct reg_net {
     bool record;               // keep every layer's output gradient (reg_net_layer_tensor)
     bf16* dz_rec[NLAYER];
     reg_ctx* proj_fine;        // output map on the (2H, 2W) grid of reg_net_forward_fine (created on first use)
-    // restricted images (maxB x 2 x H x W), prolonged prediction and its spectra (maxB x 2 x 2H x 2W each)
-    float *coarse_img, *fine_v, *fine_spec;
+    float *coarse_img, *fine_v;  // restricted images (maxB x 2 x H x W), prolonged prediction (maxB x 2 x 2H x 2W)
 };
 
 static size_t conv_smem(int cin, int cout) {
@@ -1288,7 +1287,6 @@ extern "C" void reg_net_destroy(reg_net* n) {
     if (n->proj_fine) reg_destroy(n->proj_fine);
     cudaFree(n->coarse_img);
     cudaFree(n->fine_v);
-    cudaFree(n->fine_spec);
     void* ptrs[] = {n->d_layers, n->params, n->m1, n->m2, n->gW, n->gb, n->d_gwoff, n->d_gboff, n->d_wfoff,
                     n->wf, n->wt, n->bpad, n->dzA, n->dzB, n->out, n->pred, n->res, n->dout, n->partial,
                     n->bpartial, n->d_part, n->d_err};
@@ -1695,8 +1693,7 @@ extern "C" int reg_net_forward_fine(reg_net* n, const float* images, int B, floa
         }
         const size_t pix = (size_t)n->maxB * H * W;
         if (cudaMalloc((void**)&n->coarse_img, sizeof(float) * 2 * pix) != cudaSuccess ||
-            cudaMalloc((void**)&n->fine_v, sizeof(float) * 8 * pix) != cudaSuccess ||
-            cudaMalloc((void**)&n->fine_spec, sizeof(float) * 8 * pix) != cudaSuccess) {
+            cudaMalloc((void**)&n->fine_v, sizeof(float) * 8 * pix) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(n->coarse_img);
             cudaFree(n->fine_v);
@@ -1712,10 +1709,11 @@ extern "C" int reg_net_forward_fine(reg_net* n, const float* images, int B, floa
     k_prolong2<<<304, 256, 0, n->stream>>>(n->pred, n->fine_v, 2 * B, H, W);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));
-    // the fine grid's own output map P G (sigma = 2 h of that grid), then the output scale
+    // the fine grid's own output map P G (sigma = 2 h of that grid), then the output scale; its spectra
+    // (8 floats a pixel of the H x W grid) take the backward pass's dzA (16)
     const double sigma = 2.0 * (2.0 * M_PI / (double)(Hf > Wf ? Hf : Wf));
     st = apply_smooth_proj(n->proj_fine, (float)(0.5 * sigma * sigma), n->fine_v, v_out, B,
-                           reinterpret_cast<float2*>(n->fine_spec), n->out_scale);
+                           reinterpret_cast<float2*>(n->dzA), n->out_scale);
     if (st != REG_OK) return st;
     e = cudaGetLastError();
     return e == cudaSuccess ? REG_OK : reg_fail(REG_ERR_CUDA, cudaGetErrorString(e));

@@ -418,7 +418,10 @@ void d12(reg3_ctx* c, const float* f, const float* mul1, const float* mul2) {
     a.m2 = ColMap{D.l3 - 1, D.n2 * D.n3 / 2, D.n3 / 2, nc2};
     a.log1 = D.l1;
     a.log2 = D.l2;
-    // 16 entries a thread on axes of 128 and 256 points where that leaves several blocks per SM
+    // 16 entries a thread on axes of 128 and 256 points where that leaves several blocks per SM.  Matvec,
+    // nt = 4, us with 16 / with 8: 256 x 128 x 128 1061 / 1139, 128^3 488 / 524, 256 x 128 x 32 381 / 396,
+    // 64 x 128 x 128 263 / 265; below 2^20 points it depends on the box: 128 x 64 x 64 203 / 203,
+    // 128 x 128 x 16 192 / 229, 16 x 128 x 256 180 / 178, 128 x 16 x 16 120 / 117
     const bool wide = D.N >= (1 << 20);
     auto cols = [&](int n) { return (wide && n >= 128 ? 2048 : 1024) / n; };  // columns of a block
     auto smem = [&](int n) {
@@ -431,7 +434,9 @@ void d12(reg3_ctx* c, const float* f, const float* mul1, const float* mul2) {
     launch3(c, wide ? k3_d12<true> : k3_d12<false>, a.tiles1 + tiles2, 128, sh, a, c->tw);
 }
 
-// row kernels: 128 threads a block (64 for small boxes), at most the box's pairs of rows
+// row kernels: 128 threads a block (64 for small boxes), at most the box's pairs of rows.  Matvec,
+// nt = 4, us with 128 / with 64 threads: 32^3 111 / 100, 128 x 32 x 32 140 / 133, 64 x 64 x 32 139 / 128;
+// from 2^18 points on the same but for 64^3 149 / 142 and, the reason for the line, 128 x 128 x 16 229 / 291
 struct Row3 { int lines, threads, grid; size_t smem; };
 Row3 row3(const Dims3& D) {
     Row3 r;
